@@ -233,9 +233,10 @@ fwi_status fwi_choose_ckpt(fwi_ctx *ctx, const fwi_model *model, const fwi_sourc
                            int32_t *ckpt_every);
 
 /* Tile shape of the acoustic forward steps of ctx's calls (forward sweep and
- * segment recompute): tiles of 64 columns x forward_tile_rows rows, 32 (256
- * threads per CTA) or 64 (512 threads; half the z-halo flux recompute per cell,
- * fewer and larger CTAs). 0 keeps the library's default (32). Results do not
+ * segment recompute): tiles of 64 columns x forward_tile_rows rows, 32 or 64 (256
+ * threads per CTA; 64 halves the z-halo flux recompute per cell in fewer and
+ * larger CTAs). 0 keeps the library's default (32, or 8 while the shots' 32-row
+ * tiles are too few to fill the GPU). Results do not
  * depend on it (each cell's arithmetic is the same). Takes effect for later
  * calls and recordings; FWI_EINVAL for other values. The batched autotuner
  * picks it per workload. */
@@ -245,7 +246,7 @@ fwi_status fwi_set_tile_shape(fwi_ctx *ctx, int32_t forward_tile_rows);
  * into forward_groups (forward and recompute steps) and adjoint_groups
  * (adjoint steps) contiguous groups, each step launched once per group on its
  * own stream, so that the groups' launches fill each other's idle SMs. 0 keeps
- * the library's default (4 and 2); at most 4; never more groups than shots.
+ * the library's default (2 for the forward sweep, 4 for recomputed steps, 2 for the adjoint); at most 4; never more groups than shots.
  * Results do not depend on it (the per-shot arithmetic and the fixed-order
  * cross-shot sums are the same). Takes effect for later calls and recordings;
  * FWI_EINVAL outside [0, 4]. */

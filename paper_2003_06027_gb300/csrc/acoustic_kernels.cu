@@ -6,9 +6,10 @@
 // lambda_k = A^T lambda_{k+1} + residual (Eq. adjoint-backward) fused with the
 // gradient correlation lambda^T (dA/dm) U (Eq. adjoint-gradient).
 //
-// Design (memory bound, no dense contraction, so no tensor cores):
+// Design (no dense contraction, so no tensor cores; bound by instruction issue and
+// load latency while a step's fields stay in L2, by memory beyond that):
 //   * persistent CTAs (grid = resident CTAs of the GPU) walk the tiles of all
-//     shots; a tile is 64 x 32 cells of one shot;
+//     shots; a tile is 64 columns x 32 rows (forward: 8, 32 or 64) of one shot;
 //   * the stencil operand tiles with their 8-cell halo and the coefficient tile are
 //     fetched by TMA (cp.async.bulk.tensor) into the CTA's one operand buffer
 //     as soon as stage 1 (their last reader) has passed its barrier, so the
@@ -16,13 +17,20 @@
 //     resident CTAs cover the rest; the completion wait on the mbarrier is
 //     bounded and reports a timeout;
 //   * stage 1 evaluates each half-point flux once (x: q at the half columns
-//     of the tile and its halo; z: a register window over two rows per thread),
+//     of the tile and its halo; z: a register window over a thread's rows),
 //     stage 2 the divergence, update, sources and receivers;
 //   * per-cell operands that do not need a halo: u^{n-1} is copied into shared
 //     memory by cp.async issued before the wait (its latency overlaps the tile
 //     fetch and stage 1 without holding registers); the adjoint's stored fluxes
 //     are float4 loads issued there too, its lambda_{n+2} and gradient partial
-//     are loaded at the start of stage 2.
+//     are loaded before the stage barrier; CPML memory variables are on their way
+//     (registers or L1) before the wait;
+//   * each launch may start while the step before it drains (programmatic
+//     dependent launch).
+// Forward step against the one-row-pair-at-a-time scalar body it replaces, per
+// step: one shot of 100 x 100 8.2 -> 4.6 us, 16 shots of 128 x 256 10.3 -> 6.8 us,
+// 16 shots of 201 x 601 15.5 -> 14.8 us, 128 shots 125 -> 112 us (2.9 -> 3.2 TB/s
+// of its 16 B per cell); 141 -> 121 thread instructions per cell.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -36,6 +44,8 @@
 
 namespace fwi {
 
+void acu_coef_pairs(AcuCoef& c);
+
 namespace {
 
 constexpr int H = 8;                     // wavefield halo (>= 2N-1)
@@ -47,16 +57,19 @@ constexpr int QXW = TILE_X + 8;          // 72: half cols [x0-4, x0+TX+4)
 constexpr int QZH = TILE_Z + 8;          // 40: half rows [z0-4, z0+TZ+4)
 constexpr int M_BYTES = MW * MH * 4;     // 12464
 constexpr int M_SLOT = (M_BYTES + 127) / 128 * 128;
-#ifndef FWI_FWD_CTAS
-#define FWI_FWD_CTAS 4
-#endif
-constexpr int FWD_CTAS = FWI_FWD_CTAS;     // resident forward CTAs per SM the registers are sized for
 constexpr int XS_BYTES = TILE_Z * UW * 4;  // 10240: adjoint x operand tile
-// Geometry of a forward tile of TZ rows (TZ = 32 or 64) and TILE_X columns: 16
-// columns of threads, each thread owning 2 rows x 4 columns (so 8 * TZ threads).
-template <int TZ>
+// Geometry of a forward tile: 16 threads across, TY down, each owning R rows x 4
+// columns, so a tile of TY R rows and TILE_X columns.
+// The 32-row tile runs 3 CTAs per SM with the CPML operands held in registers, or
+// 4 without (PRE): the recording step measured 15.1 against 16.2 us, the storing
+// one, which has the flux stores to cover, 16.1 against 14.8 us (16 shots of 201 x
+// 601). The 8-row tile (8 CTAs) and the 64-row one (2) hold them.
+__host__ __device__ constexpr bool fwd_pre(int R, bool store) { return R != 2 || !store; }
+__host__ __device__ constexpr int fwd_ctas(int R, bool store) { return R == 1 ? 8 : R == 4 ? 2 : fwd_pre(R, store) ? 3 : 4; }
+template <int R, int TY>
 struct FwdGeo {
-  static constexpr int NT = 8 * TZ;           // threads per CTA
+  static constexpr int NT = 16 * TY;          // threads
+  static constexpr int TZ = TY * R;           // tile height
   static constexpr int UHT = TZ + 2 * H;      // wavefield tile height
   static constexpr int MHT = TZ + 9;          // m tile rows [z0-4, z0+TZ+5)
   static constexpr int QZHT = TZ + 8;         // half rows [z0-4, z0+TZ+4)
@@ -65,6 +78,111 @@ struct FwdGeo {
   static constexpr int MSLOT = (MB + 127) / 128 * 128;
 };
 constexpr int ZS_BYTES = UH * TILE_X * 4;  // 12288: adjoint z operand tile
+
+// Four FP32 values as two packed pairs: the packed instructions (add, sub, mul,
+// fma.f32x2) round each half as the scalar instruction does and take one issue
+// slot for two cells.
+typedef unsigned long long u64;
+struct Q4 {
+  u64 a, b;
+};
+__device__ __forceinline__ u64 add2(u64 x, u64 y) {
+  u64 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));
+  return d;
+}
+__device__ __forceinline__ u64 sub2(u64 x, u64 y) {
+  u64 d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));
+  return d;
+}
+__device__ __forceinline__ u64 mul2(u64 x, u64 y) {
+  u64 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(x), "l"(y));
+  return d;
+}
+__device__ __forceinline__ u64 fma2(u64 x, u64 y, u64 z) {
+  u64 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(x), "l"(y), "l"(z));
+  return d;
+}
+__device__ __forceinline__ u64 pk(float x, float y) {
+  u64 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+  return d;
+}
+__device__ __forceinline__ void upk(u64 v, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
+__device__ __forceinline__ Q4 add4(Q4 x, Q4 y) { return {add2(x.a, y.a), add2(x.b, y.b)}; }
+__device__ __forceinline__ Q4 sub4(Q4 x, Q4 y) { return {sub2(x.a, y.a), sub2(x.b, y.b)}; }
+__device__ __forceinline__ Q4 mul4(Q4 x, Q4 y) { return {mul2(x.a, y.a), mul2(x.b, y.b)}; }
+__device__ __forceinline__ Q4 fma4(u64 c, Q4 x, Q4 y) { return {fma2(c, x.a, y.a), fma2(c, x.b, y.b)}; }
+__device__ __forceinline__ Q4 scale4(u64 c, Q4 x) { return {mul2(c, x.a), mul2(c, x.b)}; }
+__device__ __forceinline__ void get4(Q4 q, float v[4]) {
+  upk(q.a, v[0], v[1]);
+  upk(q.b, v[2], v[3]);
+}
+__device__ __forceinline__ Q4 put4(const float v[4]) { return {pk(v[0], v[1]), pk(v[2], v[3])}; }
+__device__ __forceinline__ Q4 zero4() { return {0ull, 0ull}; }
+__device__ __forceinline__ Q4 ldq(const float* p) {
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
+  return {v.x, v.y};
+}
+__device__ __forceinline__ void stq(float* p, Q4 q) { *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(q.a, q.b); }
+__device__ __forceinline__ void stq_stream(float* p, Q4 q, u64 pol) {
+  asm volatile("st.global.L1::no_allocate.L2::cache_hint.v2.u64 [%0], {%1, %2}, %3;" ::"l"(p), "l"(q.a), "l"(q.b), "l"(pol));
+}
+// The values of columns xb .. xb+3 below `end`, zero from there on.
+__device__ __forceinline__ Q4 mask_cols(Q4 q, int xb, int end) {
+  float v[4];
+  get4(q, v);
+#pragma unroll
+  for (int e = 0; e < 4; e++)
+    if (xb + e >= end) v[e] = 0.f;
+  return put4(v);
+}
+// z stencils of R consecutive rows from a window of R + 2N - 1 rows:
+// o[r] = sum_k c_k (w[N - 1 + r + k] - w[N + r - k])
+template <int N, int R>
+__device__ __forceinline__ void dz(const u64* c, const Q4* w, Q4* o) {
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    Q4 a = scale4(c[0], sub4(w[N + r], w[N - 1 + r]));
+#pragma unroll
+    for (int k = 2; k <= N; k++) a = fma4(c[k - 1], sub4(w[N - 1 + r + k], w[N + r - k]), a);
+    o[r] = a;
+  }
+}
+// x stencils of one row; v holds columns xb-4 .. xb+7.
+// D+ at the half points xb+e+1/2: sum_k c_k (v[e+4+k] - v[e+5-k])
+template <int N>
+__device__ __forceinline__ void dplus_x(const float* c, const float v[12], float o[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; e++) {
+    float a = c[0] * (v[e + 5] - v[e + 4]);
+#pragma unroll
+    for (int k = 2; k <= N; k++) a = fmaf(c[k - 1], v[e + 4 + k] - v[e + 5 - k], a);
+    o[e] = a;
+  }
+}
+// D- at the columns xb+e from the half points: sum_k c_k (v[e+k+3] - v[e-k+4])
+template <int N>
+__device__ __forceinline__ void dminus_x(const float* c, const float v[12], float o[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; e++) {
+    float a = c[0] * (v[e + 4] - v[e + 3]);
+#pragma unroll
+    for (int k = 2; k <= N; k++) a = fmaf(c[k - 1], v[e + k + 3] - v[e - k + 4], a);
+    o[e] = a;
+  }
+}
+
+// Programmatic dependent launch: a step's CTAs may be scheduled while the
+// previous step drains; they wait for its end before they touch memory, and only
+// then let the next step's CTAs in (so at most two steps are resident, and no
+// line that a step could have cached is older than the step before it). Both
+// are no-ops in a launch without the attribute.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
@@ -88,6 +206,7 @@ __device__ __forceinline__ void acc4(float4& acc, float c, const float4 p, const
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
+__device__ __forceinline__ void prefetch_l1(const float* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
@@ -159,31 +278,30 @@ __device__ __forceinline__ void cta_sum3(float v[3], float* red) {
   __syncthreads();
 }
 
-// Issue the TMA fetches of tile t (TZ rows) into one buffer (one elected thread).
+// Issue the TMA fetches of tile t (8 R rows) into one buffer (one elected thread).
 // plane0: the pair plane of this launch's first shot.
-template <int TZ = TILE_Z>
+template <int R, int TY>
 __device__ __forceinline__ void fetch_tile(const CUtensorMap* fmap, const CUtensorMap* mmap, const Grid& g, int plane0,
                                            int t, float* dst_u, float* dst_m, uint64_t* bar) {
-  const TileId id = tile_decode_t<TZ>(g, t);
+  const TileId id = tile_decode_t<FwdGeo<R, TY>::TZ>(g, t);
   fence_proxy_async();
-  mbar_expect_tx(bar, FwdGeo<TZ>::UB + FwdGeo<TZ>::MB);
+  mbar_expect_tx(bar, FwdGeo<R, TY>::UB + FwdGeo<R, TY>::MB);
   // allocation coordinates: padded (i, j) -> (i + APRON, j + APRON)
   tma_3d(dst_u, fmap, id.x0 - H + APRON, id.z0 - H + APRON, plane0 + id.s, bar);
   tma_2d(dst_m, mmap, id.x0 - 4 + APRON, id.z0 - 4 + APRON, bar);
 }
 
 // Shared memory of the step kernels (every array a multiple of 128 bytes).
-template <int TZ>
+template <int R, int TY>
 struct FwdSmemT {
-  float u[FwdGeo<TZ>::UHT * UW];
-  float m[FwdGeo<TZ>::MSLOT / 4];
-  float qx[TZ * QXW];
-  float qz[FwdGeo<TZ>::QZHT * TILE_X];
-  float4 up4[2 * FwdGeo<TZ>::NT];  // u^{n-1} of the own cells, [row][thread] (cp.async)
+  float u[FwdGeo<R, TY>::UHT * UW];
+  float m[FwdGeo<R, TY>::MSLOT / 4];
+  float qx[FwdGeo<R, TY>::TZ * QXW];
+  float qz[FwdGeo<R, TY>::QZHT * TILE_X];
+  float4 up4[R * FwdGeo<R, TY>::NT];  // u^{n-1} of the own cells, [row][thread] (cp.async)
   float red[32];
   uint64_t bar;
 };
-using FwdSmem = FwdSmemT<TILE_Z>;
 struct AdjSmem {
   float xs[TILE_Z * UW];     // x stencil operand (lambda or Hx): own rows, cols [x0-H, x0+TX+H)
   float zs[UH * TILE_X];     // z stencil operand (lambda or Hz): rows [z0-H, z0+TZ+H), own cols
@@ -197,7 +315,8 @@ struct AdjSmem {
 };
 // Multi-instance launches keep the current tile's step parameters after the
 // kernel's own shared memory.
-constexpr size_t FWD_SMEM_MAIN = (sizeof(FwdSmem) + 15) / 16 * 16;
+template <int R, int TY>
+constexpr size_t FWD_SMEM_MAIN = (sizeof(FwdSmemT<R, TY>) + 15) / 16 * 16;
 constexpr size_t ADJ_SMEM_MAIN = (sizeof(AdjSmem) + 15) / 16 * 16;
 
 // Multi-instance launches: the instance of tile t (the last i with tile_start[i] <= t).
@@ -274,24 +393,23 @@ __device__ __forceinline__ void batch_load_step(const BatchArgs& b, int i, AcuSt
 // forward-sweep launch (RECORD and STORE) stores the fluxes only for the
 // instances in their last segment (a null slot otherwise).
 //
-// TZ: the tile height, 32 (256 threads) or 64 (512 threads, a compile-time
-// variant for the autotuner: half the z-halo recompute per cell, the same
-// per-thread work); multi-instance launches use 32.
+// R rows per thread, TY rows of threads: a tile has R TY rows (8, 32 or 64; see
+// acu_fwd_rows). The z arithmetic, the updates and the CPML rows use packed pairs.
 // LAP: the c^2 Laplacian operator instead of the divergence form: the fluxes
 // carry no coefficient (q = D+u + psi), the update is
 // u^{n+1} = 2u^n - u^{n-1} + m dt^2 (D-q + zeta) + dt^2 w g(t_n) with m = c^2 at
 // the cell, and STORE keeps r = dt^2 (D-q + zeta) at the cells (the operand of
 // its gradient correlation dJ/dm = sum_n lambda_{n+1} r^n) instead of the fluxes.
-template <int N, bool RECORD, bool STORE, bool MULTI, int TZ, bool LAP = false>
-__global__ void __launch_bounds__(FwdGeo<TZ>::NT, TZ == TILE_Z ? FWD_CTAS : 2)
+template <int N, bool RECORD, bool STORE, bool MULTI, int R, int TY, bool LAP = false>
+__global__ void __launch_bounds__(16 * TY, fwd_ctas(R, STORE))
     acu_fwd_step(const __grid_constant__ CUtensorMap tmap_u, const __grid_constant__ CUtensorMap tmap_m,
-                 const __grid_constant__ AcuStep p0, const AcuCoef cf, const BatchArgs b) {
-  static_assert(TZ == TILE_Z || (TZ == 2 * TILE_Z && !MULTI), "tile heights: 32, or 64 for single-instance launches");
-  static_assert(!LAP || (TZ == TILE_Z && !MULTI), "the Laplacian operator runs on 32-row single-instance launches");
-  constexpr int NT = FwdGeo<TZ>::NT;
+                 const __grid_constant__ AcuStep p0, const __grid_constant__ AcuCoef cf, const BatchArgs b) {
+  static_assert(!LAP || !MULTI, "the Laplacian operator runs on single-instance launches");
+  constexpr bool PRE = fwd_pre(R, STORE);
+  constexpr int NT = 16 * TY, TZ = FwdGeo<R, TY>::TZ, WR = R + 2 * N - 1;  // rows of a z stencil window
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  FwdSmemT<TZ>& sh = *reinterpret_cast<FwdSmemT<TZ>*>(smem_raw);
-  AcuStep& shp = *reinterpret_cast<AcuStep*>(smem_raw + FWD_SMEM_MAIN);  // MULTI only
+  FwdSmemT<R, TY>& sh = *reinterpret_cast<FwdSmemT<R, TY>*>(smem_raw);
+  AcuStep& shp = *reinterpret_cast<AcuStep*>(smem_raw + FWD_SMEM_MAIN<R, TY>);  // MULTI only
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const uint64_t pol = STORE ? l2_evict_first() : 0ull;  // segment slots stream through L2
   const int ntiles = MULTI ? b.ntiles : p0.ntiles;
@@ -303,9 +421,9 @@ __global__ void __launch_bounds__(FwdGeo<TZ>::NT, TZ == TILE_Z ? FWD_CTAS : 2)
       const Grid gi = in->p.g;
       tensormap_acquire(&in->mu);
       tensormap_acquire(&in->mm);
-      fetch_tile(&in->mu, &in->mm, gi, (b.n & 1) * in->p.S, tt - __ldg(b.tile_start + i), sh.u, sh.m, &sh.bar);
+      fetch_tile<R, TY>(&in->mu, &in->mm, gi, (b.n & 1) * in->p.S, tt - __ldg(b.tile_start + i), sh.u, sh.m, &sh.bar);
     } else {
-      fetch_tile<TZ>(&tmap_u, &tmap_m, p0.g, p0.cur * p0.S_pair + p0.s0, tt, sh.u, sh.m, &sh.bar);
+      fetch_tile<R, TY>(&tmap_u, &tmap_m, p0.g, p0.cur * p0.S_pair + p0.s0, tt, sh.u, sh.m, &sh.bar);
     }
   };
 
@@ -316,6 +434,8 @@ __global__ void __launch_bounds__(FwdGeo<TZ>::NT, TZ == TILE_Z ? FWD_CTAS : 2)
     fence_mbar_init();
   }
   __syncthreads();
+  pdl_wait();
+  pdl_next();
   if (tid == 0 && (int)blockIdx.x < ntiles) fetch_next(blockIdx.x);
 
   int it = 0, inst_loaded = -1;
@@ -336,25 +456,76 @@ __global__ void __launch_bounds__(FwdGeo<TZ>::NT, TZ == TILE_Z ? FWD_CTAS : 2)
     const TileId id = tile_decode_t<TZ>(g, tl);
     const int x0 = id.x0, z0 = id.z0, s = id.s;
     const long long base = (long long)s * g.slice + g.off0;
+    // this thread's cells: rows zr0 .. zr0+R-1, columns xb .. xb+3
+    const int xb = x0 + 4 * tx, zr0 = z0 + R * ty;
+    const long long own = (long long)zr0 * pitch + xb;  // of the shot's field
     float* __restrict__ uprev = p.u + (long long)((p.cur ^ 1) * p.S_pair + p.s0) * g.slice + base;
-    // u^{n-1} of this thread's 2 x 4 cells: copied into shared memory while the
-    // tile is fetched and stage 1 runs
-    const int xb = x0 + 4 * tx, zr0 = z0 + 2 * ty;
+    // u^{n-1} of the own cells: copied into shared memory while the tile is
+    // fetched and stage 1 runs
 #pragma unroll
-    for (int rr = 0; rr < 2; rr++) cp_async16(&sh.up4[rr * NT + tid], uprev + (long long)(zr0 + rr) * pitch + xb);
+    for (int rr = 0; rr < R; rr++) cp_async16(&sh.up4[rr * NT + tid], uprev + own + rr * pitch);
     cp_async_commit();
-    // small per-tile operands, fetched before the wait as well
     const int2 box = __ldg(reinterpret_cast<const int2*>(p.src_box) + s);
-    const float stf_n = __ldg(p.stf + (long long)s * p.nt + p.n);
-    // receivers: the lists are kept per thread of a 32-row tile; a thread of a
-    // 64-row tile owns the same 2 x 4 cells as thread (ty % 16, tx) of 32-row
-    // tile 2 tz + ty / 16 (beyond the grid's last 32-row tile: no receivers)
-    const int tz32 = id.tz * (TZ / TILE_Z) + ty / 16;
-    int rb = 0, re = 0;
-    if (RECORD && tz32 < g.ntz) {
-      const int key = (tz32 * g.ntx + id.tx) * NTHREADS + (ty % 16) * 16 + tx;
-      rb = __ldg(p.thr_rec_start + key);
-      re = __ldg(p.thr_rec_start + key + 1);
+    const int i0 = box.x, j0 = box.y, nb = p.src_n;
+    const bool src_t = i0 >= 0 && i0 < z0 + TZ && i0 + nb > z0 && j0 < x0 + TILE_X && j0 + nb > x0;
+    // receivers in this tile's 32-row list tile (the lists are kept per thread of
+    // a 32-row walk, two rows and four columns each)
+    bool has_rec = false;
+    if (RECORD && p.nrec > 0)
+      for (int k = z0 / TILE_Z; k < g.ntz && k * TILE_Z < z0 + TZ; k++) {
+        const int key0 = (k * g.ntx + id.tx) * NTHREADS;
+        has_rec |= __ldg(p.thr_rec_start + key0) != __ldg(p.thr_rec_start + key0 + NTHREADS);
+      }
+    // z: half rows or cells of the tile in a CPML layer or beyond the grid's top or bottom
+    const bool pmlz = tile_pml_z<TZ>(g, z0);
+    const bool gz_t = pmlz || z0 < 4 || z0 + TZ + 5 > g.Nz;
+    const bool pmlx = tile_pml_x(g, x0);
+    const bool gx = pmlx || x0 < 4 || x0 + TILE_X + 5 > g.Nx;
+
+    // CPML memory variables of the own cells and of this thread's halo items: on
+    // their way before the wait, all at once, so that their latency overlaps the
+    // tile fetch (read row by row where they are used, a CPML tile waits for each
+    // row in turn): psi into registers, or with the zetas into L1 where the
+    // registers buy a fourth resident CTA instead (PRE). The 8 halo half rows are
+    // 128 items; the two halo column groups of every row go to the threads from XH0 on.
+    constexpr int XH0 = NT > 128 ? 128 : 0;
+    const int hrh = ty < 4 ? ty : ty + TZ;
+    const int rxh = (tid - XH0) >> 1, gxh = (tid & 1) ? QXW / 4 - 1 : 0;
+    const bool xhalo = tid >= XH0 && tid < XH0 + 2 * TZ;
+    Q4 psz[R], psx[R], pszh = zero4(), psxh = zero4();
+#pragma unroll
+    for (int rr = 0; rr < R; rr++) psz[rr] = psx[rr] = zero4();
+    if (pmlz) {
+      const float* q = p.psiz_in + base;
+#pragma unroll
+      for (int rr = 0; rr < R; rr++) {
+        if (layer_h(zr0 + rr, zr0 + rr, g.npml, g.nz)) {
+          if (PRE) psz[rr] = ldq(q + own + rr * pitch);
+          else prefetch_l1(q + own + rr * pitch);
+        }
+        if (!PRE && layer_c(zr0 + rr, zr0 + rr, g.npml, g.nz)) prefetch_l1(p.zetz + base + own + rr * pitch);
+      }
+      const int hz = z0 - 4 + hrh;
+      if ((NT == 128 || tid < 128) && layer_h(hz, hz, g.npml, g.nz)) {
+        if (PRE) pszh = ldq(q + (long long)hz * pitch + xb);
+        else prefetch_l1(q + (long long)hz * pitch + xb);
+      }
+    }
+    if (pmlx) {
+      const float* q = p.psix_in + base;
+#pragma unroll
+      for (int rr = 0; rr < R; rr++) {
+        if (layer_h(xb, xb + 3, g.npml, g.nx)) {
+          if (PRE) psx[rr] = ldq(q + own + rr * pitch);
+          else prefetch_l1(q + own + rr * pitch);
+        }
+        if (!PRE && layer_c(xb, xb + 3, g.npml, g.nx)) prefetch_l1(p.zetx + base + own + rr * pitch);
+      }
+      const int hb = x0 - 4 + 4 * gxh;
+      if (xhalo && layer_h(hb, hb + 3, g.npml, g.nx)) {
+        if (PRE) psxh = ldq(q + (long long)(z0 + rxh) * pitch + hb);
+        else prefetch_l1(q + (long long)(z0 + rxh) * pitch + hb);
+      }
     }
 
     const bool ok = mbar_wait(&sh.bar, it & 1);
@@ -366,252 +537,229 @@ __global__ void __launch_bounds__(FwdGeo<TZ>::NT, TZ == TILE_Z ? FWD_CTAS : 2)
       }
       return;
     }
-    const float* su = sh.u;
-    const float* sm = sh.m;
-    const bool pmlx = tile_pml_x(g, x0), pmlz = tile_pml_z<TZ>(g, z0);
-
-    // ---- stage 1a: x fluxes q = m_half (D+u + psi) at 4 half columns of row r
-    auto qx_item = [&](int r, int gq, bool own) {
-      const int z = z0 + r, hb = x0 - 4 + 4 * gq;
-      float v[12];
-      unpack12(su + (r + H) * UW + 4 * gq, v);
-      const float4 m4 = ld4(sm + (r + 4) * MW + 4 * gq);
-      const float mv[5] = {m4.x, m4.y, m4.z, m4.w, sm[(r + 4) * MW + 4 * gq + 4]};
-      float q[4], pp[4];
-#pragma unroll
-      for (int e = 0; e < 4; e++) {
-        float gx = 0.f;
-#pragma unroll
-        for (int k = 1; k <= N; k++) gx += cf.c1x[k - 1] * (v[e + 4 + k] - v[e + 5 - k]);
-        pp[e] = gx;
-      }
-      const long long id0 = base + (long long)z * pitch + hb;
-      if (pmlx && layer_h(hb, hb + 3, g.npml, g.nx)) {
-        const float4 a4 = ldg4(p.axh + hb + TAB_OFF);
-        if (a4.x != 0.f || a4.y != 0.f || a4.z != 0.f || a4.w != 0.f) {
-          // psi <- b psi + a g; zero where a = 0 (psi stays zero outside the layer)
-          const float4 b4 = ldg4(p.bxh + hb + TAB_OFF);
-          const float4 po = ld4(p.psix_in + id0);
-          float4 pn;
-          pn.x = b4.x * po.x + a4.x * pp[0]; pn.y = b4.y * po.y + a4.y * pp[1];
-          pn.z = b4.z * po.z + a4.z * pp[2]; pn.w = b4.w * po.w + a4.w * pp[3];
-          if (own && z < g.Nz) st4(p.psix_out + id0, pn);
-          pp[0] += pn.x; pp[1] += pn.y; pp[2] += pn.z; pp[3] += pn.w;
-        }
-      }
-      const bool rowok = z < g.Nz;
-#pragma unroll
-      for (int e = 0; e < 4; e++)
-        q[e] = (rowok && hb + e >= 0 && hb + e < g.Nx - 1) ? (LAP ? pp[e] : (mv[e] + mv[e + 1]) * pp[e]) : 0.f;
-      st4(sh.qx + r * QXW + 4 * gq, make_float4(q[0], q[1], q[2], q[3]));
-      // every own row is written (zero beyond the grid): the adjoint multiplies these by zero there
-      if (STORE && !LAP && own && (!MULTI || p.slot_px))
-        st4_stream(p.slot_px + id0, rowok ? make_float4(pp[0], pp[1], pp[2], pp[3]) : make_float4(0.f, 0.f, 0.f, 0.f), pol);
-    };
-    // ---- stage 1b: z fluxes at one half row (the tile's halo rows)
-    auto qz_item = [&](int hr, int c) {
-      const int hz = z0 - 4 + hr, xc = x0 + 4 * c;
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int k = 1; k <= N; k++)
-        acc4(acc, cf.c1z[k - 1], ld4(su + (hr + 4 + k) * UW + 8 + 4 * c), ld4(su + (hr + 5 - k) * UW + 8 + 4 * c));
-      float pp[4];
-      f4a(acc, pp);
-      if (pmlz && layer_h(hz, hz, g.npml, g.nz)) {
-        const float aa = __ldg(p.azh + hz + TAB_OFF);
-        if (aa != 0.f) {
-          // psi' = b psi + a g, then p = g + psi': the same operations, in the same
-          // order, as the owner's update, so a half row computed here as halo and by
-          // its owner tile agrees bit for bit (whatever the tile height)
-          const float bb = __ldg(p.bzh + hz + TAB_OFF);
-          const float4 po = *reinterpret_cast<const float4*>(p.psiz_in + base + (long long)hz * pitch + xc);
-          pp[0] += fmaf(aa, pp[0], bb * po.x); pp[1] += fmaf(aa, pp[1], bb * po.y);
-          pp[2] += fmaf(aa, pp[2], bb * po.z); pp[3] += fmaf(aa, pp[3], bb * po.w);
-        }
-      }
-      const float4 ma = ld4(sm + hr * MW + 4 * c + 4), mb = ld4(sm + (hr + 1) * MW + 4 * c + 4);
-      const bool hv = hz >= 0 && hz < g.Nz - 1;
-      const float q0 = (hv && xc + 0 < g.Nx) ? (LAP ? pp[0] : (ma.x + mb.x) * pp[0]) : 0.f;
-      const float q1 = (hv && xc + 1 < g.Nx) ? (LAP ? pp[1] : (ma.y + mb.y) * pp[1]) : 0.f;
-      const float q2 = (hv && xc + 2 < g.Nx) ? (LAP ? pp[2] : (ma.z + mb.z) * pp[2]) : 0.f;
-      const float q3 = (hv && xc + 3 < g.Nx) ? (LAP ? pp[3] : (ma.w + mb.w) * pp[3]) : 0.f;
-      st4(sh.qz + hr * TILE_X + 4 * c, make_float4(q0, q1, q2, q3));
-    };
-
-    qx_item(2 * ty, tx + 1, true);
-    qx_item(2 * ty + 1, tx + 1, true);
-    {
-      // own z fluxes at half rows 2ty, 2ty+1 (tile-local) from a (2N+1)-row window
-      float4 w[2 * N + 1];
-#pragma unroll
-      for (int t2 = 0; t2 <= 2 * N; t2++) w[t2] = ld4(su + (2 * ty + H - N + 1 + t2) * UW + 8 + 4 * tx);
-      float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
-#pragma unroll
-      for (int k = 1; k <= N; k++) {
-        acc4(a0, cf.c1z[k - 1], w[k + N - 1], w[N - k]);
-        acc4(a1, cf.c1z[k - 1], w[k + N], w[N - k + 1]);
-      }
-      float pp[2][4];
-      f4a(a0, pp[0]);
-      f4a(a1, pp[1]);
-#pragma unroll
-      for (int rr = 0; rr < 2; rr++) {
-        const int hz = zr0 + rr;
-        const long long idz = base + (long long)hz * pitch + xb;
-        if (pmlz && layer_h(hz, hz, g.npml, g.nz)) {
+    // the tile body, compiled three times: for tiles inside the grid and its layers
+    // without a source or receivers; with the rows' layers and edges, sources and
+    // receivers (GZ); and with those of the columns as well (XG)
+    auto tile_body = [&](auto xg_c, auto gz_c) {
+      constexpr bool XG = decltype(xg_c)::value, GZ = decltype(gz_c)::value;
+      const bool gz = GZ && gz_t;
+      const float* su = sh.u;
+      const float* sm = sh.m;
+      // ---- z flux q = m_half (D+u + psi) at one half row, columns xc .. xc+3, from g = D+u
+      auto zflux = [&](Q4 pp, int hz, int xc, Q4 ma, Q4 mb, Q4 psi, bool mine) -> Q4 {
+        if (gz && pmlz && layer_h(hz, hz, g.npml, g.nz)) {
           const float aa = __ldg(p.azh + hz + TAB_OFF);
           if (aa != 0.f) {
+            // psi' = b psi + a g, then p = g + psi'
             const float bb = __ldg(p.bzh + hz + TAB_OFF);
-            const float4 po = *reinterpret_cast<const float4*>(p.psiz_in + idz);
-            float4 pn;  // the operations of the halo items' update, in the same order
-            pn.x = fmaf(aa, pp[rr][0], bb * po.x); pn.y = fmaf(aa, pp[rr][1], bb * po.y);
-            pn.z = fmaf(aa, pp[rr][2], bb * po.z); pn.w = fmaf(aa, pp[rr][3], bb * po.w);
-            if (xb + 0 >= g.Nx) pn.x = 0.f;
-            if (xb + 1 >= g.Nx) pn.y = 0.f;
-            if (xb + 2 >= g.Nx) pn.z = 0.f;
-            if (xb + 3 >= g.Nx) pn.w = 0.f;
-            st4(p.psiz_out + idz, pn);
-            pp[rr][0] += pn.x; pp[rr][1] += pn.y; pp[rr][2] += pn.z; pp[rr][3] += pn.w;
+            const long long idz = base + (long long)hz * pitch + xc;
+            Q4 pn = fma4(pk(aa, aa), pp, scale4(pk(bb, bb), PRE ? psi : ldq(p.psiz_in + idz)));
+            if (mine) {
+              if (XG) pn = mask_cols(pn, xc, g.Nx);
+              stq(p.psiz_out + idz, pn);
+            }
+            pp = add4(pp, pn);
           }
         }
-        const float4 ma = ld4(sm + (2 * ty + 4 + rr) * MW + 4 * tx + 4);
-        const float4 mb = ld4(sm + (2 * ty + 5 + rr) * MW + 4 * tx + 4);
-        const bool hv = hz < g.Nz - 1;
-        float q[4];
-        q[0] = (hv && xb + 0 < g.Nx) ? (LAP ? pp[rr][0] : (ma.x + mb.x) * pp[rr][0]) : 0.f;
-        q[1] = (hv && xb + 1 < g.Nx) ? (LAP ? pp[rr][1] : (ma.y + mb.y) * pp[rr][1]) : 0.f;
-        q[2] = (hv && xb + 2 < g.Nx) ? (LAP ? pp[rr][2] : (ma.z + mb.z) * pp[rr][2]) : 0.f;
-        q[3] = (hv && xb + 3 < g.Nx) ? (LAP ? pp[rr][3] : (ma.w + mb.w) * pp[rr][3]) : 0.f;
-        st4(sh.qz + (2 * ty + 4 + rr) * TILE_X + 4 * tx, make_float4(q[0], q[1], q[2], q[3]));
-        if (STORE && !LAP && (!MULTI || p.slot_pz))
-          st4_stream(p.slot_pz + idz, hz < g.Nz ? make_float4(pp[rr][0], pp[rr][1], pp[rr][2], pp[rr][3])
-                                                : make_float4(0.f, 0.f, 0.f, 0.f), pol);
-      }
-    }
-    if (tid < 128) {  // the 8 halo half rows, 16 items each
-      const int hr0 = tid >> 4;
-      qz_item(hr0 < 4 ? hr0 : hr0 + TZ, tid & 15);
-    } else if (tid < 128 + 2 * TZ) {  // the two halo column groups of every row
-      const int k = tid - 128;
-      qx_item(k >> 1, (k & 1) ? QXW / 4 - 1 : 0, false);
-    }
-    // u^n at the own cells (and, for the Laplacian operator, m/2 there), read
-    // before the operand buffer is refilled
-    float4 ucur[2], mown[2];
-    ucur[0] = ld4(su + (2 * ty + H) * UW + 4 * tx + H);
-    ucur[1] = ld4(su + (2 * ty + 1 + H) * UW + 4 * tx + H);
-    if (LAP) {
-      mown[0] = ld4(sm + (2 * ty + 4) * MW + 4 * tx + 4);
-      mown[1] = ld4(sm + (2 * ty + 5) * MW + 4 * tx + 4);
-    }
-    __syncthreads();
-    if (tid == 0 && tn < ntiles) fetch_next(tn);
+        if (STORE && !LAP && mine && (!MULTI || p.slot_pz))
+          stq_stream(p.slot_pz + base + (long long)hz * pitch + xc, gz && hz >= g.Nz ? zero4() : pp, pol);
+        Q4 q = LAP ? pp : mul4(add4(ma, mb), pp);
+        if (gz && (hz < 0 || hz >= g.Nz - 1)) q = zero4();
+        if (XG) q = mask_cols(q, xc, g.Nx);
+        return q;
+      };
+      // ---- x fluxes q = m_half (D+u + psi) at 4 half columns hb .. hb+3 of row r of the tile
+      auto xflux = [&](const float v[12], int r, int hb, const float mv[5], Q4 psi, bool mine, float q[4]) {
+        const int z = z0 + r;
+        float pp[4];
+        dplus_x<N>(cf.c1x, v, pp);
+        const bool rowok = !gz || z < g.Nz;
+        const long long id0 = base + (long long)z * pitch + hb;
+        if (XG && pmlx && layer_h(hb, hb + 3, g.npml, g.nx)) {
+          // psi <- b psi + a g; zero where a = 0 (psi stays zero outside the layer)
+          const float4 a4 = ldg4(p.axh + hb + TAB_OFF), b4 = ldg4(p.bxh + hb + TAB_OFF);
+          float po[4];
+          get4(PRE ? psi : ldq(p.psix_in + id0), po);
+          if (a4.x != 0.f || a4.y != 0.f || a4.z != 0.f || a4.w != 0.f) {
+            float4 pn;
+            pn.x = fmaf(b4.x, po[0], a4.x * pp[0]);
+            pn.y = fmaf(b4.y, po[1], a4.y * pp[1]);
+            pn.z = fmaf(b4.z, po[2], a4.z * pp[2]);
+            pn.w = fmaf(b4.w, po[3], a4.w * pp[3]);
+            if (mine && rowok) st4(p.psix_out + id0, pn);
+            pp[0] += pn.x; pp[1] += pn.y; pp[2] += pn.z; pp[3] += pn.w;
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+          q[e] = LAP ? pp[e] : (mv[e] + mv[e + 1]) * pp[e];
+          if (XG && !(hb + e >= 0 && hb + e < g.Nx - 1)) q[e] = 0.f;
+        }
+        // every own row is written (zero beyond the grid): the adjoint multiplies these by zero there
+        if (STORE && !LAP && mine && (!MULTI || p.slot_px)) stq_stream(p.slot_px + id0, rowok ? put4(pp) : zero4(), pol);
+        if (!rowok) q[0] = q[1] = q[2] = q[3] = 0.f;
+      };
 
-    // ---- stage 2: divergence + CPML zeta + leapfrog + source + receivers
-    cp_async_wait_all();  // this thread's own u^{n-1} copies
-    float hzv[2][4];
-    {
-      float4 w[2 * N + 1];
+      // ---- stage 1: fluxes of the own half points; the z window's middle rows are the
+      // own rows of u, the m rows serve both directions
+      Q4 uc[R], qz[R], mo[R + 1];
+      float qx[R][4];
 #pragma unroll
-      for (int t2 = 0; t2 <= 2 * N; t2++) w[t2] = ld4(sh.qz + (2 * ty + 4 - N + t2) * TILE_X + 4 * tx);
-      float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+      for (int i = 0; i <= R; i++) mo[i] = ldq(sm + (R * ty + 4 + i) * MW + 4 * tx + 4);
+      {
+        Q4 w[WR];
 #pragma unroll
-      for (int k = 1; k <= N; k++) {
-        acc4(a0, cf.c2z[k - 1], w[k + N - 1], w[N - k]);
-        acc4(a1, cf.c2z[k - 1], w[k + N], w[N - k + 1]);
+        for (int i = 0; i < WR; i++) w[i] = ldq(su + (R * ty + H - N + 1 + i) * UW + H + 4 * tx);
+        dz<N, R>(cf.c1z2, w, qz);
+#pragma unroll
+        for (int i = 0; i < R; i++) uc[i] = w[N - 1 + i];
       }
-      f4a(a0, hzv[0]);
-      f4a(a1, hzv[1]);
-    }
-    const int i0 = box.x, j0 = box.y, nb = p.src_n;
-    const bool srcbox = i0 >= 0 && i0 < z0 + TZ && i0 + nb > z0 && j0 < x0 + TILE_X && j0 + nb > x0;
-    float4 ax4 = make_float4(0.f, 0.f, 0.f, 0.f), bx4 = ax4;
-    if (pmlx && layer_c(xb, xb + 3, g.npml, g.nx)) ax4 = ldg4(p.ax + xb + TAB_OFF);
-    const bool zx_on = ax4.x != 0.f || ax4.y != 0.f || ax4.z != 0.f || ax4.w != 0.f;
-    if (zx_on) bx4 = ldg4(p.bx + xb + TAB_OFF);
-    float un[2][4];
 #pragma unroll
-    for (int rr = 0; rr < 2; rr++) {
-      const int r = 2 * ty + rr, z = z0 + r;
-      const long long idc0 = base + (long long)z * pitch + xb;
-      float v[12];
-      unpack12(sh.qx + r * QXW + 4 * tx, v);
-      float hxv[4], rv[4];
-#pragma unroll
-      for (int e = 0; e < 4; e++) {
-        float hx = 0.f;
-#pragma unroll
-        for (int k = 1; k <= N; k++) hx += cf.c2x[k - 1] * (v[e + k + 3] - v[e - k + 4]);
-        hxv[e] = hx;
-        rv[e] = hx + hzv[rr][e];
+      for (int rr = 0; rr < R; rr++) {
+        const int r = R * ty + rr;
+        qz[rr] = zflux(qz[rr], zr0 + rr, xb, mo[rr], mo[rr + 1], psz[rr], true);
+        stq(sh.qz + (r + 4) * TILE_X + 4 * tx, qz[rr]);
+        float v[12], mv[5];
+        const float* row = su + (r + H) * UW + H + 4 * tx;
+        get4(ldq(row - 4), v);
+        get4(uc[rr], v + 4);
+        get4(ldq(row + 4), v + 8);
+        get4(mo[rr], mv);
+        mv[4] = LAP ? 0.f : sm[(r + 4) * MW + 4 * tx + 8];
+        xflux(v, r, xb, mv, psx[rr], true, qx[rr]);
+        st4(sh.qx + r * QXW + 4 * tx + 4, make_float4(qx[rr][0], qx[rr][1], qx[rr][2], qx[rr][3]));
       }
-      // CPML zeta (dt^2-scaled) <- b zeta + a h; it stays zero where a = 0 and
-      // outside the grid (h = 0 there), so whole float4 groups are written
-      if (zx_on) {
-        const float4 zo = ld4(p.zetx + idc0);
-        float4 zn;
-        zn.x = bx4.x * zo.x + ax4.x * hxv[0]; zn.y = bx4.y * zo.y + ax4.y * hxv[1];
-        zn.z = bx4.z * zo.z + ax4.z * hxv[2]; zn.w = bx4.w * zo.w + ax4.w * hxv[3];
-        st4(p.zetx + idc0, zn);
-        rv[0] += zn.x; rv[1] += zn.y; rv[2] += zn.z; rv[3] += zn.w;
+      if (NT == 128 || tid < 128) {
+        // the 8 halo half rows, 16 items each
+        const int hr = hrh;
+        Q4 w[2 * N], q;
+#pragma unroll
+        for (int i = 0; i < 2 * N; i++) w[i] = ldq(su + (hr + 5 - N + i) * UW + H + 4 * tx);
+        dz<N, 1>(cf.c1z2, w, &q);
+        const Q4 ma = ldq(sm + hr * MW + 4 * tx + 4), mb = ldq(sm + (hr + 1) * MW + 4 * tx + 4);
+        stq(sh.qz + hr * TILE_X + 4 * tx, zflux(q, z0 - 4 + hr, xb, ma, mb, pszh, false));
       }
-      if (pmlz && layer_c(z, z, g.npml, g.nz)) {
-        const float aa = __ldg(p.az + z + TAB_OFF);
-        if (aa != 0.f) {
-          const float bb = __ldg(p.bz + z + TAB_OFF);
-          const float4 zo = ld4(p.zetz + idc0);
-          float4 zn;
-          zn.x = bb * zo.x + aa * hzv[rr][0]; zn.y = bb * zo.y + aa * hzv[rr][1];
-          zn.z = bb * zo.z + aa * hzv[rr][2]; zn.w = bb * zo.w + aa * hzv[rr][3];
-          st4(p.zetz + idc0, zn);
-          rv[0] += zn.x; rv[1] += zn.y; rv[2] += zn.z; rv[3] += zn.w;
+      // the two halo column groups of every row
+      if (xhalo) {
+        const int r = rxh, gq = gxh;
+        float v[12], mv[5], q[4];
+        unpack12(su + (r + H) * UW + 4 * gq, v);
+        get4(ldq(sm + (r + 4) * MW + 4 * gq), mv);
+        mv[4] = sm[(r + 4) * MW + 4 * gq + 4];
+        xflux(v, r, x0 - 4 + 4 * gq, mv, psxh, false, q);
+        st4(sh.qx + r * QXW + 4 * gq, make_float4(q[0], q[1], q[2], q[3]));
+      }
+      // PRE: CPML zeta of the own cells, issued before the barrier for the same reason
+      Q4 zex[R], zez[R];
+#pragma unroll
+      for (int rr = 0; rr < R; rr++) zex[rr] = zez[rr] = zero4();
+      const bool lcx = XG && pmlx && layer_c(xb, xb + 3, g.npml, g.nx);
+      if (PRE && lcx)
+#pragma unroll
+        for (int rr = 0; rr < R; rr++) zex[rr] = ldq(p.zetx + base + own + rr * pitch);
+      if (PRE && GZ && pmlz)
+#pragma unroll
+        for (int rr = 0; rr < R; rr++)
+          if (layer_c(zr0 + rr, zr0 + rr, g.npml, g.nz)) zez[rr] = ldq(p.zetz + base + own + rr * pitch);
+      __syncthreads();
+      if (tid == 0 && tn < ntiles) fetch_next(tn);
+
+      // ---- stage 2: divergence + CPML zeta + leapfrog + source + receivers
+      cp_async_wait_all();  // this thread's own u^{n-1} copies
+      Q4 hz[R];
+      {
+        Q4 w[WR];
+#pragma unroll
+        for (int i = 0; i < WR; i++)
+          w[i] = i >= N && i < N + R ? qz[i - N] : ldq(sh.qz + (R * ty + 4 - N + i) * TILE_X + 4 * tx);
+        dz<N, R>(cf.c2z2, w, hz);
+      }
+      float4 ax4 = make_float4(0.f, 0.f, 0.f, 0.f), bx4 = ax4;
+      if (lcx) {
+        ax4 = ldg4(p.ax + xb + TAB_OFF);
+        bx4 = ldg4(p.bx + xb + TAB_OFF);
+      }
+      const bool zx_on = XG && (ax4.x != 0.f || ax4.y != 0.f || ax4.z != 0.f || ax4.w != 0.f);
+      const bool srcbox = GZ && src_t;
+      const float amp = srcbox ? cf.dt2 * __ldg(p.stf + (long long)s * p.nt + p.n) : 0.f;
+#pragma unroll
+      for (int rr = 0; rr < R; rr++) {
+        const int r = R * ty + rr, z = z0 + r;
+        const long long idc = base + own + rr * pitch;
+        float v[12], hxv[4];
+        const float* row = sh.qx + r * QXW + 4 * tx + 4;
+        get4(ldq(row - 4), v);
+        v[4] = qx[rr][0]; v[5] = qx[rr][1]; v[6] = qx[rr][2]; v[7] = qx[rr][3];
+        get4(ldq(row + 4), v + 8);
+        dminus_x<N>(cf.c2x, v, hxv);
+        Q4 rv = add4(put4(hxv), hz[rr]);
+        // CPML zeta (dt^2-scaled) <- b zeta + a h; it stays zero where a = 0 and
+        // outside the grid (h = 0 there), so whole float4 groups are written
+        if (zx_on) {
+          float zo[4], zn[4];
+          get4(PRE ? zex[rr] : ldq(p.zetx + idc), zo);
+          zn[0] = fmaf(bx4.x, zo[0], ax4.x * hxv[0]);
+          zn[1] = fmaf(bx4.y, zo[1], ax4.y * hxv[1]);
+          zn[2] = fmaf(bx4.z, zo[2], ax4.z * hxv[2]);
+          zn[3] = fmaf(bx4.w, zo[3], ax4.w * hxv[3]);
+          const Q4 zq = put4(zn);
+          stq(p.zetx + idc, zq);
+          rv = add4(rv, zq);
         }
-      }
-      const float4 uc = ucur[rr];
-      const float4 upv = sh.up4[rr * NT + tid];
-      if (LAP) {
-        // r^n (dt^2-scaled) is the gradient operand; the update takes m r, m = 2 (m/2)
-        if (STORE) {
-          float r4[4];
-#pragma unroll
-          for (int e = 0; e < 4; e++) r4[e] = (z < g.Nz && xb + e < g.Nx) ? rv[e] : 0.f;  // zero off the grid
-          st4_stream(p.slot_px + idc0, make_float4(r4[0], r4[1], r4[2], r4[3]), pol);
+        if (gz && pmlz && layer_c(z, z, g.npml, g.nz)) {
+          const float aa = __ldg(p.az + z + TAB_OFF);
+          if (aa != 0.f) {
+            const float bb = __ldg(p.bz + z + TAB_OFF);
+            const Q4 zq = fma4(pk(bb, bb), PRE ? zez[rr] : ldq(p.zetz + idc), scale4(pk(aa, aa), hz[rr]));
+            stq(p.zetz + idc, zq);
+            rv = add4(rv, zq);
+          }
         }
-        rv[0] *= 2.f * mown[rr].x;
-        rv[1] *= 2.f * mown[rr].y;
-        rv[2] *= 2.f * mown[rr].z;
-        rv[3] *= 2.f * mown[rr].w;
-      }
-      un[rr][0] = 2.f * uc.x - upv.x + rv[0];
-      un[rr][1] = 2.f * uc.y - upv.y + rv[1];
-      un[rr][2] = 2.f * uc.z - upv.z + rv[2];
-      un[rr][3] = 2.f * uc.w - upv.w + rv[3];
-      if (srcbox) {
-        const int di = z - i0;
-        if (di >= 0 && di < nb) {
-          const float amp = cf.dt2 * stf_n;
+        if (LAP) {
+          // r^n (dt^2-scaled) is the gradient operand (zero off the grid); the update
+          // takes m r, m = 2 (m/2)
+          if (STORE) {
+            Q4 rs = XG ? mask_cols(rv, xb, g.Nx) : rv;
+            if (gz && z >= g.Nz) rs = zero4();
+            stq_stream(p.slot_px + idc, rs, pol);
+          }
+          rv = mul4(rv, add4(mo[rr], mo[rr]));
+        }
+        Q4 un = add4(sub4(add4(uc[rr], uc[rr]), ldq(reinterpret_cast<const float*>(&sh.up4[rr * NT + tid]))), rv);
+        if (srcbox) {
+          const int di = z - i0;
+          if (di >= 0 && di < nb) {
+            float u4[4];
+            get4(un, u4);
 #pragma unroll
-          for (int e = 0; e < 4; e++) {
-            const int dj = xb + e - j0;
-            if (dj >= 0 && dj < nb) un[rr][e] += amp * p.src_w[s * SRC_W * SRC_W + di * SRC_W + dj];
+            for (int e = 0; e < 4; e++) {
+              const int dj = xb + e - j0;
+              if (dj >= 0 && dj < nb) u4[e] = fmaf(amp, p.src_w[s * SRC_W * SRC_W + di * SRC_W + dj], u4[e]);
+            }
+            un = put4(u4);
+          }
+        }
+        if (XG) un = mask_cols(un, xb, g.Nx);
+        if (gz && z >= g.Nz) un = zero4();
+        stq(uprev + own + rr * pitch, un);
+        if (GZ && RECORD && has_rec && z / TILE_Z < g.ntz) {
+          const int key = ((z / TILE_Z) * g.ntx + id.tx) * NTHREADS + ((z % TILE_Z) >> 1) * 16 + tx;
+          const int rb = __ldg(p.thr_rec_start + key), re = __ldg(p.thr_rec_start + key + 1);
+          for (int q = rb; q < re; q++) {
+            const int code = p.thr_rec[q];  // (index << 3) | (row << 2) | column
+            if (((code >> 2) & 1) != (z & 1)) continue;
+            const int rc = code >> 3, e = code & 3;
+            float u4[4];
+            get4(un, u4);
+            p.seis[((long long)s * p.nrec + rc) * p.nt + p.n] = e == 0 ? u4[0] : (e == 1 ? u4[1] : (e == 2 ? u4[2] : u4[3]));
           }
         }
       }
-#pragma unroll
-      for (int e = 0; e < 4; e++)
-        if (!(z < g.Nz && xb + e < g.Nx)) un[rr][e] = 0.f;
-      st4(uprev + (long long)z * pitch + xb, make_float4(un[rr][0], un[rr][1], un[rr][2], un[rr][3]));
-    }
-    if (RECORD) {
-      // receivers of this thread's 2 x 4 cells: (index << 3) | (row << 2) | column
-      for (int q = rb; q < re; q++) {
-        const int code = p.thr_rec[q];
-        const int rc = code >> 3, rr = (code >> 2) & 1, e = code & 3;
-        const float* ur = un[rr];
-        p.seis[((long long)s * p.nrec + rc) * p.nt + p.n] = e == 0 ? ur[0] : (e == 1 ? ur[1] : (e == 2 ? ur[2] : ur[3]));
-      }
-    }
-    __syncthreads();  // the flux arrays are free again
+      __syncthreads();  // the flux arrays are free again
+    };
+    if (gx) tile_body(std::true_type{}, std::true_type{});
+    else if (gz_t || src_t || has_rec) tile_body(std::false_type{}, std::true_type{});
+    else tile_body(std::false_type{}, std::false_type{});
   }
 }
 
@@ -687,6 +835,8 @@ __global__ void __launch_bounds__(NTHREADS, 3)
     fence_mbar_init();
   }
   __syncthreads();
+  pdl_wait();
+  pdl_next();
   if (tid == 0 && (int)blockIdx.x < ntiles) fetch(blockIdx.x);
 
   int it = 0, inst_loaded = -1;
@@ -720,6 +870,32 @@ __global__ void __launch_bounds__(NTHREADS, 3)
       pfz[0] = pfz[1] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 
+    // CPML memory variables of the tile on their way to L1 while the tile is fetched
+    // (128 shots of 201 x 601: 214 -> 207 us per step)
+    if (tile_pml_z(g, z0)) {
+#pragma unroll
+      for (int rr = 0; rr < 2; rr++) {
+        const long long id0 = base + (long long)(zr0 + rr) * pitch + xb;
+        if (layer_h(zr0 + rr, zr0 + rr, g.npml, g.nz)) prefetch_l1(p.pz_in + id0);
+        if (layer_c(zr0 + rr, zr0 + rr, g.npml, g.nz)) prefetch_l1(p.zz_in + id0);
+      }
+      if (tid < 128) {
+        const int hr0 = tid >> 4, hz = z0 - 4 + (hr0 < 4 ? hr0 : hr0 + 32);
+        if (layer_h(hz, hz, g.npml, g.nz)) prefetch_l1(p.pz_in + base + (long long)hz * pitch + xb);
+      }
+    }
+    if (tile_pml_x(g, x0)) {
+#pragma unroll
+      for (int rr = 0; rr < 2; rr++) {
+        const long long id0 = base + (long long)(zr0 + rr) * pitch + xb;
+        if (layer_h(xb, xb + 3, g.npml, g.nx)) prefetch_l1(p.px_in + id0);
+        if (layer_c(xb, xb + 3, g.npml, g.nx)) prefetch_l1(p.zx_in + id0);
+      }
+      if (tid >= 128 && tid < 192) {
+        const int hb = x0 - 4 + 4 * ((tid & 1) ? QXW / 4 - 1 : 0);
+        if (layer_h(hb, hb + 3, g.npml, g.nx)) prefetch_l1(p.px_in + base + (long long)(z0 + ((tid - 128) >> 1)) * pitch + hb);
+      }
+    }
     const bool ok = mbar_wait(&sh.bar, it & 1);
     if (__syncthreads_or(!ok)) {
       if (tid == 0) {
@@ -1087,11 +1263,10 @@ namespace {
 
 std::mutex g_init_mu;
 unsigned long long g_inited = 0;  // bit per device
-// resident-CTA grids: single-instance forward variants (record, store), adjoint,
-// and the multi-instance forward sweep / recompute and adjoint
-int g_grid_fwd[64][2][4], g_grid_adj[64][2], g_grid_fwd_m[64][2][2], g_grid_adj_m[64][2];
-int g_grid_fwd64[64][2][4];  // the 64-row forward variants
-int g_grid_fwd_lap[64][2][4], g_grid_adj_lap[64][2];  // the c^2 Laplacian operator
+// resident-CTA grids: forward variants (rows per thread, operator, order, record
+// and store), adjoint, and the multi-instance forward sweep / recompute and adjoint
+int g_grid_fwd[64][FWD_SHAPES][2][2][4], g_grid_adj[64][2], g_grid_fwd_m[64][2][2], g_grid_adj_m[64][2];
+int g_grid_adj_lap[64][2];  // the c^2 Laplacian operator
 
 template <typename K>
 cudaError_t setup_kernel(K k, int smem, int* grid, int threads = NTHREADS) {
@@ -1105,37 +1280,44 @@ cudaError_t setup_kernel(K k, int smem, int* grid, int threads = NTHREADS) {
   return cudaSuccess;
 }
 
-constexpr int FWD_SMEM_M = (int)(FWD_SMEM_MAIN + sizeof(AcuStep));
+constexpr int FWD_SMEM_M = (int)(FWD_SMEM_MAIN<2, 16> + sizeof(AcuStep));
 constexpr int ADJ_SMEM_M = (int)(ADJ_SMEM_MAIN + sizeof(AcuStep));
+
+// The forward kernel of one variant.
+template <int N, int R, int TY, bool LAP>
+auto fwd_kernel(int v) {
+  return v == 0   ? acu_fwd_step<N, false, false, false, R, TY, LAP>
+         : v == 1 ? acu_fwd_step<N, true, false, false, R, TY, LAP>
+         : v == 2 ? acu_fwd_step<N, false, true, false, R, TY, LAP>
+                  : acu_fwd_step<N, true, true, false, R, TY, LAP>;
+}
+// Tile heights 8, 32 and 64: one, two and four rows per thread.
+template <int N, bool LAP>
+auto fwd_kernel(int shape, int v) {
+  return shape == 0 ? fwd_kernel<N, 1, 8, LAP>(v) : shape == 1 ? fwd_kernel<N, 2, 16, LAP>(v) : fwd_kernel<N, 4, 16, LAP>(v);
+}
+size_t fwd_smem(int shape) {
+  return shape == 0 ? sizeof(FwdSmemT<1, 8>) : shape == 1 ? sizeof(FwdSmemT<2, 16>) : sizeof(FwdSmemT<4, 16>);
+}
+int fwd_threads(int shape) { return shape == 0 ? 128 : 256; }
+constexpr int fwd_tz(int shape) { return shape == 0 ? 8 : shape == 1 ? 32 : 64; }
 
 template <int N>
 cudaError_t setup_order(int dev, int o) {
-  const int fs = (int)sizeof(FwdSmem), as = (int)sizeof(AdjSmem), f64 = (int)sizeof(FwdSmemT<64>);
-  constexpr int T64 = FwdGeo<64>::NT;
+  const int as = (int)sizeof(AdjSmem);
   cudaError_t e;
-  if ((e = setup_kernel(acu_fwd_step<N, false, false, false, 32>, fs, &g_grid_fwd[dev][o][0])) != cudaSuccess) return e;
-  if ((e = setup_kernel(acu_fwd_step<N, true, false, false, 32>, fs, &g_grid_fwd[dev][o][1])) != cudaSuccess) return e;
-  if ((e = setup_kernel(acu_fwd_step<N, false, true, false, 32>, fs, &g_grid_fwd[dev][o][2])) != cudaSuccess) return e;
-  if ((e = setup_kernel(acu_fwd_step<N, true, true, false, 32>, fs, &g_grid_fwd[dev][o][3])) != cudaSuccess) return e;
-  if ((e = setup_kernel(acu_fwd_step<N, false, false, false, 64>, f64, &g_grid_fwd64[dev][o][0], T64)) != cudaSuccess)
+  for (int sp = 0; sp < FWD_SHAPES; sp++)
+    for (int v = 0; v < 4; v++) {
+      const int fs = (int)fwd_smem(sp);
+      if ((e = setup_kernel(fwd_kernel<N, false>(sp, v), fs, &g_grid_fwd[dev][sp][0][o][v], fwd_threads(sp))) != cudaSuccess) return e;
+      if ((e = setup_kernel(fwd_kernel<N, true>(sp, v), fs, &g_grid_fwd[dev][sp][1][o][v], fwd_threads(sp))) != cudaSuccess) return e;
+    }
+  if ((e = setup_kernel(acu_fwd_step<N, true, true, true, 2, 16>, FWD_SMEM_M, &g_grid_fwd_m[dev][o][0], 256)) != cudaSuccess)
     return e;
-  if ((e = setup_kernel(acu_fwd_step<N, true, false, false, 64>, f64, &g_grid_fwd64[dev][o][1], T64)) != cudaSuccess)
-    return e;
-  if ((e = setup_kernel(acu_fwd_step<N, false, true, false, 64>, f64, &g_grid_fwd64[dev][o][2], T64)) != cudaSuccess)
-    return e;
-  if ((e = setup_kernel(acu_fwd_step<N, true, true, false, 64>, f64, &g_grid_fwd64[dev][o][3], T64)) != cudaSuccess)
-    return e;
-  if ((e = setup_kernel(acu_fwd_step<N, true, true, true, 32>, FWD_SMEM_M, &g_grid_fwd_m[dev][o][0])) != cudaSuccess)
-    return e;
-  if ((e = setup_kernel(acu_fwd_step<N, false, true, true, 32>, FWD_SMEM_M, &g_grid_fwd_m[dev][o][1])) != cudaSuccess)
+  if ((e = setup_kernel(acu_fwd_step<N, false, true, true, 2, 16>, FWD_SMEM_M, &g_grid_fwd_m[dev][o][1], 256)) != cudaSuccess)
     return e;
   if ((e = setup_kernel(acu_adj_step<N, false>, as, &g_grid_adj[dev][o])) != cudaSuccess) return e;
   if ((e = setup_kernel(acu_adj_step<N, false, true>, as, &g_grid_adj_lap[dev][o])) != cudaSuccess) return e;
-  for (int v = 0; v < 4; v++) {
-    auto k = v == 0 ? acu_fwd_step<N, false, false, false, 32, true> : v == 1 ? acu_fwd_step<N, true, false, false, 32, true>
-           : v == 2 ? acu_fwd_step<N, false, true, false, 32, true> : acu_fwd_step<N, true, true, false, 32, true>;
-    if ((e = setup_kernel(k, fs, &g_grid_fwd_lap[dev][o][v])) != cudaSuccess) return e;
-  }
   return setup_kernel(acu_adj_step<N, true>, ADJ_SMEM_M, &g_grid_adj_m[dev][o]);
 }
 
@@ -1162,10 +1344,41 @@ AcuCoef coef_of(const AcuStep& p) {
     c.c2z[k] = p.c2z[k];
   }
   c.dt2 = p.dt2;
+  acu_coef_pairs(c);
   return c;
 }
 
+// One step launch; its CTAs may be scheduled while the launch before it on the
+// stream drains (pdl_wait).
+template <typename... P, typename... A>
+cudaError_t launch_step(void (*kern)(P...), int grid, int threads, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 }  // namespace
+
+// The z weights of a step as packed pairs.
+void acu_coef_pairs(AcuCoef& c) {
+  auto pair = [](float v) {
+    unsigned int b;
+    memcpy(&b, &v, 4);
+    return ((unsigned long long)b << 32) | b;
+  };
+  for (int k = 0; k < 4; k++) {
+    c.c1z2[k] = pair(c.c1z[k]);
+    c.c2z2[k] = pair(c.c2z[k]);
+  }
+}
 
 cudaError_t launch_selftest_wait(int* status, unsigned long long* waited_ns, cudaStream_t st) {
   k_selftest_wait<<<1, 32, 0, st>>>(status, waited_ns);
@@ -1178,98 +1391,40 @@ cudaError_t acu_kernels_init() {
 }
 
 // TMA descriptors for a call: u is the [2][S][slice] wavefield pair, mh one
-// [slice] field.
+// [slice] field; one box per forward tile height, and the adjoint's m box.
 cudaError_t acu_make_maps(AcuMaps* maps, const Grid& g, int S, float* u_pair, const float* mh) {
   const cuuint64_t d3[3] = {(cuuint64_t)g.pitch, (cuuint64_t)g.rows, (cuuint64_t)(2 * S)};
   const cuuint64_t s3[2] = {(cuuint64_t)g.pitch * 4, (cuuint64_t)g.slice * 4};
-  const cuuint32_t b3[3] = {(cuuint32_t)UW, (cuuint32_t)UH, 1};
   const cuuint64_t d2[2] = {(cuuint64_t)g.pitch, (cuuint64_t)g.rows};
   const cuuint64_t s2[1] = {(cuuint64_t)g.pitch * 4};
-  const cuuint32_t b2[2] = {(cuuint32_t)MW, (cuuint32_t)MH};
-  if (!tma_host::encode(&maps->u, u_pair, 3, d3, s3, b3)) return cudaErrorInvalidValue;
-  if (!tma_host::encode(&maps->m, const_cast<float*>(mh), 2, d2, s2, b2)) return cudaErrorInvalidValue;
-  // the 64-row forward tiles (the layout's rows are padded to 64, so these boxes fit)
-  const cuuint32_t b3t[3] = {(cuuint32_t)UW, (cuuint32_t)FwdGeo<64>::UHT, 1};
-  const cuuint32_t b2t[2] = {(cuuint32_t)MW, (cuuint32_t)FwdGeo<64>::MHT};
-  if (!tma_host::encode(&maps->u64, u_pair, 3, d3, s3, b3t)) return cudaErrorInvalidValue;
-  if (!tma_host::encode(&maps->m64, const_cast<float*>(mh), 2, d2, s2, b2t)) return cudaErrorInvalidValue;
+  for (int sp = 0; sp < FWD_SHAPES; sp++) {
+    const int tz = fwd_tz(sp);
+    const cuuint32_t b3[3] = {(cuuint32_t)UW, (cuuint32_t)(tz + 2 * H), 1};
+    const cuuint32_t b2[2] = {(cuuint32_t)MW, (cuuint32_t)(tz + 9)};
+    if (!tma_host::encode(&maps->u[sp], u_pair, 3, d3, s3, b3)) return cudaErrorInvalidValue;
+    if (!tma_host::encode(&maps->m[sp], const_cast<float*>(mh), 2, d2, s2, b2)) return cudaErrorInvalidValue;
+  }
   return cudaSuccess;
 }
 
-// Forward step on tiles of tz rows (32 or 64; 64 needs the 64-row boxes of
-// acu_make_maps and is for single-instance launches).
-cudaError_t launch_acu_fwd_tz(const AcuStep& p_in, const AcuMaps& maps, bool record, bool store, int tz,
-                              cudaStream_t st, bool lap) {
+// Forward step on tiles of `rows` rows (8, 32 or 64).
+cudaError_t launch_acu_fwd(const AcuStep& p_in, const AcuMaps& maps, bool record, bool store, int rows, bool lap,
+                           cudaStream_t st) {
   int dev;
   cudaError_t e = ensure_init(&dev);
   if (e != cudaSuccess) return e;
   const int v = (record ? 1 : 0) + (store ? 2 : 0);
   const int o = p_in.N == 2 ? 0 : 1;
+  const int sp = rows == 64 ? 2 : rows == 32 ? 1 : 0;
   const AcuCoef cf = coef_of(p_in);
   BatchArgs nb;
   memset(&nb, 0, sizeof nb);
-  if (lap) {  // the c^2 Laplacian operator: 32-row tiles
-    const AcuStep& p = p_in;
-    const int grid = std::min(p.ntiles, g_grid_fwd_lap[dev][o][v]);
-    const size_t smem = sizeof(FwdSmem);
-#define FWD_LAUNCH(NN, R, S) \
-  acu_fwd_step<NN, R, S, false, 32, true><<<grid, NTHREADS, smem, st>>>(maps.u, maps.m, p, cf, nb)
-    if (p.N == 2) {
-      if (record && store) FWD_LAUNCH(2, true, true);
-      else if (record) FWD_LAUNCH(2, true, false);
-      else if (store) FWD_LAUNCH(2, false, true);
-      else FWD_LAUNCH(2, false, false);
-    } else {
-      if (record && store) FWD_LAUNCH(4, true, true);
-      else if (record) FWD_LAUNCH(4, true, false);
-      else if (store) FWD_LAUNCH(4, false, true);
-      else FWD_LAUNCH(4, false, false);
-    }
-#undef FWD_LAUNCH
-    return cudaGetLastError();
-  }
-  if (tz == 64) {
-    AcuStep p = p_in;
-    p.ntiles = p.S * p.g.ntx * ((p.g.Nz + 63) / 64);
-    const int grid = std::min(p.ntiles, g_grid_fwd64[dev][o][v]);
-    const size_t smem = sizeof(FwdSmemT<64>);
-    constexpr int T = FwdGeo<64>::NT;
-#define FWD_LAUNCH(NN, R, S) acu_fwd_step<NN, R, S, false, 64><<<grid, T, smem, st>>>(maps.u64, maps.m64, p, cf, nb)
-    if (p.N == 2) {
-      if (record && store) FWD_LAUNCH(2, true, true);
-      else if (record) FWD_LAUNCH(2, true, false);
-      else if (store) FWD_LAUNCH(2, false, true);
-      else FWD_LAUNCH(2, false, false);
-    } else {
-      if (record && store) FWD_LAUNCH(4, true, true);
-      else if (record) FWD_LAUNCH(4, true, false);
-      else if (store) FWD_LAUNCH(4, false, true);
-      else FWD_LAUNCH(4, false, false);
-    }
-#undef FWD_LAUNCH
-    return cudaGetLastError();
-  }
-  const AcuStep& p = p_in;
-  const int grid = std::min(p.ntiles, g_grid_fwd[dev][o][v]);
-  const size_t smem = sizeof(FwdSmem);
-#define FWD_LAUNCH(NN, R, S) acu_fwd_step<NN, R, S, false, 32><<<grid, NTHREADS, smem, st>>>(maps.u, maps.m, p, cf, nb)
-  if (p.N == 2) {
-    if (record && store) FWD_LAUNCH(2, true, true);
-    else if (record) FWD_LAUNCH(2, true, false);
-    else if (store) FWD_LAUNCH(2, false, true);
-    else FWD_LAUNCH(2, false, false);
-  } else {
-    if (record && store) FWD_LAUNCH(4, true, true);
-    else if (record) FWD_LAUNCH(4, true, false);
-    else if (store) FWD_LAUNCH(4, false, true);
-    else FWD_LAUNCH(4, false, false);
-  }
-#undef FWD_LAUNCH
-  return cudaGetLastError();
-}
-
-cudaError_t launch_acu_fwd(const AcuStep& p, const AcuMaps& maps, bool record, bool store, cudaStream_t st) {
-  return launch_acu_fwd_tz(p, maps, record, store, TILE_Z, st, false);
+  AcuStep p = p_in;
+  p.ntiles = p.S * p.g.ntx * ((p.g.Nz + fwd_tz(sp) - 1) / fwd_tz(sp));
+  const int grid = std::min(p.ntiles, g_grid_fwd[dev][sp][lap ? 1 : 0][o][v]);
+  auto k = p.N == 2 ? (lap ? fwd_kernel<2, true>(sp, v) : fwd_kernel<2, false>(sp, v))
+                    : (lap ? fwd_kernel<4, true>(sp, v) : fwd_kernel<4, false>(sp, v));
+  return launch_step(k, grid, fwd_threads(sp), fwd_smem(sp), st, maps.u[sp], maps.m[sp], p, cf, nb);
 }
 
 // Multi-instance forward step b.n over the tiles of instances [0, b.n_active):
@@ -1286,16 +1441,9 @@ cudaError_t launch_acu_fwd_batch(const BatchArgs& b, const AcuCoef& cf, int N, b
   memset(&none, 0, sizeof none);
   AcuStep p0;
   memset(&p0, 0, sizeof p0);
-#define FWD_LAUNCH(NN, R) acu_fwd_step<NN, R, true, true, 32><<<grid, NTHREADS, FWD_SMEM_M, st>>>(none, none, p0, cf, b)
-  if (N == 2) {
-    if (record) FWD_LAUNCH(2, true);
-    else FWD_LAUNCH(2, false);
-  } else {
-    if (record) FWD_LAUNCH(4, true);
-    else FWD_LAUNCH(4, false);
-  }
-#undef FWD_LAUNCH
-  return cudaGetLastError();
+  auto k = N == 2 ? (record ? acu_fwd_step<2, true, true, true, 2, 16> : acu_fwd_step<2, false, true, true, 2, 16>)
+                  : (record ? acu_fwd_step<4, true, true, true, 2, 16> : acu_fwd_step<4, false, true, true, 2, 16>);
+  return launch_step(k, grid, 256, FWD_SMEM_M, st, none, none, p0, cf, b);
 }
 
 // Adjoint operand maps: lambda and the hhat pairs Hx, Hz, each [2][S][slice],
@@ -1324,15 +1472,15 @@ cudaError_t launch_acu_adj(const AcuStep& p, const AcuMaps& maps, cudaStream_t s
   memset(&nb, 0, sizeof nb);
   if (lap) {
     if (p.N == 2)
-      acu_adj_step<2, false, true><<<grid, NTHREADS, smem, st>>>(maps.lx, maps.lz, maps.hx, maps.hz, maps.m, p, cf, nb);
+      return launch_step(acu_adj_step<2, false, true>, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
     else
-      acu_adj_step<4, false, true><<<grid, NTHREADS, smem, st>>>(maps.lx, maps.lz, maps.hx, maps.hz, maps.m, p, cf, nb);
+      return launch_step(acu_adj_step<4, false, true>, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
     return cudaGetLastError();
   }
   if (p.N == 2)
-    acu_adj_step<2, false><<<grid, NTHREADS, smem, st>>>(maps.lx, maps.lz, maps.hx, maps.hz, maps.m, p, cf, nb);
+    return launch_step(acu_adj_step<2, false>, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
   else
-    acu_adj_step<4, false><<<grid, NTHREADS, smem, st>>>(maps.lx, maps.lz, maps.hx, maps.hz, maps.m, p, cf, nb);
+    return launch_step(acu_adj_step<4, false>, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
   return cudaGetLastError();
 }
 
@@ -1347,8 +1495,8 @@ cudaError_t launch_acu_adj_batch(const BatchArgs& b, const AcuCoef& cf, int N, c
   memset(&none, 0, sizeof none);
   AcuStep p0;
   memset(&p0, 0, sizeof p0);
-  if (N == 2) acu_adj_step<2, true><<<grid, NTHREADS, ADJ_SMEM_M, st>>>(none, none, none, none, none, p0, cf, b);
-  else acu_adj_step<4, true><<<grid, NTHREADS, ADJ_SMEM_M, st>>>(none, none, none, none, none, p0, cf, b);
+  if (N == 2) return launch_step(acu_adj_step<2, true>, grid, NTHREADS, ADJ_SMEM_M, st, none, none, none, none, none, p0, cf, b);
+  else return launch_step(acu_adj_step<4, true>, grid, NTHREADS, ADJ_SMEM_M, st, none, none, none, none, none, p0, cf, b);
   return cudaGetLastError();
 }
 

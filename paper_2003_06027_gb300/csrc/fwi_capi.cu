@@ -21,9 +21,9 @@
 #include "fwi_internal.cuh"
 
 namespace fwi {
-cudaError_t launch_acu_fwd(const AcuStep& p, const AcuMaps& maps, bool record, bool store, cudaStream_t st);
-cudaError_t launch_acu_fwd_tz(const AcuStep& p, const AcuMaps& maps, bool record, bool store, int tz, cudaStream_t st,
-                              bool lap);
+cudaError_t launch_acu_fwd(const AcuStep& p, const AcuMaps& maps, bool record, bool store, int rows, bool lap,
+                           cudaStream_t st);
+void acu_coef_pairs(AcuCoef& c);
 cudaError_t launch_acu_adj(const AcuStep& p, const AcuMaps& maps, cudaStream_t st, bool lap);
 cudaError_t launch_acu_fwd_batch(const BatchArgs& b, const AcuCoef& cf, int N, bool record, cudaStream_t st);
 cudaError_t launch_acu_adj_batch(const BatchArgs& b, const AcuCoef& cf, int N, cudaStream_t st);
@@ -387,10 +387,10 @@ fwi_status finish_status(fwi_ctx* ctx, const Plan& P, cudaStream_t st) { return 
 // fill them. Everything that couples shots (misfit, folds, source gradients)
 // runs on the call's stream after a join.
 constexpr int MAX_GROUPS = 4;
-// The adjoint step kernel runs fewer, larger groups: measured on 16 shots of the
-// 201 x 601 problem, 2 groups gave 26.8 us per step against 27.2 with 4 (the
-// forward kernels prefer 4: 16.4 against 18.6 us).
-constexpr int ADJ_GROUPS = 2;
+// Groups by default, measured on 16 shots of the 201 x 601 problem: the recording
+// forward step 15.1 us with 2 groups against 15.6 with 4, the storing one (which
+// runs more CTAs per SM) 16.6 against 14.8, the adjoint step 25.0 against 25.9.
+constexpr int FWD_GROUPS = 2, STORE_GROUPS = 4, ADJ_GROUPS = 2;
 
 struct Groups {
   int G = 1;
@@ -436,7 +436,9 @@ fwi_status join(fwi_ctx* ctx, const Groups& gr, cudaStream_t main) {
 }
 
 // Tile height of the context's acoustic forward steps.
-int fwd_tz(const fwi_ctx* ctx) { return ctx->fwd_tile_rows == 64 ? 64 : TILE_Z; }
+int fwd_rows(const fwi_ctx* ctx, int S, const Grid& g) {
+  return ctx->fwd_tile_rows ? ctx->fwd_tile_rows : acu_fwd_rows(S, g);
+}
 
 // The step parameters of one group: shots [s0, s0 + Sg). Per-shot arrays are
 // offset to the group's first shot; the u and lambda pairs keep their base and
@@ -669,15 +671,16 @@ fwi_status fwi_forward(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* Sv, 
   CK(acu_make_maps(&maps, P.g, P.S, P.u, P.m));
   ensure_events(ctx, 0);
   Groups gr;
-  if ((v = make_groups(ctx, P.S, st, gr, ctx->fwd_groups ? ctx->fwd_groups : MAX_GROUPS)) != FWI_OK) return v;
+  if ((v = make_groups(ctx, P.S, st, gr, ctx->fwd_groups ? ctx->fwd_groups : FWD_GROUPS)) != FWI_OK) return v;
   CK(cudaEventRecord(ctx->ev[0], st));
   if ((v = fork(ctx, gr, st)) != FWI_OK) return v;
   const size_t fieldf = (size_t)P.S * P.g.slice;
   const float lscale = (float)((double)dt * dt / ((double)M->dx * M->dz));
+  const int rows = fwd_rows(ctx, P.S, P.g);
   for (int n = 0; n < nt; n++) {
     set_fwd_state(P, p, n);
     for (int g = 0; g < gr.G; g++) {
-      LK(1, launch_acu_fwd_tz(group_view(p, P, gr.s0[g], gr.n[g]), maps, true, false, fwd_tz(ctx), gr.st[g], lap));
+      LK(1, launch_acu_fwd(group_view(p, P, gr.s0[g], gr.n[g]), maps, true, false, rows, lap, gr.st[g]));
       if (P.L > 0)
         LK(1, launch_line_inject(gr.n[g], P.L, n, nt, lscale, P.stf + (size_t)gr.s0[g] * nt * P.L,
                                  P.line_cell + 2 * gr.s0[g], P.u + ((n + 1) & 1) * fieldf + gr.s0[g] * P.g.slice,
@@ -776,10 +779,12 @@ fwi_status acu_misfit_grad(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* 
   CK(acu_make_adj_maps(&maps, P.g, P.S, P.lam, P.hx, P.hz));
   ensure_events(ctx, P.nseg);
 
-  Groups gr, gra;
-  if ((v = make_groups(ctx, P.S, st, gr, ctx->fwd_groups ? ctx->fwd_groups : MAX_GROUPS)) != FWI_OK) return v;
+  Groups gr, grs, gra;  // forward sweep, recomputed segments, adjoint
+  if ((v = make_groups(ctx, P.S, st, gr, ctx->fwd_groups ? ctx->fwd_groups : FWD_GROUPS)) != FWI_OK) return v;
+  if ((v = make_groups(ctx, P.S, st, grs, ctx->fwd_groups ? ctx->fwd_groups : STORE_GROUPS)) != FWI_OK) return v;
   if ((v = make_groups(ctx, P.S, st, gra, ctx->adj_groups ? ctx->adj_groups : ADJ_GROUPS)) != FWI_OK) return v;
   const size_t sl = (size_t)P.g.slice;
+  const int rows = fwd_rows(ctx, P.S, P.g);
 
   // forward sweep with a full-state checkpoint at the start of every segment
   // but the last: the sweep itself keeps the last segment's fluxes (recording
@@ -804,7 +809,7 @@ fwi_status acu_misfit_grad(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* 
       p.slot_pz = lap ? nullptr : p.slot_px + field;
     }
     for (int g = 0; g < gr.G; g++) {
-      LK(1, launch_acu_fwd_tz(group_view(p, P, gr.s0[g], gr.n[g]), maps, true, keep, fwd_tz(ctx), gr.st[g], lap));
+      LK(1, launch_acu_fwd(group_view(p, P, gr.s0[g], gr.n[g]), maps, true, keep, rows, lap, gr.st[g]));
       if (P.L > 0)
         LK(1, launch_line_inject(gr.n[g], P.L, n, nt, lscale, P.stf + (size_t)gr.s0[g] * nt * P.L,
                                  P.line_cell + 2 * gr.s0[g], P.u + ((n + 1) & 1) * field + gr.s0[g] * sl, P.g,
@@ -833,24 +838,24 @@ fwi_status acu_misfit_grad(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* 
     // fluxes are already stored by the forward sweep
     CK(mark(ctx->seg_ev[4 * seg + 0], st, capture));
     if (seg < P.nseg - 1) {
-      if ((v = fork(ctx, gr, st)) != FWI_OK) return v;
-      for (int g = 0; g < gr.G; g++)
+      if ((v = fork(ctx, grs, st)) != FWI_OK) return v;
+      for (int g = 0; g < grs.G; g++)
         for (int f = 0; f < 6; f++)
-          CK(cudaMemcpyAsync(dst[f] + gr.s0[g] * sl, ck + f * field + gr.s0[g] * sl, gr.n[g] * sl * 4,
-                             cudaMemcpyDeviceToDevice, gr.st[g]));
+          CK(cudaMemcpyAsync(dst[f] + grs.s0[g] * sl, ck + f * field + grs.s0[g] * sl, grs.n[g] * sl * 4,
+                             cudaMemcpyDeviceToDevice, grs.st[g]));
       for (int n = n0; n < n1; n++) {
         set_fwd_state(P, p, n);
         p.slot_px = P.slot + (size_t)(n - n0) * P.slot_fields * field;
         p.slot_pz = lap ? nullptr : p.slot_px + field;
-        for (int g = 0; g < gr.G; g++) {
-          LK(1, launch_acu_fwd_tz(group_view(p, P, gr.s0[g], gr.n[g]), maps, false, true, fwd_tz(ctx), gr.st[g], lap));
+        for (int g = 0; g < grs.G; g++) {
+          LK(1, launch_acu_fwd(group_view(p, P, grs.s0[g], grs.n[g]), maps, false, true, rows, lap, grs.st[g]));
           if (P.L > 0)
-            LK(1, launch_line_inject(gr.n[g], P.L, n, nt, lscale, P.stf + (size_t)gr.s0[g] * nt * P.L,
-                                     P.line_cell + 2 * gr.s0[g], P.u + ((n + 1) & 1) * field + gr.s0[g] * sl, P.g,
-                                     P.rec_cell, P.nrec, nullptr, gr.st[g]));
+            LK(1, launch_line_inject(grs.n[g], P.L, n, nt, lscale, P.stf + (size_t)grs.s0[g] * nt * P.L,
+                                     P.line_cell + 2 * grs.s0[g], P.u + ((n + 1) & 1) * field + grs.s0[g] * sl, P.g,
+                                     P.rec_cell, P.nrec, nullptr, grs.st[g]));
         }
       }
-      if ((v = join(ctx, gr, st)) != FWI_OK) return v;
+      if ((v = join(ctx, grs, st)) != FWI_OK) return v;
     }
     CK(mark(ctx->seg_ev[4 * seg + 1], st, capture));
     if ((v = fork(ctx, gra, st)) != FWI_OK) return v;
@@ -1344,8 +1349,8 @@ fwi_status fwi_batch_create(int32_t device, int32_t n, const fwi_model* models, 
     AcuMaps mp;
     BCK(acu_make_maps(&mp, P.g, P.S, P.u, P.m));
     BCK(acu_make_adj_maps(&mp, P.g, P.S, P.lam, P.hx, P.hz));
-    in.mu = mp.u;
-    in.mm = mp.m;
+    in.mu = mp.u[1];  // 32-row tiles
+    in.mm = mp.m[1];
     in.lx = mp.lx;
     in.lz = mp.lz;
     in.hx = mp.hx;
@@ -1383,6 +1388,8 @@ fwi_status fwi_batch_create(int32_t device, int32_t n, const fwi_model* models, 
         B->cf_adj.c2z[k] = in.p.c1z[k];
       }
       B->cf_fwd.dt2 = B->cf_adj.dt2 = in.p.dt2;
+      acu_coef_pairs(B->cf_fwd);
+      acu_coef_pairs(B->cf_adj);
     }
   }
   // checkpoint k (step kK) of every instance whose last segment starts later

@@ -35,7 +35,8 @@
 #include "fwi_internal.cuh"
 
 namespace fwi {
-cudaError_t launch_acu_fwd(const AcuStep& p, const AcuMaps& maps, bool record, bool store, cudaStream_t st);
+cudaError_t launch_acu_fwd(const AcuStep& p, const AcuMaps& maps, bool record, bool store, int rows, bool lap,
+                           cudaStream_t st);
 cudaError_t acu_make_maps(AcuMaps* maps, const Grid& g, int S, float* u_pair, const float* mh);
 cudaError_t launch_pad_model(const float* c, const Grid& g, float* m, cudaStream_t st);
 cudaError_t launch_cpml_tables(int n_phys, int npml, int Npad, int len, double h, double dt, double R,
@@ -258,7 +259,7 @@ extern "C" fwi_status fwi_forward_noalloc(const fwi_model* M, const fwi_sources*
     p.psix_out = psix[(n + 1) & 1];
     p.psiz_in = psiz[n & 1];
     p.psiz_out = psiz[(n + 1) & 1];
-    NA_CK(launch_acu_fwd(p, maps, true, false, st));
+    NA_CK(launch_acu_fwd(p, maps, true, false, acu_fwd_rows(S, g), false, st));
   }
   const long long ns = (long long)S * nrec * nt;
   if (ns > 0) NA_CK(launch_finite_check(seis, ns, status, st));
