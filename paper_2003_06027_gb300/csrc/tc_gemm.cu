@@ -107,7 +107,9 @@ __device__ __forceinline__ uint32_t mulhi_div(uint32_t n, unsigned long long m, 
 // warps 0-7 gather A (two threads per tile row, 32 taps each; warps 0-3 also
 // run the epilogue), warp 8 loads B by TMA, warp 9 issues the MMAs. Up to two
 // CONV CTAs share an SM, so that one's gather covers the other's load latency.
-template <bool CONV>
+// CONV: 0 A by TMA, 1 gathered tap by tap through a table (any layer), 2 and 3
+// gathered by pixel pairs (layers of horizontal stride 1 and 2).
+template <int CONV>
 struct TcRoles {
   static constexpr int THREADS = CONV ? 320 : TC_THREADS;
   static constexpr int GATHER = 2 * TC_BM;  // gathering threads (CONV)
@@ -174,7 +176,118 @@ __device__ __forceinline__ void gather_store(const float v[GATHER_K], int row, i
   }
 }
 
-template <bool CONV>
+// Gathers A by pixel pairs: thread (pair, sub) of 64 x 4 builds rows 2 pair and
+// 2 pair + 1 of every stage tile (two neighbouring output pixels of one image
+// row), taking every fourth run of 8 channels. The 72 taps of 8 channels are 9
+// whole 16-byte chunks of a row, so a run's values go from registers to shared
+// memory without a table: per channel a thread reads the 3 x (2 SW + 2) input
+// values of its pair once (9 loads for 18 operand elements at SW = 1), and each
+// BF16 word is one packed conversion of two of them. About 1.6 instructions per
+// element against 6 for the table (each tap decoded, tested and loaded by
+// itself), which is what bounds these GEMMs: their layers are thin, and the
+// tensor pipe waits for A. The operand is the same, so the results are too.
+// Every thread enters (waits for) and leaves (arrives on) every k-block's stage
+// in order, whether it has chunks there or not.
+template <int SW>
+__device__ __forceinline__ bool gather_pairs(const TcConvA& c, long long m0, long long M, int nk, unsigned char* smA,
+                                             uint64_t* empty, uint64_t* fulla) {
+  constexpr int NV = SW + 3;  // input columns SW j - 1 .. SW j + SW + 1 of a pair
+  const int pair = threadIdx.x & 63, sub = threadIdx.x >> 6, row = 2 * pair;
+  const long long m = m0 + row, plane = (long long)c.B * c.H * c.W;
+  const float* base = c.x;
+  bool rok[3] = {false, false, false}, left = false, right = false;
+  if (m < M) {  // the pair's pixels are both inside: Wo is even
+    const uint32_t bi = mulhi_div((uint32_t)m, c.wo_m, c.wo_s);
+    const int j = (int)((uint32_t)m - bi * (uint32_t)c.Wo);
+    const uint32_t b = mulhi_div(bi, c.ho_m, c.ho_s);
+    const int i = (int)(bi - b * (uint32_t)c.Ho), r0 = c.sh * i - 1;
+    base += ((long long)b * c.H + r0) * c.W + SW * j;
+#pragma unroll
+    for (int p = 0; p < 3; p++) rok[p] = r0 + p >= 0 && r0 + p < c.H;
+    left = SW * j - 1 >= 0;
+    right = SW == 2 || j + 2 < c.W;
+  }
+  const int nchunk = nk * (TC_BK / 8);
+  int cur = -1;  // k-block whose stage this thread has entered
+  auto enter = [&](int kb) -> bool {
+    while (cur < kb) {
+      if (cur >= 0) {
+        fence_proxy_async();  // the generic-proxy writes before the tensor core reads them
+        mbar_arrive(&fulla[cur % TC_STAGES]);
+      }
+      cur++;
+      if (!mbar_wait(&empty[cur % TC_STAGES], ((uint32_t)(cur / TC_STAGES) & 1u) ^ 1u)) return false;
+    }
+    return true;
+  };
+  const int sw0 = row & 7;
+  for (int g0 = 9 * sub; g0 < nchunk; g0 += 36) {  // chunks g0 .. g0 + 8: channels 8 g0 / 9 ..
+    const int ch0 = 8 * (g0 / 9);
+    uint32_t w0[20], w1[20];  // BF16 words of the two rows: two carried over, 18 of four channels
+#pragma unroll
+    for (int half = 0; half < 2; half++) {
+      float v[4][3][NV];
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        const int ch = ch0 + 4 * half + u;
+        const float* xc = base + (long long)ch * plane;
+        const bool cok = ch < c.C;
+#pragma unroll
+        for (int p = 0; p < 3; p++) {
+          const float* q = xc + p * c.W;
+          const bool ok = cok && rok[p];
+          v[u][p][0] = ok && left ? __ldg(q - 1) : 0.f;
+          if (SW == 1) {
+            const float2 t = ok ? __ldg(reinterpret_cast<const float2*>(q)) : make_float2(0.f, 0.f);
+            v[u][p][1] = t.x;
+            v[u][p][2] = t.y;
+            v[u][p][3] = ok && right ? __ldg(q + 2) : 0.f;
+          } else {
+            const float4 t = ok ? __ldg(reinterpret_cast<const float4*>(q)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[u][p][1] = t.x;
+            v[u][p][2] = t.y;
+            v[u][p][3] = t.z;
+            v[u][p][NV - 1] = t.w;
+          }
+        }
+      }
+      // tap e of the four channels: (channel e / 9, row e % 9 / 3, column e % 3)
+#pragma unroll
+      for (int k = 0; k < 18; k++) {
+        const int e = 2 * k, f = 2 * k + 1;
+        const __nv_bfloat162 h0 = __floats2bfloat162_rn(v[e / 9][e % 9 / 3][e % 3], v[f / 9][f % 9 / 3][f % 3]);
+        const __nv_bfloat162 h1 =
+            __floats2bfloat162_rn(v[e / 9][e % 9 / 3][e % 3 + SW], v[f / 9][f % 9 / 3][f % 3 + SW]);
+        w0[(half ? 2 : 0) + k] = *reinterpret_cast<const uint32_t*>(&h0);
+        w1[(half ? 2 : 0) + k] = *reinterpret_cast<const uint32_t*>(&h1);
+      }
+#pragma unroll
+      for (int k = 0; k < 4 + half; k++) {
+        const int g = g0 + 4 * half + k;
+        if (g < nchunk) {
+          if (!enter(g >> 3)) return false;
+          unsigned char* rp = smA + (cur % TC_STAGES) * A_STAGE + row * 128;
+          *reinterpret_cast<uint4*>(rp + (((g & 7) ^ sw0) << 4)) =
+              make_uint4(w0[4 * k], w0[4 * k + 1], w0[4 * k + 2], w0[4 * k + 3]);
+          *reinterpret_cast<uint4*>(rp + 128 + (((g & 7) ^ (sw0 + 1)) << 4)) =
+              make_uint4(w1[4 * k], w1[4 * k + 1], w1[4 * k + 2], w1[4 * k + 3]);
+        }
+      }
+      if (half == 0) {  // words 16, 17 open the fifth chunk
+        w0[0] = w0[16];
+        w0[1] = w0[17];
+        w1[0] = w1[16];
+        w1[1] = w1[17];
+      }
+    }
+  }
+  if (!enter(nk - 1)) return false;
+  fence_proxy_async();
+  mbar_arrive(&fulla[cur % TC_STAGES]);
+  return true;
+}
+
+template <int CONV>
 __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
     k_tc_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, const TcArgs a,
               const TcConvA conv) {
@@ -189,7 +302,7 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
   const int B_STAGE = a.BN * TC_BK * 2;
   unsigned char* smB = smA + TC_STAGES * A_STAGE;
   int2* tab = nullptr;
-  if (CONV) {  // after the stages: a.nkb k-blocks of (offset, tap bit) entries
+  if (CONV == 1) {  // after the stages: a.nkb k-blocks of (offset, tap bit) entries
     const int K9 = 9 * conv.C, len = a.nkb * TC_BK;
     tab = reinterpret_cast<int2*>(smB + TC_STAGES * a.BN * TC_BK * 2);
     const int plane = conv.B * conv.H * conv.W;
@@ -257,7 +370,9 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
       tc_commit(&empty[s]);
     }
     tc_commit(&accb);
-  } else if (CONV && (int)threadIdx.x < R::GATHER) {
+  } else if (CONV >= 2 && (int)threadIdx.x < R::GATHER) {
+    if (!gather_pairs<CONV >= 2 ? CONV - 1 : 1>(conv, m0, a.M, nk, smA, empty, fulla)) err = 1;
+  } else if (CONV == 1 && (int)threadIdx.x < R::GATHER) {
     // A gatherers: half threadIdx.x / 128 of row threadIdx.x % 128 of every stage tile
     const int row = threadIdx.x % TC_BM, half = threadIdx.x / TC_BM;
     const GatherRow g = gather_row(conv, m0 + row, a.M);
@@ -401,14 +516,23 @@ cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st) {
   if (!encode_bf16_sw128(&tb, g.B, g.K, g.N, g.ldb, BN)) return cudaErrorInvalidValue;
   if (conv) ta = tb;  // unused: A is gathered
   else if (!encode_bf16_sw128(&ta, g.A, g.K, g.M, g.lda, TC_BM)) return cudaErrorInvalidValue;
-  const int smem = TC_STAGES * (A_STAGE + BN * TC_BK * 2) + 1024 + (conv ? (int)nkb * TC_BK * 8 : 0);
+  // pixel pairs need an even row of outputs, 8 (16) byte aligned pairs of inputs, and
+  // whole K (no splits); with fewer than 8 channels most of a run would be padding
+  int kind = 0;
+  if (conv) {
+    const TcConvA& c = *g.conv;
+    kind = 1;
+    if (c.C >= 8 && splits == 1 && c.sw == 1 && c.W % 2 == 0 && (uintptr_t)c.x % 8 == 0) kind = 2;
+    if (c.C >= 8 && splits == 1 && c.sw == 2 && c.W % 4 == 0 && (uintptr_t)c.x % 16 == 0) kind = 3;
+  }
+  const int smem = TC_STAGES * (A_STAGE + BN * TC_BK * 2) + 1024 + (kind == 1 ? (int)nkb * TC_BK * 8 : 0);
   const dim3 grid((unsigned)((g.M + TC_BM - 1) / TC_BM), (unsigned)((g.N + BN - 1) / BN), (unsigned)splits);
   TcConvA c{};
   if (conv) c = *g.conv;
-  auto kern = conv ? k_tc_gemm<true> : k_tc_gemm<false>;
+  auto kern = kind == 0 ? k_tc_gemm<0> : kind == 1 ? k_tc_gemm<1> : kind == 2 ? k_tc_gemm<2> : k_tc_gemm<3>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  kern<<<grid, conv ? TcRoles<true>::THREADS : TcRoles<false>::THREADS, smem, st>>>(ta, tb, a, c);
+  kern<<<grid, conv ? TcRoles<1>::THREADS : TcRoles<0>::THREADS, smem, st>>>(ta, tb, a, c);
   return cudaGetLastError();
 }
 
