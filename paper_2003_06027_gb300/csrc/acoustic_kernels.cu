@@ -176,14 +176,6 @@ __device__ __forceinline__ void dminus_x(const float* c, const float v[12], floa
   }
 }
 
-// Programmatic dependent launch: a step's CTAs may be scheduled while the
-// previous step drains; they wait for its end before they touch memory, and only
-// then let the next step's CTAs in (so at most two steps are resident, and no
-// line that a step could have cached is older than the step before it). Both
-// are no-ops in a launch without the attribute.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
@@ -206,7 +198,6 @@ __device__ __forceinline__ void acc4(float4& acc, float c, const float4 p, const
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
-__device__ __forceinline__ void prefetch_l1(const float* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
@@ -1063,7 +1054,7 @@ __global__ void __launch_bounds__(NTHREADS, 3)
         const int r = 2 * ty + rr;
         if (!LAP && !pmlx) lc[rr] = ld4(sx + r * UW + H + 4 * tx);
         else if (!LAP && !pmlz) lc[rr] = ld4(sz + (r + H) * TILE_X + 4 * tx);
-        else lc[rr] = ldg4(p.lam + (long long)(p.cur * p.S_pair + p.s0) * g.slice + base + (long long)(z0 + r) * pitch + xb);
+        else lc[rr] = ld4(p.lam + (long long)(p.cur * p.S_pair + p.s0) * g.slice + base + (long long)(z0 + r) * pitch + xb);
         if (LAP) {
           const float4 mh = ld4(sm + (r + 4) * MW + 4 * tx + 4);
           m2[rr] = make_float4(2.f * mh.x, 2.f * mh.y, 2.f * mh.z, 2.f * mh.w);
@@ -1074,10 +1065,10 @@ __global__ void __launch_bounds__(NTHREADS, 3)
       float* __restrict__ lprev = p.lam + (long long)((p.cur ^ 1) * p.S_pair + p.s0) * g.slice + base;
       float* __restrict__ gp = p.gpart + base;
       float4 lo[2], go[2];
-      lo[0] = ldg4(lprev + (long long)zr0 * pitch + xb);
-      lo[1] = ldg4(lprev + (long long)(zr0 + 1) * pitch + xb);
-      go[0] = ldg4(gp + (long long)zr0 * pitch + xb);
-      go[1] = ldg4(gp + (long long)(zr0 + 1) * pitch + xb);
+      lo[0] = ld4(lprev + (long long)zr0 * pitch + xb);
+      lo[1] = ld4(lprev + (long long)(zr0 + 1) * pitch + xb);
+      go[0] = ld4(gp + (long long)zr0 * pitch + xb);
+      go[1] = ld4(gp + (long long)(zr0 + 1) * pitch + xb);
       __syncthreads();
       if (tid == 0 && tn < ntiles) fetch(tn);  // the operand buffer is free
 
@@ -1348,23 +1339,6 @@ AcuCoef coef_of(const AcuStep& p) {
   return c;
 }
 
-// One step launch; its CTAs may be scheduled while the launch before it on the
-// stream drains (pdl_wait).
-template <typename... P, typename... A>
-cudaError_t launch_step(void (*kern)(P...), int grid, int threads, size_t smem, cudaStream_t st, const A&... args) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 }  // namespace
 
 // The z weights of a step as packed pairs.
@@ -1424,7 +1398,7 @@ cudaError_t launch_acu_fwd(const AcuStep& p_in, const AcuMaps& maps, bool record
   const int grid = std::min(p.ntiles, g_grid_fwd[dev][sp][lap ? 1 : 0][o][v]);
   auto k = p.N == 2 ? (lap ? fwd_kernel<2, true>(sp, v) : fwd_kernel<2, false>(sp, v))
                     : (lap ? fwd_kernel<4, true>(sp, v) : fwd_kernel<4, false>(sp, v));
-  return launch_step(k, grid, fwd_threads(sp), fwd_smem(sp), st, maps.u[sp], maps.m[sp], p, cf, nb);
+  return launch_step(k, p.ntiles, grid, fwd_threads(sp), fwd_smem(sp), st, maps.u[sp], maps.m[sp], p, cf, nb);
 }
 
 // Multi-instance forward step b.n over the tiles of instances [0, b.n_active):
@@ -1443,7 +1417,7 @@ cudaError_t launch_acu_fwd_batch(const BatchArgs& b, const AcuCoef& cf, int N, b
   memset(&p0, 0, sizeof p0);
   auto k = N == 2 ? (record ? acu_fwd_step<2, true, true, true, 2, 16> : acu_fwd_step<2, false, true, true, 2, 16>)
                   : (record ? acu_fwd_step<4, true, true, true, 2, 16> : acu_fwd_step<4, false, true, true, 2, 16>);
-  return launch_step(k, grid, 256, FWD_SMEM_M, st, none, none, p0, cf, b);
+  return launch_step(k, b.ntiles, grid, 256, FWD_SMEM_M, st, none, none, p0, cf, b);
 }
 
 // Adjoint operand maps: lambda and the hhat pairs Hx, Hz, each [2][S][slice],
@@ -1472,15 +1446,15 @@ cudaError_t launch_acu_adj(const AcuStep& p, const AcuMaps& maps, cudaStream_t s
   memset(&nb, 0, sizeof nb);
   if (lap) {
     if (p.N == 2)
-      return launch_step(acu_adj_step<2, false, true>, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
+      return launch_step(acu_adj_step<2, false, true>, p.ntiles, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
     else
-      return launch_step(acu_adj_step<4, false, true>, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
+      return launch_step(acu_adj_step<4, false, true>, p.ntiles, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
     return cudaGetLastError();
   }
   if (p.N == 2)
-    return launch_step(acu_adj_step<2, false>, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
+    return launch_step(acu_adj_step<2, false>, p.ntiles, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
   else
-    return launch_step(acu_adj_step<4, false>, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
+    return launch_step(acu_adj_step<4, false>, p.ntiles, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
   return cudaGetLastError();
 }
 
@@ -1495,8 +1469,8 @@ cudaError_t launch_acu_adj_batch(const BatchArgs& b, const AcuCoef& cf, int N, c
   memset(&none, 0, sizeof none);
   AcuStep p0;
   memset(&p0, 0, sizeof p0);
-  if (N == 2) return launch_step(acu_adj_step<2, true>, grid, NTHREADS, ADJ_SMEM_M, st, none, none, none, none, none, p0, cf, b);
-  else return launch_step(acu_adj_step<4, true>, grid, NTHREADS, ADJ_SMEM_M, st, none, none, none, none, none, p0, cf, b);
+  if (N == 2) return launch_step(acu_adj_step<2, true>, b.ntiles, grid, NTHREADS, ADJ_SMEM_M, st, none, none, none, none, none, p0, cf, b);
+  else return launch_step(acu_adj_step<4, true>, b.ntiles, grid, NTHREADS, ADJ_SMEM_M, st, none, none, none, none, none, p0, cf, b);
   return cudaGetLastError();
 }
 

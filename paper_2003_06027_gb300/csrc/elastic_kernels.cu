@@ -106,6 +106,9 @@ __device__ __forceinline__ bool pml_z(const Grid& g, int z0) {
   return g.npml > 0 && (z0 - 8 < g.npml || z0 + TILE_Z + 8 > g.npml + g.nz - 1);
 }
 
+// Points in the reach of a CPML layer (integer or half).
+__device__ __forceinline__ bool in_layer(int a, int b, int npml, int n) { return a < npml || b >= npml + n - 1; }
+
 // Node-local CPML update of 4 consecutive x nodes with x-dependent tables:
 // psi <- b psi + a d (zero where a = 0), returns d + psi.
 __device__ __forceinline__ void cpml_x4(bool on, const float* ta, const float* tb, int j, float* psi, long long id,
@@ -145,7 +148,7 @@ __device__ __forceinline__ void cpml_adj_x4(bool on, const float* ta, const floa
   if (!any4(a4)) return;
   const float4 b4 = ldg4(tb + j + TAB_OFF);
   float M[4], a[4], b[4];
-  f4a(ldg4(Min + id), M);  // read-only in this kernel (the pair's other half is written)
+  f4a(ld4(Min + id), M);
   f4a(a4, a);
   f4a(b4, b);
   float Mn[4];
@@ -165,7 +168,7 @@ __device__ __forceinline__ void cpml_adj_z4(bool on, const float* ta, const floa
   if (a == 0.f) return;
   const float b = __ldg(tb + z + TAB_OFF);
   float M[4], Mn[4];
-  f4a(ldg4(Min + id), M);  // read-only in this kernel (the pair's other half is written)
+  f4a(ld4(Min + id), M);
 #pragma unroll
   for (int e = 0; e < 4; e++) {
     const float u = M[e] + t[e];
@@ -173,6 +176,34 @@ __device__ __forceinline__ void cpml_adj_z4(bool on, const float* ta, const floa
     Mn[e] = b * u;
   }
   if (own) st4(Mout + id, a4f(Mn));
+}
+
+// The same for an adjoint tile: its own nodes' groups are the items k = tid, tid +
+// NTHREADS of a 32 x 16 walk, and the halo items belong to the threads as below.
+__device__ __forceinline__ void adj_prefetch(const EleStep& p, const Grid& g, int x0, int z0, long long base, int mx0,
+                                             int mx1, int mz0, int mz1, int tid) {
+  const bool px = pml_x(g, x0), pz = pml_z(g, z0);
+  if (!px && !pz) return;
+  auto one = [&](int z, int j, bool x, bool zz) {
+    const long long id = base + (long long)z * g.pitch + j;
+    if (x && px && in_layer(j, j + 3, g.npml, g.nx)) {
+      prefetch_l1(p.Min[mx0] + id);
+      prefetch_l1(p.Min[mx1] + id);
+    }
+    if (zz && pz && in_layer(z, z, g.npml, g.nz)) {
+      prefetch_l1(p.Min[mz0] + id);
+      prefetch_l1(p.Min[mz1] + id);
+    }
+  };
+  const int c = tid & 15, r = tid >> 4;
+  one(z0 + r, x0 + 4 * c, true, true);
+  one(z0 + r + 16, x0 + 4 * c, true, true);
+  if (tid < 2 * TILE_Z) {
+    one(z0 + (tid >> 1), x0 - 4 + ((tid & 1) ? TILE_X + 4 : 0), true, false);
+  } else if (tid < 2 * TILE_Z + 8 * (TILE_X / 4)) {
+    const int h = (tid - 2 * TILE_Z) >> 4, hr = h < 4 ? h : h + TILE_Z;
+    one(z0 - 4 + hr, x0 + 4 * c, false, true);
+  }
 }
 
 // Deterministic CTA sum of three floats (fixed shuffle tree, fixed warp order).
@@ -205,6 +236,8 @@ __device__ __forceinline__ void cta_sum3(float v[3], float* red) {
     fence_mbar_init();                                                           \
   }                                                                              \
   __syncthreads();                                                               \
+  pdl_wait();                                                                    \
+  pdl_next();                                                                    \
   if (tid == 0 && (int)blockIdx.x < ntiles) FETCH(blockIdx.x, 0);                \
   int it = 0;                                                                    \
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {                   \
@@ -242,6 +275,8 @@ __device__ __forceinline__ void cta_sum3(float v[3], float* red) {
     fence_mbar_init();                                              \
   }                                                                 \
   __syncthreads();                                                  \
+  pdl_wait();                                                       \
+  pdl_next();                                                       \
   if (tid == 0 && (int)blockIdx.x < ntiles) FETCH(blockIdx.x);      \
   int it = 0;                                                       \
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {      \
@@ -282,9 +317,9 @@ __global__ void __launch_bounds__(NTHREADS, N == 2 ? 3 : 2)  // 3 CTAs per SM at
     float* d = smem_e + bb * VEL_BUF;
     fence_proxy_async();
     mbar_expect_tx(&bar[bb], VEL_BUF * 4);
-    tma_3d(d, &m_xx, f.x0 - 4 + APRON, f.z0 + APRON, f.s, &bar[bb]);
-    tma_3d(d + TILE_Z * W72, &m_zz, f.x0 + APRON, f.z0 - 4 + APRON, f.s, &bar[bb]);
-    tma_3d(d + TILE_Z * W72 + H40 * TILE_X, &m_xz, f.x0 - 4 + APRON, f.z0 - 4 + APRON, f.s, &bar[bb]);
+    tma_3d(d, &m_xx, f.x0 - 4 + APRON, f.z0 + APRON, p.s0 + f.s, &bar[bb]);
+    tma_3d(d + TILE_Z * W72, &m_zz, f.x0 + APRON, f.z0 - 4 + APRON, p.s0 + f.s, &bar[bb]);
+    tma_3d(d + TILE_Z * W72 + H40 * TILE_X, &m_xz, f.x0 - 4 + APRON, f.z0 - 4 + APRON, p.s0 + f.s, &bar[bb]);
   };
   ELA_WALK_BEGIN(fetch)
   const int xb = x0 + 4 * tx, zr0 = z0 + 2 * ty;
@@ -391,8 +426,8 @@ __global__ void __launch_bounds__(NTHREADS, N == 2 ? 3 : 2)  // 3 CTAs per SM at
     float* d = smem_e + bb * STR_BUF;
     fence_proxy_async();
     mbar_expect_tx(&bar[bb], STR_BUF * 4);
-    tma_3d(d, &m_vx, f.x0 - 4 + APRON, f.z0 - 4 + APRON, f.s, &bar[bb]);
-    tma_3d(d + H40 * W72, &m_vz, f.x0 - 4 + APRON, f.z0 - 4 + APRON, f.s, &bar[bb]);
+    tma_3d(d, &m_vx, f.x0 - 4 + APRON, f.z0 - 4 + APRON, p.s0 + f.s, &bar[bb]);
+    tma_3d(d + H40 * W72, &m_vz, f.x0 - 4 + APRON, f.z0 - 4 + APRON, p.s0 + f.s, &bar[bb]);
   };
   ELA_WALK_BEGIN(fetch)
   const int xb = x0 + 4 * tx, zr0 = z0 + 2 * ty;
@@ -510,9 +545,9 @@ __global__ void __launch_bounds__(NTHREADS, N == 2 ? 3 : 2)  // 3 CTAs per SM at
     const TileId f = tile_decode(g, tt);
     fence_proxy_async();
     mbar_expect_tx(&bar[0], ADJA_BUF * 4);
-    tma_3d(smem_e, &m_Sxx, f.x0 - 4 + APRON, f.z0 - 4 + APRON, f.s, &bar[0]);
-    tma_3d(smem_e + H40 * W72, &m_Szz, f.x0 - 4 + APRON, f.z0 - 4 + APRON, f.s, &bar[0]);
-    tma_3d(smem_e + 2 * H40 * W72, &m_Sxz, f.x0 - 4 + APRON, f.z0 - 4 + APRON, f.s, &bar[0]);
+    tma_3d(smem_e, &m_Sxx, f.x0 - 4 + APRON, f.z0 - 4 + APRON, p.s0 + f.s, &bar[0]);
+    tma_3d(smem_e + H40 * W72, &m_Szz, f.x0 - 4 + APRON, f.z0 - 4 + APRON, p.s0 + f.s, &bar[0]);
+    tma_3d(smem_e + 2 * H40 * W72, &m_Sxz, f.x0 - 4 + APRON, f.z0 - 4 + APRON, p.s0 + f.s, &bar[0]);
   };
   ELA_WALK1_BEGIN(fetch)
   const int xb = x0 + 4 * tx, zr0 = z0 + 2 * ty;
@@ -525,6 +560,16 @@ __global__ void __launch_bounds__(NTHREADS, N == 2 ? 3 : 2)  // 3 CTAs per SM at
   }
   const int key = (id.tz * g.ntx + id.tx) * NTHREADS + tid;
   const int rb = __ldg(p.thr_rec_start + key), re = __ldg(p.thr_rec_start + key + 1);
+  adj_prefetch(p, g, x0, z0, base, 4, 7, 5, 6, tid);
+  // the stored strains of the own nodes (read after the stage barrier, from HBM)
+  if ((tx & 7) == 0)
+#pragma unroll
+    for (int rr = 0; rr < 2; rr++) {
+      const long long id = base + (long long)(zr0 + rr) * pitch + xb;
+      prefetch_l2(p.slot[2] + id);
+      prefetch_l2(p.slot[3] + id);
+      prefetch_l2(p.slot[4] + id);
+    }
   ELA_WAIT1()
   const float* s_Sxx = smem_e;
   const float* s_Szz = s_Sxx + H40 * W72;
@@ -772,8 +817,8 @@ __global__ void __launch_bounds__(NTHREADS, N == 2 ? 3 : 2)  // 3 CTAs per SM at
     const TileId f = tile_decode(g, tt);
     fence_proxy_async();
     mbar_expect_tx(&bar[0], ADJB_BUF * 4);
-    tma_3d(smem_e, &m_Vx, f.x0 - 4 + APRON, f.z0 - 4 + APRON, f.s, &bar[0]);
-    tma_3d(smem_e + H40 * W72, &m_Vz, f.x0 - 4 + APRON, f.z0 - 4 + APRON, f.s, &bar[0]);
+    tma_3d(smem_e, &m_Vx, f.x0 - 4 + APRON, f.z0 - 4 + APRON, p.s0 + f.s, &bar[0]);
+    tma_3d(smem_e + H40 * W72, &m_Vz, f.x0 - 4 + APRON, f.z0 - 4 + APRON, p.s0 + f.s, &bar[0]);
   };
   ELA_WALK1_BEGIN(fetch)
   const int xb = x0 + 4 * tx, zr0 = z0 + 2 * ty;
@@ -785,6 +830,14 @@ __global__ void __launch_bounds__(NTHREADS, N == 2 ? 3 : 2)  // 3 CTAs per SM at
     spre[rr][1] = ld4(p.Szz + id);
     spre[rr][2] = ld4(p.Sxz + id);
   }
+  adj_prefetch(p, g, x0, z0, base, 0, 2, 1, 3, tid);
+  if ((tx & 7) == 0)
+#pragma unroll
+    for (int rr = 0; rr < 2; rr++) {
+      const long long id = base + (long long)(zr0 + rr) * pitch + xb;
+      prefetch_l2(p.slot[0] + id);
+      prefetch_l2(p.slot[1] + id);
+    }
   ELA_WAIT1()
   const float* s_Vx = smem_e;
   const float* s_Vz = s_Vx + H40 * W72;
@@ -1244,17 +1297,17 @@ cudaError_t launch_ela_vel(const EleStep& p, const EleMaps& m, bool record, bool
   if (e != cudaSuccess) return e;
   const int grid = ela_grid(p, dev, record ? (store ? 7 : 1) : (store ? 2 : 0));
   if (p.N == 2) {
-    if (record && store) ela_vel_step<2, true, true><<<grid, NTHREADS, VEL_SMEM, st>>>(m.sxx, m.szz, m.sxz, p);
-    else if (record) ela_vel_step<2, true, false><<<grid, NTHREADS, VEL_SMEM, st>>>(m.sxx, m.szz, m.sxz, p);
-    else if (store) ela_vel_step<2, false, true><<<grid, NTHREADS, VEL_SMEM, st>>>(m.sxx, m.szz, m.sxz, p);
-    else ela_vel_step<2, false, false><<<grid, NTHREADS, VEL_SMEM, st>>>(m.sxx, m.szz, m.sxz, p);
+    if (record && store) e = launch_step(ela_vel_step<2, true, true>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, VEL_SMEM, st, m.sxx, m.szz, m.sxz, p);
+    else if (record) e = launch_step(ela_vel_step<2, true, false>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, VEL_SMEM, st, m.sxx, m.szz, m.sxz, p);
+    else if (store) e = launch_step(ela_vel_step<2, false, true>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, VEL_SMEM, st, m.sxx, m.szz, m.sxz, p);
+    else e = launch_step(ela_vel_step<2, false, false>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, VEL_SMEM, st, m.sxx, m.szz, m.sxz, p);
   } else {
-    if (record && store) ela_vel_step<4, true, true><<<grid, NTHREADS, VEL_SMEM, st>>>(m.sxx, m.szz, m.sxz, p);
-    else if (record) ela_vel_step<4, true, false><<<grid, NTHREADS, VEL_SMEM, st>>>(m.sxx, m.szz, m.sxz, p);
-    else if (store) ela_vel_step<4, false, true><<<grid, NTHREADS, VEL_SMEM, st>>>(m.sxx, m.szz, m.sxz, p);
-    else ela_vel_step<4, false, false><<<grid, NTHREADS, VEL_SMEM, st>>>(m.sxx, m.szz, m.sxz, p);
+    if (record && store) e = launch_step(ela_vel_step<4, true, true>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, VEL_SMEM, st, m.sxx, m.szz, m.sxz, p);
+    else if (record) e = launch_step(ela_vel_step<4, true, false>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, VEL_SMEM, st, m.sxx, m.szz, m.sxz, p);
+    else if (store) e = launch_step(ela_vel_step<4, false, true>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, VEL_SMEM, st, m.sxx, m.szz, m.sxz, p);
+    else e = launch_step(ela_vel_step<4, false, false>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, VEL_SMEM, st, m.sxx, m.szz, m.sxz, p);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_ela_str(const EleStep& p, const EleMaps& m, bool store, cudaStream_t st) {
@@ -1263,13 +1316,13 @@ cudaError_t launch_ela_str(const EleStep& p, const EleMaps& m, bool store, cudaS
   if (e != cudaSuccess) return e;
   const int grid = ela_grid(p, dev, store ? 4 : 3);
   if (p.N == 2) {
-    if (store) ela_str_step<2, true><<<grid, NTHREADS, STR_SMEM, st>>>(m.vx, m.vz, p);
-    else ela_str_step<2, false><<<grid, NTHREADS, STR_SMEM, st>>>(m.vx, m.vz, p);
+    if (store) e = launch_step(ela_str_step<2, true>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, STR_SMEM, st, m.vx, m.vz, p);
+    else e = launch_step(ela_str_step<2, false>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, STR_SMEM, st, m.vx, m.vz, p);
   } else {
-    if (store) ela_str_step<4, true><<<grid, NTHREADS, STR_SMEM, st>>>(m.vx, m.vz, p);
-    else ela_str_step<4, false><<<grid, NTHREADS, STR_SMEM, st>>>(m.vx, m.vz, p);
+    if (store) e = launch_step(ela_str_step<4, true>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, STR_SMEM, st, m.vx, m.vz, p);
+    else e = launch_step(ela_str_step<4, false>, (long long)p.S * p.g.ntx * p.g.ntz, grid, NTHREADS, STR_SMEM, st, m.vx, m.vz, p);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_ela_adj(const EleStep& p, const EleMaps& m, cudaStream_t st) {
@@ -1278,13 +1331,15 @@ cudaError_t launch_ela_adj(const EleStep& p, const EleMaps& m, cudaStream_t st) 
   if (e != cudaSuccess) return e;
   const int ga = ela_grid(p, dev, 5), gb = ela_grid(p, dev, 6);
   if (p.N == 2) {
-    ela_str_adj<2><<<ga, NTHREADS, ADJ_A_SMEM, st>>>(m.Sxx, m.Szz, m.Sxz, p);
-    ela_vel_adj<2><<<gb, NTHREADS, ADJ_B_SMEM, st>>>(m.Vx, m.Vz, p);
+    e = launch_step(ela_str_adj<2>, (long long)p.S * p.g.ntx * p.g.ntz, ga, NTHREADS, ADJ_A_SMEM, st, m.Sxx, m.Szz, m.Sxz, p);
+    if (e != cudaSuccess) return e;
+    e = launch_step(ela_vel_adj<2>, (long long)p.S * p.g.ntx * p.g.ntz, gb, NTHREADS, ADJ_B_SMEM, st, m.Vx, m.Vz, p);
   } else {
-    ela_str_adj<4><<<ga, NTHREADS, ADJ_A_SMEM, st>>>(m.Sxx, m.Szz, m.Sxz, p);
-    ela_vel_adj<4><<<gb, NTHREADS, ADJ_B_SMEM, st>>>(m.Vx, m.Vz, p);
+    e = launch_step(ela_str_adj<4>, (long long)p.S * p.g.ntx * p.g.ntz, ga, NTHREADS, ADJ_A_SMEM, st, m.Sxx, m.Szz, m.Sxz, p);
+    if (e != cudaSuccess) return e;
+    e = launch_step(ela_vel_adj<4>, (long long)p.S * p.g.ntx * p.g.ntz, gb, NTHREADS, ADJ_B_SMEM, st, m.Vx, m.Vz, p);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_ela_medium(const float* vp, const float* vs, const float* rho, const Grid& g, float* lam,

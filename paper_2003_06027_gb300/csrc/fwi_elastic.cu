@@ -303,6 +303,84 @@ fwi_status ela_prepare(fwi_ctx* ctx, EPlan& P, const fwi_model* M, const fwi_sou
   return FWI_OK;
 }
 
+// Shot groups: a step's shots as two launches on their own streams, forked from
+// and joined to the call's stream, so that one launch's last tiles and the gap to
+// the next are filled by the other (every elastic field is per shot). Per step
+// (forward / recompute / adjoint pair), one group against two, 300 x 800: 32 shots
+// 185/208/334 -> 161/184/321 us, 8 shots 48/55/92 -> 42/49/82, 4 shots 28/31/49 ->
+// 24/28/39; three or four groups give no more, and below one tile per resident CTA
+// (3 on each of 152 SMs) the launches only wait for each other: 4 shots of 200 x 400
+// (288 tiles) 18.5/20/27 -> 20/23/26.5.
+struct EGroups {
+  int G = 1;
+  int s0[2] = {0, 0}, n[2] = {0, 0};
+  cudaStream_t st[2] = {};
+};
+
+fwi_status ela_groups(fwi_ctx* ctx, const EPlan& P, cudaStream_t main, EGroups& gr) {
+  gr.G = P.S >= 2 && (long long)P.S * P.g.ntx * P.g.ntz > 3 * 152 ? 2 : 1;
+  for (int g = 0, s0 = 0; g < gr.G; g++) {
+    gr.n[g] = P.S / gr.G + (g < P.S % gr.G ? 1 : 0);
+    gr.s0[g] = s0;
+    s0 += gr.n[g];
+  }
+  gr.st[0] = main;
+  if (gr.G == 1) return FWI_OK;
+  for (int g = 0; g < gr.G; g++) {
+    if (!ctx->gstream[g]) ECK(cudaStreamCreateWithFlags(&ctx->gstream[g], cudaStreamNonBlocking));
+    if (!ctx->join_ev[g]) ECK(cudaEventCreateWithFlags(&ctx->join_ev[g], cudaEventDisableTiming));
+    gr.st[g] = ctx->gstream[g];
+  }
+  if (!ctx->fork_ev) ECK(cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming));
+  return FWI_OK;
+}
+fwi_status ela_fork(fwi_ctx* ctx, const EGroups& gr, cudaStream_t main) {
+  if (gr.G == 1) return FWI_OK;
+  ECK(cudaEventRecord(ctx->fork_ev, main));
+  for (int g = 0; g < gr.G; g++) ECK(cudaStreamWaitEvent(gr.st[g], ctx->fork_ev, 0));
+  return FWI_OK;
+}
+fwi_status ela_join(fwi_ctx* ctx, const EGroups& gr, cudaStream_t main) {
+  if (gr.G == 1) return FWI_OK;
+  for (int g = 0; g < gr.G; g++) {
+    ECK(cudaEventRecord(ctx->join_ev[g], gr.st[g]));
+    ECK(cudaStreamWaitEvent(main, ctx->join_ev[g], 0));
+  }
+  return FWI_OK;
+}
+
+// The step parameters of one group, shots [s0, s0 + Sg): per-shot arrays are
+// offset to its first shot, the tensor maps are indexed from it (p.s0).
+EleStep ela_group_view(const EleStep& p, const EPlan& P, int s0, int Sg) {
+  EleStep q = p;
+  const long long sl = P.g.slice, ns = 2LL * p.nrec * p.nt;
+  auto off = [&](auto*& ptr, long long per) {
+    if (ptr) ptr += s0 * per;
+  };
+  q.S = Sg;
+  q.s0 = s0;
+  for (float** f : {&q.vx, &q.vz, &q.sxx, &q.szz, &q.sxz, &q.Vx, &q.Vz, &q.Sxx, &q.Szz, &q.Sxz, &q.g_lam, &q.g_mu,
+                    &q.g_mxz, &q.g_bx, &q.g_bz})
+    off(*f, sl);
+  for (int k = 0; k < 8; k++) {
+    off(q.psi[k], sl);
+    off(q.Min[k], sl);
+    off(q.Mout[k], sl);
+  }
+  for (int k = 0; k < 5; k++) off(q.slot[k], sl);
+  off(q.box_n, 2);
+  off(q.box_s, 2);
+  off(q.w_n, SRC_W * SRC_W);
+  off(q.w_s, SRC_W * SRC_W);
+  off(q.stf, p.nt);
+  off(q.mt, 3);
+  off(q.x0, 2);
+  off(q.seis, ns);
+  off(q.res, ns);
+  off(q.src_part, (long long)p.nt * ELA_SLOTS * 3);
+  return q;
+}
+
 }  // namespace
 
 fwi_status ela_forward(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* Sv, const fwi_receivers* R, int32_t nt,
@@ -323,12 +401,19 @@ fwi_status ela_forward(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* Sv, 
   EleMaps maps;
   ECK(ela_make_maps(&maps, P.g, P.S, P.f, nullptr));
   ensure_events(ctx, 0);
+  EGroups gr;
+  if ((v = ela_groups(ctx, P, st, gr)) != FWI_OK) return v;
   ECK(cudaEventRecord(ctx->ev[0], st));
+  if ((v = ela_fork(ctx, gr, st)) != FWI_OK) return v;
   for (int n = 0; n < nt; n++) {
     p.n = n;
-    ELK(1, launch_ela_vel(p, maps, true, false, st));
-    ELK(1, launch_ela_str(p, maps, false, st));
+    for (int g = 0; g < gr.G; g++) {
+      const EleStep q = ela_group_view(p, P, gr.s0[g], gr.n[g]);
+      ELK(1, launch_ela_vel(q, maps, true, false, gr.st[g]));
+      ELK(1, launch_ela_str(q, maps, false, gr.st[g]));
+    }
   }
+  if ((v = ela_join(ctx, gr, st)) != FWI_OK) return v;
   ECK(cudaEventRecord(ctx->ev[1], st));
   const long long ns = (long long)P.S * 2 * P.nrec * nt;
   if (ns > 0) {
@@ -380,20 +465,30 @@ fwi_status ela_misfit_grad(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* 
   // strains itself (recording and storing in one launch), so that segment is
   // never recomputed
   const int nlast = (P.nseg - 1) * K;
+  const size_t sl = (size_t)P.g.slice;
+  EGroups gr;
+  if ((v = ela_groups(ctx, P, st, gr)) != FWI_OK) return v;
   ECK(cudaEventRecord(ctx->ev[0], st));
+  if ((v = ela_fork(ctx, gr, st)) != FWI_OK) return v;
   for (int n = 0; n < nt; n++) {
     if (n % K == 0 && n < nlast) {
       float* ck = P.ckpt + (size_t)(n / K) * NSTATE * field;
-      for (int f = 0; f < NSTATE; f++)
-        ECK(cudaMemcpyAsync(ck + f * field, P.f[f], field * 4, cudaMemcpyDeviceToDevice, st));
+      for (int g = 0; g < gr.G; g++)
+        for (int f = 0; f < NSTATE; f++)
+          ECK(cudaMemcpyAsync(ck + f * field + gr.s0[g] * sl, P.f[f] + gr.s0[g] * sl, gr.n[g] * sl * 4,
+                              cudaMemcpyDeviceToDevice, gr.st[g]));
     }
     p.n = n;
     const bool keep = n >= nlast;
     if (keep)
       for (int k = 0; k < 5; k++) p.slot[k] = P.slot + ((size_t)(n - nlast) * 5 + k) * field;
-    ELK(1, launch_ela_vel(p, maps, true, keep, st));
-    ELK(1, launch_ela_str(p, maps, keep, st));
+    for (int g = 0; g < gr.G; g++) {
+      const EleStep q = ela_group_view(p, P, gr.s0[g], gr.n[g]);
+      ELK(1, launch_ela_vel(q, maps, true, keep, gr.st[g]));
+      ELK(1, launch_ela_str(q, maps, keep, gr.st[g]));
+    }
   }
+  if ((v = ela_join(ctx, gr, st)) != FWI_OK) return v;
   ECK(cudaEventRecord(ctx->ev[1], st));
   if (ns > 0) ELK(2, launch_misfit(P.seis, P.res, ns, P.Jpart, MISFIT_BLOCKS, P.J, P.status, ctx->vjp, st));
   else ECK(cudaMemsetAsync(P.J, 0, 8, st));
@@ -416,16 +511,24 @@ fwi_status ela_misfit_grad(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* 
     ECK(cudaEventRecord(ctx->seg_ev[4 * seg + 0], st));
     if (seg < P.nseg - 1) {  // the last segment's slots are already filled by the forward sweep
       const float* ck = P.ckpt + (size_t)seg * NSTATE * field;
-      for (int f = 0; f < NSTATE; f++)
-        ECK(cudaMemcpyAsync(P.f[f], ck + f * field, field * 4, cudaMemcpyDeviceToDevice, st));
+      if ((v = ela_fork(ctx, gr, st)) != FWI_OK) return v;
+      for (int g = 0; g < gr.G; g++)
+        for (int f = 0; f < NSTATE; f++)
+          ECK(cudaMemcpyAsync(P.f[f] + gr.s0[g] * sl, ck + f * field + gr.s0[g] * sl, gr.n[g] * sl * 4,
+                              cudaMemcpyDeviceToDevice, gr.st[g]));
       for (int n = n0; n < n1; n++) {
         p.n = n;
         for (int k = 0; k < 5; k++) p.slot[k] = P.slot + ((size_t)(n - n0) * 5 + k) * field;
-        ELK(1, launch_ela_vel(p, maps, false, true, st));
-        ELK(1, launch_ela_str(p, maps, true, st));
+        for (int g = 0; g < gr.G; g++) {
+          const EleStep q = ela_group_view(p, P, gr.s0[g], gr.n[g]);
+          ELK(1, launch_ela_vel(q, maps, false, true, gr.st[g]));
+          ELK(1, launch_ela_str(q, maps, true, gr.st[g]));
+        }
       }
+      if ((v = ela_join(ctx, gr, st)) != FWI_OK) return v;
     }
     ECK(cudaEventRecord(ctx->seg_ev[4 * seg + 1], st));
+    if ((v = ela_fork(ctx, gr, st)) != FWI_OK) return v;
     for (int n = n1 - 1; n >= n0; n--) {
       p.n = n;
       for (int k = 0; k < 5; k++) p.slot[k] = P.slot + ((size_t)(n - n0) * 5 + k) * field;
@@ -434,8 +537,10 @@ fwi_status ela_misfit_grad(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* 
         p.Min[k] = P.M[in][k];
         p.Mout[k] = P.M[out][k];
       }
-      ELK(2, launch_ela_adj(p, maps, st));
+      for (int g = 0; g < gr.G; g++)
+        ELK(2, launch_ela_adj(ela_group_view(p, P, gr.s0[g], gr.n[g]), maps, gr.st[g]));
     }
+    if ((v = ela_join(ctx, gr, st)) != FWI_OK) return v;
     ECK(cudaEventRecord(ctx->seg_ev[4 * seg + 2], st));
     ELK(1, launch_ela_fold(P.gp, P.S, P.g.slice, P.G, st));
   }

@@ -51,7 +51,7 @@ __device__ __forceinline__ uint64_t l2_evict_first() {
 }
 __device__ __forceinline__ float4 ld4_stream(const float* ptr, uint64_t pol) {
   float4 v;
-  asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
       : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
       : "l"(ptr), "l"(pol));
   return v;
@@ -199,7 +199,8 @@ struct AcuCoef {
 constexpr int ELA_SLOTS = 8;  // source partial slots: 4 tiles x (normal box, shear box)
 struct EleStep {
   Grid g;
-  int S, N, n, nt, nrec;
+  int S, N, n, nt, nrec;  // S: shots of this launch (one shot group)
+  int s0;                 // its first shot in the tensor maps
   float cx[4], cz[4];     // a_k/dx, a_k/dz
   float dt;
   const float *bx, *bz, *lam, *lp2m, *mxz;   // [slice] medium on the nodes (zero outside)
