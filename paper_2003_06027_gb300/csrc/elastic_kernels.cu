@@ -1097,7 +1097,8 @@ __global__ void k_ela_src_prep(int S, int kind, const float* __restrict__ x0, Gr
   }
 }
 
-// vp, vs, rho finite with vp > 0, rho > 0, vs >= 0, lambda >= 0; CFL on vp.
+// vp, vs, rho finite with vp > 0, rho > 0, vs >= 0, lambda >= 0; CFL on vp. Each
+// block judges its own cells.
 __global__ void k_ela_model_check(const float* __restrict__ vp, const float* __restrict__ vs,
                                   const float* __restrict__ rho, long long n, float coef, int* status) {
   __shared__ float smax[32];
@@ -1106,7 +1107,7 @@ __global__ void k_ela_model_check(const float* __restrict__ vp, const float* __r
   __syncthreads();
   float mx = 0.f;
   int bad = 0;
-  for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const float a = vp[i], b = vs[i], r = rho[i];
     if (!(a > 0.f) || !isfinite(a) || !(b >= 0.f) || !isfinite(b) || !(r > 0.f) || !isfinite(r) ||
         a * a < 2.f * b * b)
@@ -1130,18 +1131,38 @@ __global__ void k_ela_model_check(const float* __restrict__ vp, const float* __r
 struct Parts5 {
   float* f[5];
 };
-__global__ void k_ela_fold(Parts5 parts, int S, long long slice, double* G) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < slice;
-       i += (long long)gridDim.x * blockDim.x) {
-    for (int f = 0; f < 5; f++) {
-      float* pp = parts.f[f];
-      double acc = 0.0;
-      for (int s = 0; s < S; s++) {
-        acc += (double)pp[(long long)s * slice + i];
-        pp[(long long)s * slice + i] = 0.f;
-      }
-      G[(long long)f * slice + i] += acc;
+// A thread takes 4 consecutive cells of one field (the slice is a multiple of 4
+// floats) and has the partials of 8 shots in flight before it adds them, in shot
+// order.
+__global__ void k_ela_fold(Parts5 parts, int S, long long slice, double* __restrict__ G) {
+  const long long n4 = slice / 4;
+  float4* __restrict__ p4 = reinterpret_cast<float4*>(parts.f[blockIdx.y]);
+  double2* __restrict__ G2 = reinterpret_cast<double2*>(G + blockIdx.y * slice);
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x) {
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    for (int s0 = 0; s0 < S; s0 += 8) {
+      const int m = min(8, S - s0);
+      float4 v[8];
+#pragma unroll
+      for (int u = 0; u < 8; u++)
+        if (u < m) v[u] = p4[(long long)(s0 + u) * n4 + i];
+#pragma unroll
+      for (int u = 0; u < 8; u++)
+        if (u < m) {
+          a0 += (double)v[u].x;
+          a1 += (double)v[u].y;
+          a2 += (double)v[u].z;
+          a3 += (double)v[u].w;
+          p4[(long long)(s0 + u) * n4 + i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
     }
+    double2 g0 = G2[2 * i], g1 = G2[2 * i + 1];
+    g0.x += a0;
+    g0.y += a1;
+    g1.x += a2;
+    g1.y += a3;
+    G2[2 * i] = g0;
+    G2[2 * i + 1] = g1;
   }
 }
 
@@ -1150,46 +1171,68 @@ __global__ void k_ela_fold(Parts5 parts, int S, long long slice, double* G) {
 // rho collects the buoyancy correlations (d b / d rho = -b^2 / 2 for each of
 // the two cells averaged), and a physical cell collects the CPML cells that
 // replicate it. G = [lam, mu, mxz, bx, bz] FP64 partials on the padded nodes.
-__global__ void k_ela_grad(const double* __restrict__ G, Grid g, const float* __restrict__ mxz,
-                           const float* __restrict__ mu_pad, const float* __restrict__ bx,
-                           const float* __restrict__ bz, float* out) {
+// A boundary cell collects up to (npml + 1)^2 padded cells: a warp takes it
+// (blocks from `inner` on); the other cells take one thread each.
+__global__ void __launch_bounds__(256) k_ela_grad(const double* __restrict__ G, Grid g, const float* __restrict__ mxz,
+                                                  const float* __restrict__ mu_pad, const float* __restrict__ bx,
+                                                  const float* __restrict__ bz, float* out, int inner) {
   const long long n = (long long)g.nz * g.nx;
   const long long sl = g.slice;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int iz = (int)(idx / g.nx), ix = (int)(idx - (long long)iz * g.nx);
-    const int i_lo = iz == 0 ? 0 : iz + g.npml, i_hi = iz == g.nz - 1 ? g.Nz - 1 : iz + g.npml;
-    const int j_lo = ix == 0 ? 0 : ix + g.npml, j_hi = ix == g.nx - 1 ? g.Nx - 1 : ix + g.npml;
-    double gl = 0.0, gm = 0.0, gr = 0.0;
-    for (int i = i_lo; i <= i_hi; i++)
-      for (int j = j_lo; j <= j_hi; j++) {
-        const long long c = g.off0 + (long long)i * g.pitch + j;
-        gl += G[c];
-        gm += G[sl + c];
-        const double mu = mu_pad[c];
-        for (int di = -1; di <= 0; di++)
-          for (int dj = -1; dj <= 0; dj++) {
-            const int si = i + di, sj = j + dj;
-            if (si < 0 || sj < 0 || si >= g.Nz - 1 || sj >= g.Nx - 1) continue;
-            const long long sc = g.off0 + (long long)si * g.pitch + sj;
-            const double m = mxz[sc];
-            if (m != 0.0) gm += G[2 * sl + sc] * m * m / (4.0 * mu * mu);
-          }
-        for (int dj = -1; dj <= 0; dj++) {
-          const int sj = j + dj;
-          if (sj < 0 || sj >= g.Nx - 1) continue;
-          const long long sc = g.off0 + (long long)i * g.pitch + sj;
-          const double b = bx[sc];
-          gr += -0.5 * b * b * G[3 * sl + sc];
-        }
-        for (int di = -1; di <= 0; di++) {
-          const int si = i + di;
-          if (si < 0 || si >= g.Nz - 1) continue;
-          const long long sc = g.off0 + (long long)si * g.pitch + j;
-          const double b = bz[sc];
-          gr += -0.5 * b * b * G[4 * sl + sc];
-        }
+  // the derivatives with respect to lambda, mu, rho of one padded cell
+  auto cell = [&](int i, int j, double& gl, double& gm, double& gr) {
+    const long long c = g.off0 + (long long)i * g.pitch + j;
+    gl += G[c];
+    gm += G[sl + c];
+    const double mu = mu_pad[c];
+    for (int di = -1; di <= 0; di++)
+      for (int dj = -1; dj <= 0; dj++) {
+        const int si = i + di, sj = j + dj;
+        if (si < 0 || sj < 0 || si >= g.Nz - 1 || sj >= g.Nx - 1) continue;
+        const long long sc = g.off0 + (long long)si * g.pitch + sj;
+        const double m = mxz[sc];
+        if (m != 0.0) gm += G[2 * sl + sc] * m * m / (4.0 * mu * mu);
       }
+    for (int dj = -1; dj <= 0; dj++) {
+      const int sj = j + dj;
+      if (sj < 0 || sj >= g.Nx - 1) continue;
+      const long long sc = g.off0 + (long long)i * g.pitch + sj;
+      const double b = bx[sc];
+      gr += -0.5 * b * b * G[3 * sl + sc];
+    }
+    for (int di = -1; di <= 0; di++) {
+      const int si = i + di;
+      if (si < 0 || si >= g.Nz - 1) continue;
+      const long long sc = g.off0 + (long long)si * g.pitch + j;
+      const double b = bz[sc];
+      gr += -0.5 * b * b * G[4 * sl + sc];
+    }
+  };
+  if ((int)blockIdx.x < inner) {
+    for (long long idx = blockIdx.x * 256LL + threadIdx.x; idx < n; idx += (long long)inner * 256) {
+      const int iz = (int)(idx / g.nx), ix = (int)(idx - (long long)iz * g.nx);
+      if (is_boundary(g, iz, ix)) continue;
+      double gl = 0.0, gm = 0.0, gr = 0.0;
+      cell(iz + g.npml, ix + g.npml, gl, gm, gr);
+      out[idx] = (float)gl;
+      out[n + idx] = (float)gm;
+      out[2 * n + idx] = (float)gr;
+    }
+    return;
+  }
+  const long long q = (blockIdx.x - inner) * 8LL + (threadIdx.x >> 5);
+  if (q >= n_boundary(g)) return;
+  int iz, ix;
+  boundary_cell(g, q, &iz, &ix);
+  const int i_lo = iz == 0 ? 0 : iz + g.npml, i_hi = iz == g.nz - 1 ? g.Nz - 1 : iz + g.npml;
+  const int j_lo = ix == 0 ? 0 : ix + g.npml, j_hi = ix == g.nx - 1 ? g.Nx - 1 : ix + g.npml;
+  const int w = j_hi - j_lo + 1, cells = (i_hi - i_lo + 1) * w;
+  double gl = 0.0, gm = 0.0, gr = 0.0;
+  for (int k = threadIdx.x & 31; k < cells; k += 32) cell(i_lo + k / w, j_lo + k % w, gl, gm, gr);
+  gl = warp_sum(gl);
+  gm = warp_sum(gm);
+  gr = warp_sum(gr);
+  const long long idx = (long long)iz * g.nx + ix;
+  if ((threadIdx.x & 31) == 0) {
     out[idx] = (float)gl;
     out[n + idx] = (float)gm;
     out[2 * n + idx] = (float)gr;
@@ -1354,13 +1397,14 @@ cudaError_t launch_ela_src_prep(int S, int kind, const float* x0, const Grid& g,
 }
 cudaError_t launch_ela_model_check(const float* vp, const float* vs, const float* rho, long long n, float coef,
                                    int* status, cudaStream_t st) {
-  k_ela_model_check<<<1, 1024, 0, st>>>(vp, vs, rho, n, coef, status);
+  k_ela_model_check<<<(unsigned)std::max<long long>(1, std::min<long long>((n + 1023) / 1024, 304)), 1024, 0, st>>>(
+      vp, vs, rho, n, coef, status);
   return cudaGetLastError();
 }
 cudaError_t launch_ela_fold(float* const* parts, int S, long long slice, double* G, cudaStream_t st) {
   Parts5 p5;
   for (int f = 0; f < 5; f++) p5.f[f] = parts[f];
-  k_ela_fold<<<608, 256, 0, st>>>(p5, S, slice, G);
+  k_ela_fold<<<dim3(304, 5), 256, 0, st>>>(p5, S, slice, G);
   return cudaGetLastError();
 }
 cudaError_t launch_ela_velocity_grad(const float* vp, const float* vs, const float* rho, const float* gin,
@@ -1372,7 +1416,8 @@ cudaError_t launch_ela_velocity_grad(const float* vp, const float* vs, const flo
 }
 cudaError_t launch_ela_grad(const double* G, const Grid& g, const float* mxz, const float* mu_pad, const float* bx,
                             const float* bz, float* out, cudaStream_t st) {
-  k_ela_grad<<<304, 256, 0, st>>>(G, g, mxz, mu_pad, bx, bz, out);
+  const int inner = 304;
+  k_ela_grad<<<(unsigned)(inner + (n_boundary(g) + 7) / 8), 256, 0, st>>>(G, g, mxz, mu_pad, bx, bz, out, inner);
   return cudaGetLastError();
 }
 

@@ -40,6 +40,32 @@ struct Grid {
   long long off0;     // offset of padded cell (0,0)
 };
 
+// The physical grid's boundary cells in a fixed order: first and last row, then the
+// first and last column of the rows between (every cell, if a side has one).
+__host__ __device__ inline long long n_boundary(const Grid& g) {
+  return g.nz == 1 || g.nx == 1 ? (long long)g.nz * g.nx : 2LL * g.nx + 2LL * (g.nz - 2);
+}
+__device__ __forceinline__ void boundary_cell(const Grid& g, long long q, int* iz, int* ix) {
+  if (g.nz == 1 || g.nx == 1) {
+    *iz = (int)(q / g.nx);
+    *ix = (int)(q % g.nx);
+  } else if (q < 2LL * g.nx) {
+    *iz = q < g.nx ? 0 : g.nz - 1;
+    *ix = (int)(q < g.nx ? q : q - g.nx);
+  } else {
+    const long long r = q - 2LL * g.nx;
+    *iz = 1 + (int)(r >> 1);
+    *ix = (r & 1) ? g.nx - 1 : 0;
+  }
+}
+__device__ __forceinline__ bool is_boundary(const Grid& g, int iz, int ix) {
+  return iz == 0 || iz == g.nz - 1 || ix == 0 || ix == g.nx - 1;
+}
+__device__ __forceinline__ double warp_sum(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // L2 policy for data that is streamed once per sweep (the segment slots: written
 // by the recompute step, read back once by the adjoint step): such lines are
 // evicted first, so they do not push the step's resident fields (wavefield

@@ -8,6 +8,7 @@
 // folds of the gradient of Eq. adjoint-gradient over time segments and shots.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "fwi_internal.cuh"
@@ -154,8 +155,27 @@ __global__ void k_rec_csr(int nrec, const int* __restrict__ iz, const int* __res
   for (int k = lo; k < hi; k++) acc += start[k];
   ssum[threadIdx.x] = acc;
   __syncthreads();
-  if (threadIdx.x == 0)
-    for (int t = 1; t < (int)blockDim.x; t++) ssum[t] += ssum[t - 1];
+  {  // inclusive scan of the 1024 chunk sums: within warps, then over the warp totals
+    __shared__ int wsum[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int v = acc;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += u;
+    }
+    if (lane == 31) wsum[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+      int w = wsum[lane];
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, w, o);
+        if (lane >= o) w += u;
+      }
+      wsum[lane] = w;
+    }
+    __syncthreads();
+    ssum[threadIdx.x] = v + (warp > 0 ? wsum[warp - 1] : 0);
+  }
   __syncthreads();
   int run = threadIdx.x == 0 ? 0 : ssum[threadIdx.x - 1];
   for (int k = lo; k < hi; k++) {
@@ -185,7 +205,9 @@ __global__ void k_rec_csr(int nrec, const int* __restrict__ iz, const int* __res
   }
 }
 
-// CFL: c_max dt sqrt(1/dx^2 + 1/dz^2) sum|a_k| <= 1, and c finite and > 0.
+// CFL: c_max dt sqrt(1/dx^2 + 1/dz^2) sum|a_k| <= 1, and c finite and > 0. Each
+// block judges its own cells (a bad model is reported before a CFL violation,
+// whichever blocks see them).
 __global__ void k_model_check(const float* __restrict__ c, long long n, float coef, int* status) {
   __shared__ float smax[1024 / 32];
   __shared__ int sbad;
@@ -193,7 +215,7 @@ __global__ void k_model_check(const float* __restrict__ c, long long n, float co
   __syncthreads();
   float mx = 0.f;
   int bad = 0;
-  for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const float v = c[i];
     if (!(v > 0.f) || !isfinite(v)) bad = 1;
     else mx = fmaxf(mx, v);
@@ -266,9 +288,18 @@ __global__ void k_superpose(const float* __restrict__ seis, int S, long long n, 
 }
 
 __global__ void k_misfit_final(const double* part, int nb, double scale, double* J, int* status) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  // the partials come in together and are added in block order by one thread
+  __shared__ double sp[512];
   double s = 0.0;
-  for (int b = 0; b < nb; b++) s += part[b];
+  for (int b0 = 0; b0 < nb; b0 += 512) {
+    const int m = min(512, nb - b0);
+    for (int b = threadIdx.x; b < m; b += blockDim.x) sp[b] = part[b0 + b];
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int b = 0; b < m; b++) s += sp[b];
+    __syncthreads();
+  }
+  if (threadIdx.x != 0) return;
   s *= scale;
   *J = s;
   if (!isfinite(s)) atomicOr(status, ST_NONFINITE);
@@ -286,21 +317,39 @@ __global__ void k_finite_check(const float* __restrict__ a, long long n, int* st
 // receivers (in receiver order), and its source-parameter partial (index nt-1).
 __global__ void k_adj_init(AcuStep p, float* lam, float* hx, float* hz, bool lap) {
   const int s = blockIdx.x;
-  if (threadIdx.x != 0) return;
   const long long sh = (long long)s * p.g.slice + p.g.off0;
-  for (int r = 0; r < p.nrec; r++) {
-    const int ri = p.rec_cell[2 * r], rj = p.rec_cell[2 * r + 1];
-    if (ri < 0) continue;
+  // a block per shot; the lists keep a cell pair's receivers together in receiver
+  // order, so the thread that takes a list entry with no earlier entry of its cell
+  // adds up that cell's receivers in that order
+  const int nlist = p.thr_rec_start[p.g.ntx * p.g.ntz * NTHREADS];
+  for (int q = threadIdx.x; q < nlist; q += blockDim.x) {
+    const int r0 = p.thr_rec[q] >> 3;
+    const int ri = p.rec_cell[2 * r0], rj = p.rec_cell[2 * r0 + 1];
+    const int key = ((ri / TILE_Z) * p.g.ntx + rj / TILE_X) * NTHREADS + ((ri % TILE_Z) >> 1) * 16 + ((rj % TILE_X) >> 2);
+    const int b = p.thr_rec_start[key], e = p.thr_rec_start[key + 1], cell = p.thr_rec[q] & 7;
+    bool first = true;
+    for (int k = b; k < q; k++) first = first && (p.thr_rec[k] & 7) != cell;
+    if (!first) continue;
     const long long c = sh + (long long)ri * p.g.pitch + rj;
-    const float rv = p.res[((long long)s * p.nrec + r) * p.nt + p.nt - 1];
     // hhat = lambda at a receiver (never inside the CPML layer); m lambda for the
     // Laplacian operator (m = 2 (m/2) at the cell)
-    const float hv = lap ? 2.f * p.mh[p.g.off0 + (long long)ri * p.g.pitch + rj] * rv : rv;
-    lam[c] += rv;
-    hx[c] += hv;
-    hz[c] += hv;
+    const float m2 = lap ? 2.f * p.mh[p.g.off0 + (long long)ri * p.g.pitch + rj] : 0.f;
+    float l = lam[c], x = hx[c], z = hz[c];
+    for (int k = q; k < e; k++) {
+      if ((p.thr_rec[k] & 7) != cell) continue;
+      const float rv = p.res[((long long)s * p.nrec + (p.thr_rec[k] >> 3)) * p.nt + p.nt - 1];
+      const float hv = lap ? m2 * rv : rv;
+      l += rv;
+      x += hv;
+      z += hv;
+    }
+    lam[c] = l;
+    hx[c] = x;
+    hz[c] = z;
   }
   if (p.src_part == nullptr) return;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   const int i0 = p.src_box[2 * s], j0 = p.src_box[2 * s + 1], nb = p.src_n;
   float acc[3] = {0.f, 0.f, 0.f};
   if (i0 >= 0) {
@@ -362,21 +411,33 @@ __global__ void k_fold(float* __restrict__ gpart, int S, long long slice, double
 // half-point correlation to both neighbours without the factor 1/2) and a
 // physical cell also collects the CPML cells that replicate it (transpose of
 // the edge padding).
-__global__ void k_grad_c(const double* __restrict__ G, Grid g, const float* __restrict__ c,
-                         float* grad) {
-  const long long n = (long long)g.nz * g.nx;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int iz = (int)(idx / g.nx), ix = (int)(idx - (long long)iz * g.nx);
-    const int i_lo = iz == 0 ? 0 : iz + g.npml;
-    const int i_hi = iz == g.nz - 1 ? g.Nz - 1 : iz + g.npml;
-    const int j_lo = ix == 0 ? 0 : ix + g.npml;
-    const int j_hi = ix == g.nx - 1 ? g.Nx - 1 : ix + g.npml;
-    double acc = 0.0;
-    for (int i = i_lo; i <= i_hi; i++)
-      for (int j = j_lo; j <= j_hi; j++) acc += G[g.off0 + (long long)i * g.pitch + j];
-    grad[idx] = (float)((double)c[idx] * acc);
+// A boundary cell collects up to (npml + 1)^2 padded cells: a warp takes it
+// (blocks from `inner` on), so that its loads are in flight together; the other
+// cells take one thread each.
+__global__ void __launch_bounds__(256) k_grad_c(const double* __restrict__ G, Grid g, const float* __restrict__ c,
+                                                float* grad, int inner) {
+  if ((int)blockIdx.x < inner) {
+    const long long n = (long long)g.nz * g.nx;
+    for (long long idx = blockIdx.x * 256LL + threadIdx.x; idx < n; idx += (long long)inner * 256) {
+      const int iz = (int)(idx / g.nx), ix = (int)(idx - (long long)iz * g.nx);
+      if (!is_boundary(g, iz, ix))
+        grad[idx] = (float)((double)c[idx] * G[g.off0 + (long long)(iz + g.npml) * g.pitch + ix + g.npml]);
+    }
+    return;
   }
+  const long long q = (blockIdx.x - inner) * 8LL + (threadIdx.x >> 5);
+  if (q >= n_boundary(g)) return;
+  int iz, ix;
+  boundary_cell(g, q, &iz, &ix);
+  const int i_lo = iz == 0 ? 0 : iz + g.npml, i_hi = iz == g.nz - 1 ? g.Nz - 1 : iz + g.npml;
+  const int j_lo = ix == 0 ? 0 : ix + g.npml, j_hi = ix == g.nx - 1 ? g.Nx - 1 : ix + g.npml;
+  const int w = j_hi - j_lo + 1, cells = (i_hi - i_lo + 1) * w;
+  double acc = 0.0;
+  for (int k = threadIdx.x & 31; k < cells; k += 32)
+    acc += G[g.off0 + (long long)(i_lo + k / w) * g.pitch + j_lo + k % w];
+  acc = warp_sum(acc);
+  const long long idx = (long long)iz * g.nx + ix;
+  if ((threadIdx.x & 31) == 0) grad[idx] = (float)((double)c[idx] * acc);
 }
 
 // Source-parameter gradients from the per-step partials (nslots per step,
@@ -518,20 +579,21 @@ cudaError_t launch_rec_csr(int nrec, const int* iz, const int* ix, const Grid& g
   return cudaGetLastError();
 }
 cudaError_t launch_model_check(const float* c, long long n, float coef, int* status, cudaStream_t st) {
-  k_model_check<<<1, 1024, 0, st>>>(c, n, coef, status);
+  k_model_check<<<(unsigned)std::max<long long>(1, std::min<long long>((n + 1023) / 1024, 304)), 1024, 0, st>>>(
+      c, n, coef, status);
   return cudaGetLastError();
 }
 cudaError_t launch_misfit(const float* seis, float* res, long long n, double* part, int nb, double* J,
                           int* status, bool vjp, cudaStream_t st) {
   if (vjp) k_misfit<true><<<nb, 256, 0, st>>>(seis, res, n, part);
   else k_misfit<false><<<nb, 256, 0, st>>>(seis, res, n, part);
-  k_misfit_final<<<1, 32, 0, st>>>(part, nb, vjp ? 1.0 : 0.5, J, status);
+  k_misfit_final<<<1, 256, 0, st>>>(part, nb, vjp ? 1.0 : 0.5, J, status);
   return cudaGetLastError();
 }
 cudaError_t launch_superpose(const float* seis, int S, long long n, const float* obs, float* cot, double* part,
                              int nb, double* J, int* status, cudaStream_t st) {
   k_superpose<<<nb, 256, 0, st>>>(seis, S, n, obs, cot, part);
-  k_misfit_final<<<1, 32, 0, st>>>(part, nb, 0.5, J, status);
+  k_misfit_final<<<1, 256, 0, st>>>(part, nb, 0.5, J, status);
   return cudaGetLastError();
 }
 cudaError_t launch_finite_check(const float* a, long long n, int* status, cudaStream_t st) {
@@ -539,7 +601,7 @@ cudaError_t launch_finite_check(const float* a, long long n, int* status, cudaSt
   return cudaGetLastError();
 }
 cudaError_t launch_adj_init(const AcuStep& p, float* lam, float* hx, float* hz, cudaStream_t st, bool lap) {
-  k_adj_init<<<p.S, 32, 0, st>>>(p, lam, hx, hz, lap);
+  k_adj_init<<<p.S, 256, 0, st>>>(p, lam, hx, hz, lap);
   return cudaGetLastError();
 }
 // Copies of a descriptor table: block row y copies descriptor y.
@@ -558,7 +620,8 @@ cudaError_t launch_fold(float* gpart, int S, long long slice, double* G, cudaStr
   return cudaGetLastError();
 }
 cudaError_t launch_grad_c(const double* G, const Grid& g, const float* c, float* grad, cudaStream_t st) {
-  k_grad_c<<<304, 256, 0, st>>>(G, g, c, grad);
+  const int inner = 304;
+  k_grad_c<<<(unsigned)(inner + (n_boundary(g) + 7) / 8), 256, 0, st>>>(G, g, c, grad, inner);
   return cudaGetLastError();
 }
 cudaError_t launch_src_grad(const float* part, int S, int nt, int nslots, double scale, const float* stf,
