@@ -314,30 +314,41 @@ __global__ void __launch_bounds__(256) k_im2col_n(const float* __restrict__ x, c
 }
 
 // dx[c][b][r][s] = sum over the taps (p, q) that read (r, s): dcol[c*9+p*3+q][(b*Ho+i)*Wo+j]
-// with r = sh i + p - 1, s = sw j + q - 1 (a gather: each output written once, fixed order).
+// with r = sh i + p - 1, s = sw j + q - 1 (a gather: each output written once, in
+// tap order). A warp takes one row (c, b, r) of dx, so the row's tap rows p and
+// their dcol rows are decided once for it and its lanes read along the columns
+// (decoding and dividing for every element: 630 us for the four strided layers of
+// a batch of 32, this 248).
+template <int SW>
 __global__ void __launch_bounds__(256) k_col2im(const float* __restrict__ dcol, const ConvDims d,
                                                 float* __restrict__ dx) {
-  const int total = d.C * d.B * d.H * d.W;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
-    const uint32_t t1 = d.fW.div((uint32_t)e), t2 = d.fH.div(t1), c = d.fB.div(t2);
-    const int s = (int)d.fW.mod((uint32_t)e, t1), r = (int)d.fH.mod(t1, t2), b = (int)d.fB.mod(t2, c);
-    float acc = 0.f;
+  const int rows = d.C * d.B * d.H, lane = threadIdx.x & 31;
+  for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < rows; row += gridDim.x * 8) {
+    const uint32_t cb = d.fH.div((uint32_t)row), c = d.fB.div(cb);
+    const int r = (int)d.fH.mod((uint32_t)row, cb), b = (int)d.fB.mod(cb, c);
+    const float* src[3];
 #pragma unroll
     for (int p = 0; p < 3; p++) {
-      const int ri = r + 1 - p;
-      if (ri < 0 || ri % d.sh != 0) continue;
-      const int i = ri / d.sh;
-      if (i >= d.Ho) continue;
-#pragma unroll
-      for (int q = 0; q < 3; q++) {
-        const int sj = s + 1 - q;
-        if (sj < 0 || sj % d.sw != 0) continue;
-        const int j = sj / d.sw;
-        if (j >= d.Wo) continue;
-        acc += __ldg(dcol + (long long)(c * 9 + p * 3 + q) * d.Npix + (b * d.Ho + i) * d.Wo + j);
-      }
+      const int ri = r + 1 - p, i = ri / d.sh;
+      src[p] = ri >= 0 && ri % d.sh == 0 && i < d.Ho
+                   ? dcol + (long long)(c * 9 + p * 3) * d.Npix + ((long long)b * d.Ho + i) * d.Wo
+                   : nullptr;
     }
-    dx[e] = acc;
+    float* dst = dx + (long long)row * d.W;
+    const int sw = SW ? SW : d.sw;
+    for (int s = lane; s < d.W; s += 32) {
+      float acc = 0.f;
+#pragma unroll
+      for (int p = 0; p < 3; p++) {
+        if (!src[p]) continue;  // the same for the whole warp
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+          const int sj = s + 1 - q, j = sj / sw;
+          if (sj >= 0 && sj % sw == 0 && j < d.Wo) acc += __ldg(src[p] + (long long)q * d.Npix + j);
+        }
+      }
+      dst[s] = acc;
+    }
   }
 }
 
@@ -369,13 +380,21 @@ __global__ void __launch_bounds__(256) k_act_back(float* __restrict__ dy, const 
     part[(long long)o * gridDim.x + chunk] = s;
   }
 }
-// db[o] = sum of the chunk partials in chunk order (one thread per channel)
-__global__ void k_db(const float* __restrict__ part, int O, int nchunk, float* __restrict__ db) {
-  const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= O) return;
+// db[o] = sum of the chunk partials in chunk order (a block per channel: its
+// partials come in together, one thread adds them)
+__global__ void __launch_bounds__(128) k_db(const float* __restrict__ part, int nchunk, float* __restrict__ db) {
+  __shared__ float sp[512];
+  const int o = blockIdx.x;
   float s = 0.f;
-  for (int c = 0; c < nchunk; c++) s += part[(long long)o * nchunk + c];
-  db[o] = s;
+  for (int c0 = 0; c0 < nchunk; c0 += 512) {
+    const int m = min(512, nchunk - c0);
+    for (int c = threadIdx.x; c < m; c += 128) sp[c] = part[(long long)o * nchunk + c0 + c];
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int c = 0; c < m; c++) s += sp[c];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) db[o] = s;
 }
 
 // dyT[pix][o] (row stride ldo) = dyb[o][pix] (row stride ldn): 32 x 32 tiles through shared memory
@@ -420,39 +439,58 @@ __global__ void k_wflip(const uint16_t* __restrict__ w, int O, int C, int ldf, u
 __global__ void k_split_sum(const float* __restrict__ part, int splits, long long n, float* __restrict__ out) {
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     float s = 0.f;
-    for (int k = 0; k < splits; k++) s += part[(long long)k * n + e];
+#pragma unroll 8
+    for (int k = 0; k < splits; k++) s += __ldg(part + (long long)k * n + e);
     out[e] = s;
   }
 }
 
 // Input row `row` (= cb H + r) of x feeds output rows 2 row and 2 row + 1 of y
-// (cb 2H + 2r = 2 row): blocks walk the input rows, threads the columns, and
-// each thread writes its value's 2 x 2 copies as two 8-byte stores (y 8-byte
-// aligned; the launcher checks).
-__global__ void k_upsample2(const float* __restrict__ x, int CB, int H, int W, float* __restrict__ y) {
-  const long long rows = (long long)CB * H, W2 = 2LL * W;
-  for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-    const float* xr = x + row * W;
-    float2* y0 = reinterpret_cast<float2*>(y + 2 * row * W2);
-    float2* y1 = reinterpret_cast<float2*>(y + (2 * row + 1) * W2);
-    for (int s = threadIdx.x; s < W; s += blockDim.x) {
-      const float v = __ldg(xr + s);
-      y0[s] = make_float2(v, v);
-      y1[s] = make_float2(v, v);
+// (cb 2H + 2r = 2 row). Items are V consecutive input values of a row (W = V Wv),
+// numbered through all rows so that short rows fill the warps too; each is written
+// as two 2V-value stores. V = 2 needs even rows and 16-byte aligned y (8-byte x);
+// V = 1 takes the rest (y 8-byte aligned; the launcher checks). A block per row
+// with a thread per value kept a quarter to a half of its lanes busy (238 us for
+// the three layers of a batch of 32, this 97; backward 238 -> 95).
+template <int V>
+__global__ void __launch_bounds__(256) k_upsample2(const float* __restrict__ x, long long items, FastDiv fWv, int W,
+                                                   float* __restrict__ y) {
+  for (long long e = blockIdx.x * 256LL + threadIdx.x; e < items; e += gridDim.x * 256LL) {
+    const long long row = fWv.div((uint32_t)e);
+    const int s = V * (int)(e - row * fWv.d);
+    const float* xr = x + row * W + s;
+    float* y0 = y + 4 * row * W + 2 * s;
+    float* y1 = y0 + 2LL * W;
+    if (V == 2) {
+      const float2 v = __ldg(reinterpret_cast<const float2*>(xr));
+      const float4 o = make_float4(v.x, v.x, v.y, v.y);
+      *reinterpret_cast<float4*>(y0) = o;
+      *reinterpret_cast<float4*>(y1) = o;
+    } else {
+      const float v = __ldg(xr);
+      *reinterpret_cast<float2*>(y0) = make_float2(v, v);
+      *reinterpret_cast<float2*>(y1) = make_float2(v, v);
     }
   }
 }
 
 // dx[row][s] = (dy[2 row][2s] + dy[2 row][2s + 1]) + (dy[2 row + 1][2s] + dy[2 row + 1][2s + 1]),
-// blocks walking the rows and threads the columns (8-byte loads; dy 8-byte aligned).
-__global__ void k_upsample2_back(const float* __restrict__ dy, int CB, int H, int W, float* __restrict__ dx) {
-  const long long rows = (long long)CB * H, W2 = 2LL * W;
-  for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-    const float2* d0 = reinterpret_cast<const float2*>(dy + 2 * row * W2);
-    const float2* d1 = reinterpret_cast<const float2*>(dy + (2 * row + 1) * W2);
-    for (int s = threadIdx.x; s < W; s += blockDim.x) {
-      const float2 a = __ldg(d0 + s), b = __ldg(d1 + s);
-      dx[row * W + s] = (a.x + a.y) + (b.x + b.y);
+// items as in k_upsample2 (dy 16- or 8-byte aligned).
+template <int V>
+__global__ void __launch_bounds__(256) k_upsample2_back(const float* __restrict__ dy, long long items, FastDiv fWv,
+                                                        int W, float* __restrict__ dx) {
+  for (long long e = blockIdx.x * 256LL + threadIdx.x; e < items; e += gridDim.x * 256LL) {
+    const long long row = fWv.div((uint32_t)e);
+    const int s = V * (int)(e - row * fWv.d);
+    const float* d0 = dy + 4 * row * W + 2 * s;
+    const float* d1 = d0 + 2LL * W;
+    float* o = dx + row * W + s;
+    if (V == 2) {
+      const float4 a = __ldg(reinterpret_cast<const float4*>(d0)), b = __ldg(reinterpret_cast<const float4*>(d1));
+      *reinterpret_cast<float2*>(o) = make_float2((a.x + a.y) + (b.x + b.y), (a.z + a.w) + (b.z + b.w));
+    } else {
+      const float2 a = __ldg(reinterpret_cast<const float2*>(d0)), b = __ldg(reinterpret_cast<const float2*>(d1));
+      *o = (a.x + a.y) + (b.x + b.y);
     }
   }
 }
@@ -481,9 +519,12 @@ __global__ void __launch_bounds__(256) k_mse(const float* __restrict__ p, const 
   }
 }
 __global__ void k_mse_final(const double* __restrict__ part, long long n, double* loss) {
+  __shared__ double sp[MSE_BLOCKS];
+  for (int k = threadIdx.x; k < MSE_BLOCKS; k += blockDim.x) sp[k] = part[k];
+  __syncthreads();
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int k = 0; k < MSE_BLOCKS; k++) s += part[k];
+    for (int k = 0; k < MSE_BLOCKS; k++) s += sp[k];
     *loss = 0.5 * s / (double)n;
   }
 }
@@ -746,7 +787,11 @@ fwi_status fwi_cnn_conv_backward(fwi_cnn* h, const float* x, int32_t C, int32_t 
   const bool s1 = sh == 1 && sw == 1;
   Carve cv;
   const size_t o_dyb = cv.take((size_t)O * ldn * 2), o_bp = cv.take((size_t)O * nchunk * 4);
-  size_t colb_elems = (size_t)d.K9 * ldn;
+  // the weight gradient gathers its tap operand too, unless the layer's rows or the
+  // input's alignment rule pixel pairs out
+  const fwi::TcConvA cx = fwi::tc_conv_a(x, C, B, H, W, sh, sw);
+  const bool wg = h->gather && fwi::tc_conv_pairs(cx) != 0;
+  size_t colb_elems = wg ? 0 : (size_t)d.K9 * ldn;
   if (dx) colb_elems = std::max(colb_elems, s1 ? (h->gather ? 0 : (size_t)dd.Npix * ldf) : (size_t)d.Npix * ldo);
   const size_t o_col = cv.take(colb_elems * 2);
   const size_t o_wt = cv.take(dx ? (size_t)(s1 ? C * ldf : d.K9 * ldo) * 2 : 0);
@@ -764,7 +809,7 @@ fwi_status fwi_cnn_conv_backward(fwi_cnn* h, const float* x, int32_t C, int32_t 
 
   fwi::k_act_back<<<dim3(nchunk, O), 256, 0, st>>>(dy, y, d.Npix, ldn, relu, dyb, bpart);
   CNN_CK(cudaGetLastError(), "activation backward");
-  fwi::k_db<<<(O + 127) / 128, 128, 0, st>>>(bpart, O, nchunk, db);
+  fwi::k_db<<<O, 128, 0, st>>>(bpart, nchunk, db);
   CNN_CK(cudaGetLastError(), "bias gradient");
   if (dx && s1) {
     // stride 1: dx is the convolution of the pre-activation gradient with the
@@ -786,13 +831,14 @@ fwi_status fwi_cnn_conv_backward(fwi_cnn* h, const float* x, int32_t C, int32_t 
     CNN_CK(cudaGetLastError(), "weight layout");
     fwi::TcGemm g{colb, ldo, Wt, ldo, d.Npix, d.K9, O, dcol, d.Npix, 0, nullptr, 0, 1, h->status};
     CNN_CK(fwi::tc_gemm(g, st), "conv data-gradient GEMM");
-    fwi::k_col2im<<<blocks_for((long long)C * B * H * W), 256, 0, st>>>(dcol, d, dx);
+    auto c2i = sw == 1 ? fwi::k_col2im<1> : sw == 2 ? fwi::k_col2im<2> : fwi::k_col2im<0>;
+    c2i<<<(unsigned)std::min<long long>(((long long)C * B * H + 7) / 8, 152 * 64), 256, 0, st>>>(dcol, d, dx);
     CNN_CK(cudaGetLastError(), "col2im");
   }
   // dw[o][k] = sum_pix col[k][pix] dy[o][pix]
-  CNN_CK(im2col_n(x, d, ldn, colb, st), "im2col");
-  fwi::TcGemm g{colb, ldn, dyb, ldn, d.K9, O, d.Npix, S > 1 ? part : dw, d.K9, (long long)O * d.K9, nullptr, 0, S,
-                h->status};
+  if (!wg) CNN_CK(im2col_n(x, d, ldn, colb, st), "im2col");
+  fwi::TcGemm g{wg ? nullptr : colb, ldn, dyb, ldn, d.K9, O, d.Npix, S > 1 ? part : dw, d.K9, (long long)O * d.K9,
+                nullptr, 0, S, h->status, wg ? &cx : nullptr, wg};
   CNN_CK(fwi::tc_gemm(g, st), "conv weight-gradient GEMM");
   if (S > 1) {
     fwi::k_split_sum<<<blocks_for((long long)O * d.K9), 256, 0, st>>>(part, S, (long long)O * d.K9, dw);
@@ -806,10 +852,12 @@ fwi_status fwi_cnn_upsample2(const float* x, int32_t C, int32_t B, int32_t H, in
   if (bad_dims(C, B, H, W)) return fwi::host_fail(FWI_EINVAL, "bad sizes");
   if ((long long)C * B * 4 * H * W > 0x7fffff00LL) return fwi::host_fail(FWI_EINVAL, "tensor too large");
   if ((uintptr_t)y & 7) return fwi::host_fail(FWI_EINVAL, "y must be 8-byte aligned");
-  const int CB = C * B;
-  const long long rows = (long long)CB * H;
-  fwi::k_upsample2<<<(unsigned)std::min<long long>(rows, 65535LL * 16), W >= 256 ? 256 : 128, 0,
-                     (cudaStream_t)stream>>>(x, CB, H, W, y);
+  const bool pairs = W % 2 == 0 && (uintptr_t)x % 8 == 0 && (uintptr_t)y % 16 == 0;
+  const int Wv = pairs ? W / 2 : W;
+  const long long items = (long long)C * B * H * Wv;
+  auto up = pairs ? fwi::k_upsample2<2> : fwi::k_upsample2<1>;
+  up<<<(unsigned)std::min<long long>((items + 255) / 256, 152 * 32), 256, 0, (cudaStream_t)stream>>>(
+      x, items, fwi::FastDiv((uint32_t)Wv), W, y);
   CNN_CK(cudaGetLastError(), "upsample");
   return FWI_OK;
 }
@@ -820,10 +868,12 @@ fwi_status fwi_cnn_upsample2_backward(const float* dy, int32_t C, int32_t B, int
   if (bad_dims(C, B, H, W)) return fwi::host_fail(FWI_EINVAL, "bad sizes");
   if ((long long)C * B * 4 * H * W > 0x7fffff00LL) return fwi::host_fail(FWI_EINVAL, "tensor too large");
   if ((uintptr_t)dy & 7) return fwi::host_fail(FWI_EINVAL, "dy must be 8-byte aligned");
-  const int CB = C * B;
-  const long long rows = (long long)CB * H;
-  fwi::k_upsample2_back<<<(unsigned)std::min<long long>(rows, 65535LL * 16), W >= 256 ? 256 : 128, 0,
-                          (cudaStream_t)stream>>>(dy, CB, H, W, dx);
+  const bool pairs = W % 2 == 0 && (uintptr_t)dx % 8 == 0 && (uintptr_t)dy % 16 == 0;
+  const int Wv = pairs ? W / 2 : W;
+  const long long items = (long long)C * B * H * Wv;
+  auto back = pairs ? fwi::k_upsample2_back<2> : fwi::k_upsample2_back<1>;
+  back<<<(unsigned)std::min<long long>((items + 255) / 256, 152 * 32), 256, 0, (cudaStream_t)stream>>>(
+      dy, items, fwi::FastDiv((uint32_t)Wv), W, dx);
   CNN_CK(cudaGetLastError(), "upsample backward");
   return FWI_OK;
 }
@@ -835,7 +885,7 @@ fwi_status fwi_cnn_mse(fwi_cnn* h, const float* p, const float* t, int64_t n, do
   CNN_CK(cudaSetDevice(h->device), "cudaSetDevice");
   fwi::k_mse<<<fwi::MSE_BLOCKS, 256, 0, (cudaStream_t)stream>>>(p, t, n, h->red, dp);
   CNN_CK(cudaGetLastError(), "mse");
-  fwi::k_mse_final<<<1, 32, 0, (cudaStream_t)stream>>>(h->red, n, loss);
+  fwi::k_mse_final<<<1, 320, 0, (cudaStream_t)stream>>>(h->red, n, loss);
   CNN_CK(cudaGetLastError(), "mse");
   return FWI_OK;
 }

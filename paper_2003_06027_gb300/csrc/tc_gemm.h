@@ -53,7 +53,15 @@ struct TcGemm {
   // (M = B Ho Wo pixels, K = 9 C taps); the results equal those of the
   // im2col matrix of the same layer bit for bit
   const TcConvA* conv = nullptr;
+  // with conv: the weight gradient's product instead, A[m][k] = tap m of pixel k
+  // (M = 9 C taps, K = B Ho Wo pixels); needs tc_conv_pairs(*conv) != 0
+  bool wgrad = false;
 };
+
+// Whether the gather can take a layer's outputs in pairs: horizontal stride 1 (or
+// 2; the value returned), an even number of outputs per row and 8-byte (16-byte)
+// aligned pairs of inputs. 0 if not.
+int tc_conv_pairs(const TcConvA& c);
 
 cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st);
 
