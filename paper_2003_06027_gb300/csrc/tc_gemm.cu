@@ -121,12 +121,13 @@ __device__ __forceinline__ uint32_t mulhi_div(uint32_t n, unsigned long long m, 
 // warps 0-7 gather A (two threads per tile row, 32 taps each; warps 0-3 also
 // run the epilogue), warp 8 loads B by TMA, warp 9 issues the MMAs. Up to two
 // CONV CTAs share an SM, so that one's gather covers the other's load latency.
-// CONV: 0 A by TMA, 1 gathered tap by tap through a table (any layer), 2 and 3
-// gathered by pixel pairs (layers of horizontal stride 1 and 2), 4 and 5 the
-// weight gradient's A (rows = taps, K = pixels) gathered the same way.
+// CONV: 0 A by TMA, 1 gathered tap by tap through a table (any layer), 2 and 3 the
+// weight gradient's A (rows = taps, K = pixels) gathered by pixel pairs (layers of
+// horizontal stride 1 and 2; their forward and data-gradient products have a kernel
+// of their own, k_conv_pairs).
 template <int CONV>
 struct TcRoles {
-  static constexpr bool WG = CONV >= 4;
+  static constexpr bool WG = CONV >= 2;
   static constexpr int BM = WG ? TC_WG_ROWS : TC_BM;  // rows of D per tile
   static constexpr int ARRIVE = WG ? 64 : 2 * TC_BM;  // gathering threads of one stage
   static constexpr int THREADS = CONV ? 320 : TC_THREADS;
@@ -215,14 +216,14 @@ struct PairWin {
       right = SW == 2 || j + 2 < c.W;
     }
   }
-  // BF16 words of 4 channels' 36 taps for both pixels; channel u of them exists if cok(u)
-  template <typename F>
+  // BF16 words of NB channels' 9 NB taps for both pixels; channel u of them exists if cok(u)
+  template <int NB, typename F>
   __device__ __forceinline__ void words(const TcConvA& c, int ch0, F cok, uint32_t* w0, uint32_t* w1) const {
     constexpr int NV = SW + 3;  // input columns SW j - 1 .. SW j + SW + 1 of a pair
     const long long plane = (long long)c.B * c.H * c.W;
-    float v[4][3][NV];
+    float v[NB][3][NV];
 #pragma unroll
-    for (int u = 0; u < 4; u++) {
+    for (int u = 0; u < NB; u++) {
       const float* xc = base + (long long)(ch0 + u) * plane;
       const bool ck = cok(u);
 #pragma unroll
@@ -244,9 +245,9 @@ struct PairWin {
         }
       }
     }
-    // tap e of the four channels: (channel e / 9, row e % 9 / 3, column e % 3)
+    // tap e of the channels: (channel e / 9, row e % 9 / 3, column e % 3)
 #pragma unroll
-    for (int k = 0; k < 18; k++) {
+    for (int k = 0; k < 9 * NB / 2; k++) {
       const int e = 2 * k, f = 2 * k + 1;
       const __nv_bfloat162 h0 = __floats2bfloat162_rn(v[e / 9][e % 9 / 3][e % 3], v[f / 9][f % 9 / 3][f % 3]);
       const __nv_bfloat162 h1 =
@@ -257,67 +258,70 @@ struct PairWin {
   }
 };
 
-// Gathers A by pixel pairs: thread (pair, sub) of 64 x 4 builds rows 2 pair and
-// 2 pair + 1 of every stage tile (two neighbouring output pixels of one image
-// row), taking every fourth run of 8 channels. The 72 taps of 8 channels are 9
+// Gathers the A tile of pixels m0 .. m0 + 127 by pairs: thread (pair, sub) of 64 x
+// 4 builds two rows of every stage tile, two neighbouring output pixels of one
+// image row, taking every fourth run of 8 channels. The 72 taps of 8 channels are 9
 // whole 16-byte chunks of a row, so a run's values go from registers to shared
 // memory without a table: per channel a thread reads the 3 x (2 SW + 2) input
 // values of its pair once (9 loads for 18 operand elements at SW = 1), and each
-// BF16 word is one packed conversion of two of them. About 1.6 instructions per
-// element against 6 for the table (each tap decoded, tested and loaded by
-// itself), which is what bounds these GEMMs: their layers are thin, and the
-// tensor pipe waits for A. The operand is the same, so the results are too.
-// Every thread enters (waits for) and leaves (arrives on) every k-block's stage
-// in order, whether it has chunks there or not.
+// BF16 word is one packed conversion of two of them: about 1.6 instructions per
+// element against 6 for the table (each tap decoded, tested and loaded by itself).
+// Within 16 pixels the even ones take the first 8 rows and the odd ones the next 8:
+// the 8 lanes of a 16-byte store phase then write 8 different rows mod 8, which the
+// swizzle sends to different banks (even and odd rows in turn would meet two by two).
+// Every thread enters (waits for) and leaves (arrives on) every k-block's stage in
+// order, whether it has chunks there or not; `kb0` counts the k-blocks of the CTA's
+// earlier tiles.
+__device__ __forceinline__ int pair_row(int pair) { return ((pair & ~7) << 1) | (pair & 7); }  // and + 8
+__device__ __forceinline__ int row_pixel(int row) { return 2 * (((row >> 4) << 3) | (row & 7)) + ((row >> 3) & 1); }
 template <int SW>
-__device__ __forceinline__ bool gather_pairs(const TcConvA& c, long long m0, long long M, int nk, unsigned char* smA,
-                                             uint64_t* empty, uint64_t* fulla) {
-  const int pair = threadIdx.x & 63, sub = threadIdx.x >> 6, row = 2 * pair;
-  const PairWin<SW> win(c, m0 + row, M);
+__device__ __forceinline__ bool gather_pairs(const TcConvA& c, long long m0, long long M, int kb0, int nk,
+                                             unsigned char* smA, uint64_t* empty, uint64_t* fulla) {
+  const int pair = threadIdx.x & 63, sub = threadIdx.x >> 6;
+  const PairWin<SW> win(c, m0 + 2 * pair, M);
   const int nchunk = nk * (TC_BK / 8);
-  int cur = -1;  // k-block whose stage this thread has entered
+  int cur = -1;  // k-block of the tile whose stage this thread has entered
   auto enter = [&](int kb) -> bool {
     while (cur < kb) {
       if (cur >= 0) {
         fence_proxy_async();  // the generic-proxy writes before the tensor core reads them
-        mbar_arrive(&fulla[cur % TC_STAGES]);
+        mbar_arrive(&fulla[(kb0 + cur) % TC_STAGES]);
       }
       cur++;
-      if (!mbar_wait(&empty[cur % TC_STAGES], ((uint32_t)(cur / TC_STAGES) & 1u) ^ 1u)) return false;
+      const int k = kb0 + cur;
+      if (!mbar_wait(&empty[k % TC_STAGES], ((uint32_t)(k / TC_STAGES) & 1u) ^ 1u)) return false;
     }
     return true;
   };
-  const int sw0 = row & 7;
   for (int g0 = 9 * sub; g0 < nchunk; g0 += 36) {  // chunks g0 .. g0 + 8: channels 8 g0 / 9 ..
     const int ch0 = 8 * (g0 / 9);
-    uint32_t w0[20], w1[20];  // BF16 words of the two rows: two carried over, 18 of four channels
+    uint32_t w0[12], w1[12];  // BF16 words of the two rows: up to three carried over, 9 of two channels
 #pragma unroll
-    for (int half = 0; half < 2; half++) {
-      const int ch = ch0 + 4 * half;
-      win.words(c, ch, [&](int u) { return ch + u < c.C; }, w0 + 2 * half, w1 + 2 * half);
+    for (int u = 0; u < 4; u++) {
+      const int ch = ch0 + 2 * u;
+      win.template words<2>(c, ch, [&](int k) { return ch + k < c.C; }, w0 + u, w1 + u);
+      const int nc = u < 3 ? 2 : 3;  // whole chunks in hand
 #pragma unroll
-      for (int k = 0; k < 4 + half; k++) {
-        const int g = g0 + 4 * half + k;
+      for (int k = 0; k < nc; k++) {
+        const int g = g0 + 2 * u + k;
         if (g < nchunk) {
           if (!enter(g >> 3)) return false;
-          unsigned char* rp = smA + (cur % TC_STAGES) * A_STAGE + row * 128;
-          *reinterpret_cast<uint4*>(rp + (((g & 7) ^ sw0) << 4)) =
-              make_uint4(w0[4 * k], w0[4 * k + 1], w0[4 * k + 2], w0[4 * k + 3]);
-          *reinterpret_cast<uint4*>(rp + 128 + (((g & 7) ^ (sw0 + 1)) << 4)) =
-              make_uint4(w1[4 * k], w1[4 * k + 1], w1[4 * k + 2], w1[4 * k + 3]);
+          unsigned char* rp = smA + ((kb0 + cur) % TC_STAGES) * A_STAGE + pair_row(pair) * 128 +
+                              (((g & 7) ^ (pair & 7)) << 4);
+          *reinterpret_cast<uint4*>(rp) = make_uint4(w0[4 * k], w0[4 * k + 1], w0[4 * k + 2], w0[4 * k + 3]);
+          *reinterpret_cast<uint4*>(rp + 1024) = make_uint4(w1[4 * k], w1[4 * k + 1], w1[4 * k + 2], w1[4 * k + 3]);
         }
       }
-      if (half == 0) {  // words 16, 17 open the fifth chunk
-        w0[0] = w0[16];
-        w0[1] = w0[17];
-        w1[0] = w1[16];
-        w1[1] = w1[17];
+#pragma unroll
+      for (int k = 0; k < u + 1 && u < 3; k++) {
+        w0[k] = w0[8 + k];
+        w1[k] = w1[8 + k];
       }
     }
   }
   if (!enter(nk - 1)) return false;
   fence_proxy_async();
-  mbar_arrive(&fulla[cur % TC_STAGES]);
+  mbar_arrive(&fulla[(kb0 + cur) % TC_STAGES]);
   return true;
 }
 
@@ -342,7 +346,7 @@ __device__ __forceinline__ bool gather_wgrad(const TcConvA& c, int kb0, int nk, 
     uint32_t w0[20], w1[20];  // as in gather_pairs
 #pragma unroll
     for (int half = 0; half < 2; half++) {
-      win.words(c, ch0 + 4 * half, [&](int u) { return 4 * half + u < nch; }, w0 + 2 * half, w1 + 2 * half);
+      win.template words<4>(c, ch0 + 4 * half, [&](int u) { return 4 * half + u < nch; }, w0 + 2 * half, w1 + 2 * half);
       if (half == 0 && !mbar_wait(&empty[slot], ((uint32_t)(i / TC_STAGES) & 1u) ^ 1u)) return false;
 #pragma unroll
       for (int k = 0; k < 4 + half; k++) {
@@ -453,9 +457,7 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
     }
     tc_commit(&accb);
   } else if (R::WG && (int)threadIdx.x < R::GATHER) {
-    if (!gather_wgrad<CONV == 5 ? 2 : 1>(conv, kb0, nk, smA, empty, fulla)) err = 1;
-  } else if (CONV >= 2 && (int)threadIdx.x < R::GATHER) {
-    if (!gather_pairs<CONV == 3 ? 2 : 1>(conv, m0, a.M, nk, smA, empty, fulla)) err = 1;
+    if (!gather_wgrad<CONV == 3 ? 2 : 1>(conv, kb0, nk, smA, empty, fulla)) err = 1;
   } else if (CONV == 1 && (int)threadIdx.x < R::GATHER) {
     // A gatherers: half threadIdx.x / 128 of row threadIdx.x % 128 of every stage tile
     const int row = threadIdx.x % TC_BM, half = threadIdx.x / TC_BM;
@@ -515,6 +517,144 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols) : "memory");
 }
 
+// The forward and stride-1 data-gradient products of a layer whose outputs come in
+// pairs: persistent CTAs walk the 128-pixel tiles, and each role runs ahead through
+// the stage ring and two TMEM accumulators without waiting for the others' tiles:
+//   warps 0-7 gather A, warp 8 loads B by TMA, warp 9 issues the MMAs, warps 10-13
+//   drain the accumulator of the tile before (TMEM lane quarter = warp mod 4).
+// One tile per CTA (8192 of them for 32 images of 128 x 256) paid the set-up, the
+// last MMAs and the epilogue with its gather warps idle.
+constexpr int CP_THREADS = 448;
+template <int SW>
+__global__ void __launch_bounds__(CP_THREADS, 2)
+    k_conv_pairs(const __grid_constant__ CUtensorMap tb, const TcArgs a, const TcConvA conv, int ntn, int ntiles) {
+  extern __shared__ unsigned char tc_smem_raw[];
+  __shared__ uint64_t full[TC_STAGES], empty[TC_STAGES], fulla[TC_STAGES], accf[2], acce[2];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int err;
+  const uint32_t raw = smem_u32(tc_smem_raw);
+  unsigned char* smA = tc_smem_raw + ((1024u - (raw & 1023u)) & 1023u);
+  const int B_STAGE = a.BN * TC_BK * 2;
+  unsigned char* smB = smA + TC_STAGES * A_STAGE;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nk = a.nkb;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < TC_STAGES; s++) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+      mbar_init(&fulla[s], 2 * TC_BM);  // one arrival per gathering thread
+    }
+    for (int s = 0; s < 2; s++) {
+      mbar_init(&accf[s], 1);
+      mbar_init(&acce[s], 4);  // one arrival per epilogue warp
+    }
+    err = 0;
+    fence_mbar_init();
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(a.tmem_cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot, acc_stride = a.tmem_cols / 2;
+  volatile int* verr = &err;
+
+  if (warp < 8) {
+    int kb0 = 0;
+    for (int t = blockIdx.x; t < ntiles && !*verr; t += gridDim.x, kb0 += nk)
+      if (!gather_pairs<SW>(conv, (long long)(t / ntn) * TC_BM, a.M, kb0, nk, smA, empty, fulla)) *verr = 1;
+  } else if (warp == 8) {
+    if (lane == 0) {
+      int kb = 0;
+      for (int t = blockIdx.x; t < ntiles && !*verr; t += gridDim.x)
+        for (int i = 0; i < nk; i++, kb++) {
+          const int s = kb % TC_STAGES;
+          if (!mbar_wait(&empty[s], ((uint32_t)(kb / TC_STAGES) & 1u) ^ 1u)) {
+            *verr = 1;
+            break;
+          }
+          mbar_expect_tx(&full[s], (uint32_t)B_STAGE);
+          tma_2d(smB + s * B_STAGE, &tb, i * TC_BK, (t % ntn) * a.BN, &full[s]);
+        }
+    }
+  } else if (warp == 9) {
+    if (lane == 0) {
+      int kb = 0, it = 0;
+      for (int t = blockIdx.x; t < ntiles && !*verr; t += gridDim.x, it++) {
+        const int b = it & 1;
+        if (!mbar_wait(&acce[b], ((uint32_t)(it >> 1) & 1u) ^ 1u)) {
+          *verr = 1;
+          break;
+        }
+        tc_fence_after();
+        for (int i = 0; i < nk; i++, kb++) {
+          const int s = kb % TC_STAGES;
+          const uint32_t ph = (uint32_t)(kb / TC_STAGES) & 1u;
+          if (!mbar_wait(&full[s], ph) || !mbar_wait(&fulla[s], ph)) {
+            *verr = 1;
+            break;
+          }
+          tc_fence_after();
+          const uint64_t ad = sdesc_sw128(smem_u32(smA + s * A_STAGE));
+          const uint64_t bd = sdesc_sw128(smem_u32(smB + s * B_STAGE));
+#pragma unroll
+          for (int kk = 0; kk < TC_BK / 16; kk++)
+            tc_mma(tmem + b * acc_stride, ad + 2 * kk, bd + 2 * kk, a.idesc, (uint32_t)(i | kk));
+          tc_commit(&empty[s]);
+        }
+        tc_commit(&accf[b]);
+      }
+    }
+  } else {
+    // epilogue: TMEM lane = tile row, column = n
+    const int quarter = warp & 3, row = quarter * 32 + lane;
+    int it = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
+      const int b = it & 1;
+      const bool ok = !*verr && mbar_wait(&accf[b], (uint32_t)(it >> 1) & 1u);
+      tc_fence_after();
+      __syncwarp();
+      if (!ok) *verr = 1;
+      const bool bad = !ok || *verr;
+      const long long m = (long long)(t / ntn) * TC_BM + row_pixel(row);
+      const int n0 = (t % ntn) * a.BN;
+      for (int c0 = 0; c0 < a.BN; c0 += 16) {
+        uint32_t r[16];
+        tmem_ld16(tmem + b * acc_stride + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, r);
+        if (m < a.M) {
+#pragma unroll
+          for (int j = 0; j < 16; j++) {
+            const int n = n0 + c0 + j;
+            if (n < a.N) {
+              float v = bad ? __int_as_float(0x7fc00000) : __uint_as_float(r[j]);
+              if (a.bias) v += a.bias[n];
+              if (a.relu) v = fmaxf(v, 0.f);
+              a.out[(long long)n * a.ldo + m] = v;
+            }
+          }
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acce[b]);
+    }
+  }
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (err && threadIdx.x == 0) {
+    atomicOr(a.status, ST_TIMEOUT);
+    // copies and MMAs still in flight land before the CTA exits (bounded)
+    for (int s = 0; s < TC_STAGES; s++) mbar_wait(&full[s], 0) || mbar_wait(&full[s], 1);
+  }
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols) : "memory");
+}
+
 bool encode_bf16_sw128(CUtensorMap* map, const void* base, long long inner, long long rows, long long ld_elems,
                        int box_rows) {
   tma_host::EncodeTiled fn = tma_host::encoder();
@@ -569,6 +709,27 @@ int tc_split_count(long long K, int want) {
   return (int)((nkb + kbps - 1) / kbps);
 }
 
+namespace {
+// Persistent launch of k_conv_pairs: two CTAs per SM while two stage rings fit in
+// shared memory (227 KB) and four accumulators in TMEM (512 columns).
+cudaError_t conv_pairs(const TcConvA& c, const CUtensorMap& tb, TcArgs a, int pairs, cudaStream_t st) {
+  const int smem = TC_STAGES * (A_STAGE + a.BN * TC_BK * 2) + 1024;
+  a.tmem_cols *= 2;
+  const int per_sm = smem <= 112 * 1024 && a.tmem_cols <= 256 ? 2 : 1;
+  const long long ntn = (a.N + a.BN - 1) / a.BN, ntiles = (a.M + TC_BM - 1) / TC_BM * ntn;
+  if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+  int dev = 0, nsm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  auto kern = pairs == 1 ? k_conv_pairs<1> : k_conv_pairs<2>;
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const int grid = (int)std::min<long long>(ntiles, (long long)nsm * per_sm);
+  kern<<<grid, CP_THREADS, smem, st>>>(tb, a, c, (int)ntn, (int)ntiles);
+  return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st) {
   const bool conv = g.conv != nullptr;
   if ((!conv && !g.A) || !g.B || !g.out || !g.status || g.M < 1 || g.N < 1 || g.K < 1 || g.splits < 1)
@@ -608,30 +769,24 @@ cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st) {
   if (!encode_bf16_sw128(&tb, g.B, g.K, g.N, g.ldb, BN)) return cudaErrorInvalidValue;
   if (conv) ta = tb;  // unused: A is gathered
   else if (!encode_bf16_sw128(&ta, g.A, g.K, g.M, g.lda, TC_BM)) return cudaErrorInvalidValue;
-  // the pair gather takes whole K (no splits); with fewer than 8 channels most of a
-  // run of 8 would be padding
   int kind = 0, bm = TC_BM;
   if (conv) {
     const int pairs = tc_conv_pairs(*g.conv);
     kind = 1;
     if (g.wgrad) {
-      kind = 3 + pairs;
+      kind = 1 + pairs;
       bm = TC_WG_ROWS;
       a.idesc |= 1u << 15;  // A is M-major
     } else if (pairs && g.conv->C >= 8 && splits == 1) {
-      kind = 1 + pairs;
+      // (with fewer than 8 channels most of a run of 8 would be padding)
+      return conv_pairs(*g.conv, tb, a, pairs, st);
     }
   }
   const int smem = TC_STAGES * (A_STAGE + BN * TC_BK * 2) + 1024 + (kind == 1 ? (int)nkb * TC_BK * 8 : 0);
   const dim3 grid((unsigned)((g.M + bm - 1) / bm), (unsigned)((g.N + BN - 1) / BN), (unsigned)splits);
   TcConvA c{};
   if (conv) c = *g.conv;
-  auto kern = kind == 0   ? k_tc_gemm<0>
-              : kind == 1 ? k_tc_gemm<1>
-              : kind == 2 ? k_tc_gemm<2>
-              : kind == 3 ? k_tc_gemm<3>
-              : kind == 4 ? k_tc_gemm<4>
-                          : k_tc_gemm<5>;
+  auto kern = kind == 0 ? k_tc_gemm<0> : kind == 1 ? k_tc_gemm<1> : kind == 2 ? k_tc_gemm<2> : k_tc_gemm<3>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   kern<<<grid, conv ? TcRoles<1>::THREADS : TcRoles<0>::THREADS, smem, st>>>(ta, tb, a, c);
