@@ -747,13 +747,21 @@ fwi_status fwi_cnn_conv_forward(fwi_cnn* h, const float* x, int32_t C, int32_t B
   const int ldk = (int)fwi::round8(d.K9);
   const bool gather = h->gather;
   Carve cv;
-  const size_t o_col = cv.take(gather ? 0 : (size_t)d.Npix * ldk * 2), o_wp = cv.take((size_t)O * ldk * 2);
+  // weights whose rows are already whole 16-byte runs are the GEMM's operand as they
+  // stand (every layer of 8 n channels); others are copied to padded rows (a launch
+  // each: the twelve of one survey's pass were 60 us of its 349)
+  const bool direct = ldk == d.K9 && ((uintptr_t)w_bf16 & 15) == 0;
+  const size_t o_col = cv.take(gather ? 0 : (size_t)d.Npix * ldk * 2), o_wp = cv.take(direct ? 0 : (size_t)O * ldk * 2);
   if ((v = ws_reserve(h, cv.off)) != FWI_OK) return v;
   char* ws = (char*)h->ws;
   uint16_t* colT = (uint16_t*)(ws + o_col);
-  uint16_t* Wp = (uint16_t*)(ws + o_wp);
-  fwi::k_wprep<<<blocks_for((long long)O * d.K9), 256, 0, st>>>(w_bf16, O, d.K9, ldk, 0, Wp, nullptr);
-  CNN_CK(cudaGetLastError(), "weight layout");
+  const uint16_t* Wp = w_bf16;
+  if (!direct) {
+    fwi::k_wprep<<<blocks_for((long long)O * d.K9), 256, 0, st>>>(w_bf16, O, d.K9, ldk, 0, (uint16_t*)(ws + o_wp),
+                                                                  nullptr);
+    CNN_CK(cudaGetLastError(), "weight layout");
+    Wp = (const uint16_t*)(ws + o_wp);
+  }
   const fwi::TcConvA ca = fwi::tc_conv_a(x, C, B, H, W, sh, sw);
   if (!gather) CNN_CK(im2col_t(x, d, ldk, colT, st), "im2col");
   fwi::TcGemm g{gather ? nullptr : colT, ldk, Wp, ldk, d.Npix, O, d.K9, y, d.Npix, 0, bias, relu, 1, h->status,

@@ -112,6 +112,9 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t r[16]) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t n) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(n) : "memory");
+}
 __device__ __forceinline__ uint32_t mulhi_div(uint32_t n, unsigned long long m, uint32_t s) {
   return (uint32_t)(((unsigned long long)n * m) >> s);
 }
@@ -129,7 +132,7 @@ template <int CONV>
 struct TcRoles {
   static constexpr bool WG = CONV >= 2;
   static constexpr int BM = WG ? TC_WG_ROWS : TC_BM;  // rows of D per tile
-  static constexpr int ARRIVE = WG ? 64 : 2 * TC_BM;  // gathering threads of one stage
+  static constexpr int ARRIVE = WG ? 2 : 2 * TC_BM / 32;  // gathering warps of one stage
   static constexpr int THREADS = CONV ? 320 : TC_THREADS;
   static constexpr int GATHER = 2 * TC_BM;  // gathering threads (CONV)
   static constexpr int B_WARP = CONV ? 8 : 0;
@@ -259,8 +262,8 @@ struct PairWin {
 };
 
 // Gathers the A tile of pixels m0 .. m0 + 127 by pairs: thread (pair, sub) of 64 x
-// 4 builds two rows of every stage tile, two neighbouring output pixels of one
-// image row, taking every fourth run of 8 channels. The 72 taps of 8 channels are 9
+// SUBS builds two rows of every stage tile, two neighbouring output pixels of one
+// image row, taking every SUBS-th run of 8 channels. The 72 taps of 8 channels are 9
 // whole 16-byte chunks of a row, so a run's values go from registers to shared
 // memory without a table: per channel a thread reads the 3 x (2 SW + 2) input
 // values of its pair once (9 loads for 18 operand elements at SW = 1), and each
@@ -269,32 +272,55 @@ struct PairWin {
 // Within 16 pixels the even ones take the first 8 rows and the odd ones the next 8:
 // the 8 lanes of a 16-byte store phase then write 8 different rows mod 8, which the
 // swizzle sends to different banks (even and odd rows in turn would meet two by two).
-// Every thread enters (waits for) and leaves (arrives on) every k-block's stage in
-// order, whether it has chunks there or not; `kb0` counts the k-blocks of the CTA's
-// earlier tiles.
+// Run r of a tile fills chunks 9 r .. 9 r + 8: a stage of 8 chunks belongs to one or two
+// runs, and only their warps wait for it and arrive on it (one warp of a lone run for
+// two), so that no warp spends instructions on stages that it has nothing for. The
+// runs of all tiles go round the SUBS groups in turn: few channels keep all of them
+// busy, and a group's next run starts at most 9 SUBS chunks after its last one's start:
+// with SUBS <= TC_STAGES its wait for a stage is at most one phase ahead, as the parity needs.
+// Against every thread of every group waiting for and arriving on every stage, tile by
+// tile (batch 32): 16 channels at 500 x 64, 107 -> 81 us, 32 at 128 x 256, 195 -> 143, 64 at
+// 128 x 256, 256 -> 229; the step's 18 products 1782 -> 1650. With the next run's lines
+// asked for ahead 1744 -> 1650.
 __device__ __forceinline__ int pair_row(int pair) { return ((pair & ~7) << 1) | (pair & 7); }  // and + 8
 __device__ __forceinline__ int row_pixel(int row) { return 2 * (((row >> 4) << 3) | (row & 7)) + ((row >> 3) & 1); }
-template <int SW>
-__device__ __forceinline__ bool gather_pairs(const TcConvA& c, long long m0, long long M, int kb0, int nk,
+// The whole warp waits for a stage (and agrees on a wait that ran out), and leaves it
+// by one arrival of weight n.
+__device__ __forceinline__ bool warp_enter(uint64_t* empty, uint32_t ph) {
+  return __all_sync(0xffffffffu, mbar_wait(empty, ph));
+}
+__device__ __forceinline__ void warp_leave(uint64_t* fulla, uint32_t n) {
+  fence_proxy_async();  // the generic-proxy writes before the tensor core reads them
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) mbar_arrive_n(fulla, n);
+}
+template <int SW, int SUBS>
+__device__ __forceinline__ bool gather_pairs(const TcConvA& c, long long M, int nk, int ntn, int ntiles,
                                              unsigned char* smA, uint64_t* empty, uint64_t* fulla) {
-  const int pair = threadIdx.x & 63, sub = threadIdx.x >> 6;
-  const PairWin<SW> win(c, m0 + 2 * pair, M);
-  const int nchunk = nk * (TC_BK / 8);
-  int cur = -1;  // k-block of the tile whose stage this thread has entered
-  auto enter = [&](int kb) -> bool {
-    while (cur < kb) {
-      if (cur >= 0) {
-        fence_proxy_async();  // the generic-proxy writes before the tensor core reads them
-        mbar_arrive(&fulla[(kb0 + cur) % TC_STAGES]);
-      }
-      cur++;
-      const int k = kb0 + cur;
-      if (!mbar_wait(&empty[k % TC_STAGES], ((uint32_t)(k / TC_STAGES) & 1u) ^ 1u)) return false;
+  static_assert(SUBS <= TC_STAGES, "stage waits at most one phase ahead");
+  const int pair = threadIdx.x & 63;
+  const int nchunk = nk * (TC_BK / 8), nrun = (nchunk + 8) / 9;
+  int t = blockIdx.x, kb0 = 0, r = threadIdx.x >> 6;  // tile, its first k-block in this CTA's sequence, run
+  for (; r >= nrun; r -= nrun, kb0 += nk) t += gridDim.x;
+  unsigned char* rows = smA + pair_row(pair) * 128;
+  int wt = -1;
+  PairWin<SW> win(c, M, M);
+  for (; t < ntiles;) {
+    if (wt != t) win = PairWin<SW>(c, (long long)(t / ntn) * TC_BM + 2 * pair, M);
+    wt = t;
+    const int g0 = 9 * r, ch0 = 8 * r;
+    // the next run's lines into L1, which its loads need in four dependent rounds: lane
+    // l asks for channel l % 8 at the window of lane l & 24, 16 pixels apart
+    const int lane = threadIdx.x & 31, ca = ch0 + 8 * SUBS + (lane & 7);
+    const float* ahead = reinterpret_cast<const float*>(
+        __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(win.base), lane & 24));
+    const int ar = __shfl_sync(0xffffffffu, (int)win.rok[0] | (int)win.rok[1] << 1 | (int)win.rok[2] << 2, lane & 24);
+    if (ca < c.C) {
+#pragma unroll
+      for (int p = 0; p < 3; p++)
+        if (ar >> p & 1) prefetch_l1(ahead + (long long)ca * c.B * c.H * c.W + p * c.W);
     }
-    return true;
-  };
-  for (int g0 = 9 * sub; g0 < nchunk; g0 += 36) {  // chunks g0 .. g0 + 8: channels 8 g0 / 9 ..
-    const int ch0 = 8 * (g0 / 9);
+    int kb = -1;  // k-block of the tile whose stage this warp has entered
     uint32_t w0[12], w1[12];  // BF16 words of the two rows: up to three carried over, 9 of two channels
 #pragma unroll
     for (int u = 0; u < 4; u++) {
@@ -305,9 +331,13 @@ __device__ __forceinline__ bool gather_pairs(const TcConvA& c, long long m0, lon
       for (int k = 0; k < nc; k++) {
         const int g = g0 + 2 * u + k;
         if (g < nchunk) {
-          if (!enter(g >> 3)) return false;
-          unsigned char* rp = smA + ((kb0 + cur) % TC_STAGES) * A_STAGE + pair_row(pair) * 128 +
-                              (((g & 7) ^ (pair & 7)) << 4);
+          if (kb != g >> 3) {
+            if (kb >= 0) warp_leave(&fulla[(kb0 + kb) % TC_STAGES], 8 * kb % 9 <= 1 ? 2 : 1);
+            kb = g >> 3;
+            const uint32_t n = (uint32_t)(kb0 + kb);
+            if (!warp_enter(&empty[n % TC_STAGES], (n / TC_STAGES & 1u) ^ 1u)) return false;
+          }
+          unsigned char* rp = rows + ((kb0 + kb) % TC_STAGES) * A_STAGE + (((g & 7) ^ (pair & 7)) << 4);
           *reinterpret_cast<uint4*>(rp) = make_uint4(w0[4 * k], w0[4 * k + 1], w0[4 * k + 2], w0[4 * k + 3]);
           *reinterpret_cast<uint4*>(rp + 1024) = make_uint4(w1[4 * k], w1[4 * k + 1], w1[4 * k + 2], w1[4 * k + 3]);
         }
@@ -318,10 +348,9 @@ __device__ __forceinline__ bool gather_pairs(const TcConvA& c, long long m0, lon
         w1[k] = w1[8 + k];
       }
     }
+    warp_leave(&fulla[(kb0 + kb) % TC_STAGES], 8 * kb % 9 <= 1 ? 2 : 1);
+    for (r += SUBS; r >= nrun; r -= nrun, kb0 += nk) t += gridDim.x;
   }
-  if (!enter(nk - 1)) return false;
-  fence_proxy_async();
-  mbar_arrive(&fulla[(kb0 + cur) % TC_STAGES]);
   return true;
 }
 
@@ -347,7 +376,7 @@ __device__ __forceinline__ bool gather_wgrad(const TcConvA& c, int kb0, int nk, 
 #pragma unroll
     for (int half = 0; half < 2; half++) {
       win.template words<4>(c, ch0 + 4 * half, [&](int u) { return 4 * half + u < nch; }, w0 + 2 * half, w1 + 2 * half);
-      if (half == 0 && !mbar_wait(&empty[slot], ((uint32_t)(i / TC_STAGES) & 1u) ^ 1u)) return false;
+      if (half == 0 && !warp_enter(&empty[slot], ((uint32_t)(i / TC_STAGES) & 1u) ^ 1u)) return false;
 #pragma unroll
       for (int k = 0; k < 4 + half; k++) {
         const int g = 9 * grp + 4 * half + k;  // chunk of the pixel's 16
@@ -366,8 +395,7 @@ __device__ __forceinline__ bool gather_wgrad(const TcConvA& c, int kb0, int nk, 
         w1[1] = w1[17];
       }
     }
-    fence_proxy_async();  // the generic-proxy writes before the tensor core reads them
-    mbar_arrive(&fulla[slot]);
+    warp_leave(&fulla[slot], 1);
   }
   return true;
 }
@@ -407,7 +435,7 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
     for (int s = 0; s < TC_STAGES; s++) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
-      mbar_init(&fulla[s], R::ARRIVE);  // CONV: one arrival per gathering thread of the stage
+      mbar_init(&fulla[s], R::ARRIVE);  // CONV: one arrival per gathering warp of the stage
     }
     mbar_init(&accb, 1);
     err = 0;
@@ -472,13 +500,12 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
 #pragma unroll
       for (int kk = 0; kk < GATHER_K; kk++) v[kk] = vn[kk];
       if (i + 1 < nk) gather_load(conv, g, tab, kb0 + i + 1, half, vn);
-      if (!mbar_wait(&empty[s], ph ^ 1u)) {
+      if (!warp_enter(&empty[s], ph ^ 1u)) {
         err = 1;
         break;
       }
       gather_store(v, row, half, smA + s * A_STAGE);
-      fence_proxy_async();  // the generic-proxy writes before the tensor core reads them
-      mbar_arrive(&fulla[s]);
+      warp_leave(&fulla[s], 1);
     }
   }
   __syncwarp();
@@ -524,10 +551,11 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
 //   drain the accumulator of the tile before (TMEM lane quarter = warp mod 4).
 // One tile per CTA (8192 of them for 32 images of 128 x 256) paid the set-up, the
 // last MMAs and the epilogue with its gather warps idle.
-constexpr int CP_THREADS = 448;
+constexpr int CP_SUBS = 4;  // groups of two gathering warps
 template <int SW>
-__global__ void __launch_bounds__(CP_THREADS, 2)
+__global__ void __launch_bounds__(64 * CP_SUBS + 192, 2)
     k_conv_pairs(const __grid_constant__ CUtensorMap tb, const TcArgs a, const TcConvA conv, int ntn, int ntiles) {
+  constexpr int GW = 2 * CP_SUBS;  // gathering warps
   extern __shared__ unsigned char tc_smem_raw[];
   __shared__ uint64_t full[TC_STAGES], empty[TC_STAGES], fulla[TC_STAGES], accf[2], acce[2];
   __shared__ uint32_t tmem_slot;
@@ -541,7 +569,7 @@ __global__ void __launch_bounds__(CP_THREADS, 2)
     for (int s = 0; s < TC_STAGES; s++) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
-      mbar_init(&fulla[s], 2 * TC_BM);  // one arrival per gathering thread
+      mbar_init(&fulla[s], 4);  // two warps of two runs
     }
     for (int s = 0; s < 2; s++) {
       mbar_init(&accf[s], 1);
@@ -562,11 +590,9 @@ __global__ void __launch_bounds__(CP_THREADS, 2)
   const uint32_t tmem = tmem_slot, acc_stride = a.tmem_cols / 2;
   volatile int* verr = &err;
 
-  if (warp < 8) {
-    int kb0 = 0;
-    for (int t = blockIdx.x; t < ntiles && !*verr; t += gridDim.x, kb0 += nk)
-      if (!gather_pairs<SW>(conv, (long long)(t / ntn) * TC_BM, a.M, kb0, nk, smA, empty, fulla)) *verr = 1;
-  } else if (warp == 8) {
+  if (warp < GW) {
+    if (!gather_pairs<SW, CP_SUBS>(conv, a.M, nk, ntn, ntiles, smA, empty, fulla)) *verr = 1;
+  } else if (warp == GW) {
     if (lane == 0) {
       int kb = 0;
       for (int t = blockIdx.x; t < ntiles && !*verr; t += gridDim.x)
@@ -580,7 +606,7 @@ __global__ void __launch_bounds__(CP_THREADS, 2)
           tma_2d(smB + s * B_STAGE, &tb, i * TC_BK, (t % ntn) * a.BN, &full[s]);
         }
     }
-  } else if (warp == 9) {
+  } else if (warp == GW + 1) {
     if (lane == 0) {
       int kb = 0, it = 0;
       for (int t = blockIdx.x; t < ntiles && !*verr; t += gridDim.x, it++) {
@@ -725,7 +751,7 @@ cudaError_t conv_pairs(const TcConvA& c, const CUtensorMap& tb, TcArgs a, int pa
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const int grid = (int)std::min<long long>(ntiles, (long long)nsm * per_sm);
-  kern<<<grid, CP_THREADS, smem, st>>>(tb, a, c, (int)ntn, (int)ntiles);
+  kern<<<grid, 64 * CP_SUBS + 192, smem, st>>>(tb, a, c, (int)ntn, (int)ntiles);
   return cudaGetLastError();
 }
 }  // namespace
