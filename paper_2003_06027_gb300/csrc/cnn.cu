@@ -651,10 +651,11 @@ cudaError_t im2col_n(const float* x, const fwi::ConvDims& d, long long ldn, uint
   return cudaGetLastError();
 }
 
-int gemm_blocks(long long tiles_per_split) {
-  // splits so that about two waves of CTAs cover the GPU's 152 SMs
-  return (int)std::max<long long>(1, (2 * 152 + tiles_per_split - 1) / tiles_per_split);
-}
+// Splits of a product of few tiles: as many as two CTAs for each of the 152 SMs hold,
+// in one wave (up to 96 columns) or two. One CTA more is a wave of its own: rounding
+// up gave 305 of them for the gradient of 64 x 576 weights at 128 x 256, batch 32 (286 us,
+// now 189), and 323 for 256 x 2304 at 16 x 32 (109 us, now 85).
+int gemm_splits(long long tiles) { return (int)std::max<long long>(1, 2 * 152 / tiles); }
 
 }  // namespace
 
@@ -783,9 +784,10 @@ fwi_status fwi_cnn_conv_backward(fwi_cnn* h, const float* x, int32_t C, int32_t 
   const long long ldn = fwi::round8(d.Npix);
   const int ldo = (int)fwi::round8(O);
   const int nchunk = (d.Npix + fwi::ACT_CHUNK - 1) / fwi::ACT_CHUNK;
-  // weight gradient split over pixel runs: about two waves of CTAs
-  const long long mt = (d.K9 + 127) / 128, nt = (O + 255) / 256;
-  const int S = fwi::tc_split_count(d.Npix, gemm_blocks(mt * nt));
+  // weight gradient split over pixel runs (the same runs whether its taps are gathered,
+  // 14 channels a tile, or come from a matrix, 128 taps)
+  const long long mt = (C + fwi::TC_WG_CH - 1) / fwi::TC_WG_CH, nt = (O + 255) / 256;
+  const int S = fwi::tc_split_count(d.Npix, gemm_splits(mt * nt));
   // stride-1 data gradient: dy seen as a [O][B][H][W] activation, convolved with the flipped weights
   fwi::ConvDims dd = d;
   dd.C = O;

@@ -43,7 +43,6 @@ constexpr int TC_BK = 64;  // one 128-byte swizzle row of BF16
 constexpr int TC_STAGES = 4;
 constexpr int TC_THREADS = 128;
 constexpr int A_STAGE = TC_BM * TC_BK * 2;  // 16 KB
-constexpr int TC_WG_CH = 14;                // channels per weight-gradient tile: 126 of its 128 rows
 constexpr int TC_WG_ROWS = 9 * TC_WG_CH;
 
 struct TcArgs {

@@ -8,6 +8,8 @@
 
 namespace fwi {
 
+constexpr int TC_WG_CH = 14;  // channels per weight-gradient tile: 126 of its 128 rows
+
 // out[split][n][m] = act(sum_{k in split} A[m][k] * B[n][k] + bias[n])
 //
 //   A: M rows of K BF16 values, row stride lda elements (K-major; lda % 8 == 0)
