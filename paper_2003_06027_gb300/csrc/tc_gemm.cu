@@ -44,6 +44,7 @@ constexpr int TC_STAGES = 4;
 constexpr int TC_THREADS = 128;
 constexpr int A_STAGE = TC_BM * TC_BK * 2;  // 16 KB
 constexpr int TC_WG_ROWS = 9 * TC_WG_CH;
+constexpr int SM_SMEM = 228 * 1024;  // shared memory of an SM (a CTA takes 1 KB more than it asks for)
 
 struct TcArgs {
   long long M;
@@ -55,6 +56,7 @@ struct TcArgs {
   int* status;
   uint32_t idesc;
   uint32_t tmem_cols;
+  int stages;  // of the shared-memory ring: fewer than TC_STAGES if all k-blocks fit (CONV 0)
 };
 
 // Shared-memory matrix descriptor of a K-major operand tile written by TMA with
@@ -412,7 +414,7 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
   const uint32_t raw = smem_u32(tc_smem_raw);
   unsigned char* smA = tc_smem_raw + ((1024u - (raw & 1023u)) & 1023u);
   const int B_STAGE = a.BN * TC_BK * 2;
-  unsigned char* smB = smA + TC_STAGES * A_STAGE;
+  unsigned char* smB = smA + (CONV ? TC_STAGES : a.stages) * A_STAGE;
   int2* tab = nullptr;
   if (CONV == 1) {  // after the stages: a.nkb k-blocks of (offset, tap bit) entries
     const int K9 = 9 * conv.C, len = a.nkb * TC_BK;
@@ -768,7 +770,8 @@ cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st) {
     if (g.wgrad && !tc_conv_pairs(c)) return cudaErrorInvalidValue;
   }
   if (g.M > 0x7fffff00LL || g.N > 0x7fffff00) return cudaErrorInvalidValue;
-  const int BN = std::min(256, (g.N + 15) / 16 * 16);
+  // columns shared evenly between the fewest tiles of at most 256 (288 as 2 x 144)
+  const int ntn = (g.N + 255) / 256, BN = ((g.N + ntn - 1) / ntn + 15) / 16 * 16;
   const long long nkb = tc_kblocks(g.K);
   const long long kbps = (nkb + g.splits - 1) / g.splits;
   const int splits = (int)((nkb + kbps - 1) / kbps);
@@ -807,7 +810,14 @@ cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st) {
       return conv_pairs(*g.conv, tb, a, pairs, st);
     }
   }
-  const int smem = TC_STAGES * (A_STAGE + BN * TC_BK * 2) + 1024 + (kind == 1 ? (int)nkb * TC_BK * 8 : 0);
+  // Products of few k-blocks (a strided layer's data gradient has one to four) are bound
+  // by their epilogue: with no more stages than k-blocks several CTAs share an SM and one
+  // tile's epilogue covers another's loads; as many as TMEM's 512 columns hold, so that
+  // no allocation waits. Batch of 32, four strided layers (288 columns also as 2 x 144
+  // instead of 256 + 32): 360 -> 258 us.
+  a.stages = kind == 0 ? (int)std::min<long long>(TC_STAGES, a.kbps) : TC_STAGES;
+  int smem = a.stages * (A_STAGE + BN * TC_BK * 2) + 1024 + (kind == 1 ? (int)nkb * TC_BK * 8 : 0);
+  if (kind == 0) smem = std::max(smem, (int)(SM_SMEM / (512 / a.tmem_cols + 1)));
   const dim3 grid((unsigned)((g.M + bm - 1) / bm), (unsigned)((g.N + BN - 1) / BN), (unsigned)splits);
   TcConvA c{};
   if (conv) c = *g.conv;
