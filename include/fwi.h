@@ -362,8 +362,8 @@ fwi_status fwi_forward_noalloc(const fwi_model *model, const fwi_sources *src,
  * sweep (recompute + adjoint + folds), [2] whole call. kernel_ms3: average
  * duration of one time step of [0] the recording forward step, [1] the storing
  * forward step of the recompute (with the checkpoint restores; per recomputed
- * step), [2] the adjoint step; 0 if none ran. Acoustic calls split the shots into up to 4
- * groups whose launches run concurrently on internal streams (forked from and
+ * step), [2] the adjoint step; 0 if none ran. Calls split the shots into up to 4
+ * groups (elastic: 2) whose launches run concurrently on internal streams (forked from and
  * joined to the call's stream), so one step is one launch per group, and the
  * step time includes launch gaps. launches: number of kernels the call
  * launched. After fwi_graph_status, the values of the last graph replay on

@@ -49,8 +49,8 @@ fwi_status fwi_cnn_destroy(fwi_cnn *h);
  * this handle gave up a bounded wait since the last check, else FWI_OK. */
 fwi_status fwi_cnn_check(fwi_cnn *h, void *cuda_stream);
 
-/* How the convolution GEMMs of the forward pass and of the stride-1 data
- * gradient get their tap operand: on != 0 (the default) gathers it from the
+/* How the convolution GEMMs (forward, stride-1 data gradients, weight gradients)
+ * get their tap operand: on != 0 (the default) gathers it from the
  * activations into the GEMM's shared-memory stages (no im2col matrix in device
  * memory); 0 builds the im2col matrix first and has TMA stage it. Both give the
  * same BF16 operand and the same results bit for bit. FWI_EINVAL if h is NULL. */

@@ -562,7 +562,7 @@ struct fwi_cnn {
   size_t ws_bytes = 0;
   int* status = nullptr;  // device status word of the GEMMs (timeout bit)
   double* red = nullptr;  // block partials of the loss reduction
-  bool gather = true;     // forward / stride-1 data-gradient GEMMs gather their tap operand (no im2col matrix)
+  bool gather = true;     // forward, stride-1 data- and weight-gradient GEMMs gather their tap operand (no im2col matrix)
 };
 
 namespace {
