@@ -56,6 +56,13 @@ fwi_status fwi_cnn_check(fwi_cnn *h, void *cuda_stream);
  * same BF16 operand and the same results bit for bit. FWI_EINVAL if h is NULL. */
 fwi_status fwi_cnn_set_conv_gather(fwi_cnn *h, int32_t on);
 
+/* Self-test of the GEMMs' bounded waits: from now on the MMA issuer of every CTA
+ * of h's products gives up after `kblocks` 64-wide k-blocks (< 0: never, the
+ * default), so that the other roles' waits for the stages it would have freed run
+ * out (1 s). The products write NaN, leave nothing in flight and release what they
+ * hold; fwi_cnn_check then returns FWI_ETIMEOUT. FWI_EINVAL if h is NULL. */
+fwi_status fwi_cnn_selftest_issue_limit(fwi_cnn *h, int32_t kblocks);
+
 /* The tensor-core GEMM itself: out[n][m] = act(sum_k A[m][k] B[n][k] + bias[n]).
  * A: M rows of K BF16 values, row stride lda; B: N rows of K BF16 values, row
  * stride ldb (lda, ldb multiples of 8 and >= K; A, B 16-byte aligned).

@@ -563,6 +563,7 @@ struct fwi_cnn {
   int* status = nullptr;  // device status word of the GEMMs (timeout bit)
   double* red = nullptr;  // block partials of the loss reduction
   bool gather = true;     // forward, stride-1 data- and weight-gradient GEMMs gather their tap operand (no im2col matrix)
+  int issue_limit = -1;   // self-test of the GEMMs' bounded waits (TcGemm::issue_limit)
 };
 
 namespace {
@@ -708,6 +709,12 @@ fwi_status fwi_cnn_set_conv_gather(fwi_cnn* h, int32_t on) {
   return FWI_OK;
 }
 
+fwi_status fwi_cnn_selftest_issue_limit(fwi_cnn* h, int32_t kblocks) {
+  if (!h) return fwi::host_fail(FWI_EINVAL, "h must not be NULL");
+  h->issue_limit = kblocks < 0 ? -1 : kblocks;
+  return FWI_OK;
+}
+
 fwi_status fwi_cnn_gemm_bt(fwi_cnn* h, const uint16_t* A, int64_t lda, const uint16_t* B, int64_t ldb, int64_t M,
                            int32_t N, int64_t K, float* out, int64_t ldo, const float* bias, int32_t relu,
                            int32_t splits, void* stream) {
@@ -726,6 +733,7 @@ fwi_status fwi_cnn_gemm_bt(fwi_cnn* h, const uint16_t* A, int64_t lda, const uin
   }
   fwi::TcGemm g{A, lda, B, ldb, M, N, K, dst, ldo, (long long)N * ldo, S > 1 ? nullptr : bias, S > 1 ? 0 : relu, S,
                 h->status};
+  g.issue_limit = h->issue_limit;
   CNN_CK(fwi::tc_gemm(g, st), "tcgen05 GEMM");
   if (S > 1) {
     if (bias || relu) return fwi::host_fail(FWI_EINVAL, "bias / relu need splits == 1");
@@ -767,6 +775,7 @@ fwi_status fwi_cnn_conv_forward(fwi_cnn* h, const float* x, int32_t C, int32_t B
   if (!gather) CNN_CK(im2col_t(x, d, ldk, colT, st), "im2col");
   fwi::TcGemm g{gather ? nullptr : colT, ldk, Wp, ldk, d.Npix, O, d.K9, y, d.Npix, 0, bias, relu, 1, h->status,
                 gather ? &ca : nullptr};
+  g.issue_limit = h->issue_limit;
   CNN_CK(fwi::tc_gemm(g, st), "conv forward GEMM");
   return FWI_OK;
 }
@@ -831,6 +840,7 @@ fwi_status fwi_cnn_conv_backward(fwi_cnn* h, const float* x, int32_t C, int32_t 
     if (!h->gather) CNN_CK(im2col_t(dy, dd, ldf, colb, st), "im2col of dy");
     fwi::TcGemm g{h->gather ? nullptr : colb, ldf, Wf, ldf, dd.Npix, C, dd.K9, dx, dd.Npix, 0, nullptr, 0, 1,
                   h->status, h->gather ? &ca : nullptr};
+    g.issue_limit = h->issue_limit;
     CNN_CK(fwi::tc_gemm(g, st), "conv data-gradient GEMM");
   } else if (dx) {
     // dcol[k][pix] = sum_o dyT[pix][o] W[o][k], then the col2im gather
@@ -840,6 +850,7 @@ fwi_status fwi_cnn_conv_backward(fwi_cnn* h, const float* x, int32_t C, int32_t 
     fwi::k_wprep<<<blocks_for((long long)O * d.K9), 256, 0, st>>>(w_bf16, O, d.K9, 0, ldo, nullptr, Wt);
     CNN_CK(cudaGetLastError(), "weight layout");
     fwi::TcGemm g{colb, ldo, Wt, ldo, d.Npix, d.K9, O, dcol, d.Npix, 0, nullptr, 0, 1, h->status};
+    g.issue_limit = h->issue_limit;
     CNN_CK(fwi::tc_gemm(g, st), "conv data-gradient GEMM");
     auto c2i = sw == 1 ? fwi::k_col2im<1> : sw == 2 ? fwi::k_col2im<2> : fwi::k_col2im<0>;
     c2i<<<(unsigned)std::min<long long>(((long long)C * B * H + 7) / 8, 152 * 64), 256, 0, st>>>(dcol, d, dx);
@@ -849,6 +860,7 @@ fwi_status fwi_cnn_conv_backward(fwi_cnn* h, const float* x, int32_t C, int32_t 
   if (!wg) CNN_CK(im2col_n(x, d, ldn, colb, st), "im2col");
   fwi::TcGemm g{wg ? nullptr : colb, ldn, dyb, ldn, d.K9, O, d.Npix, S > 1 ? part : dw, d.K9, (long long)O * d.K9,
                 nullptr, 0, S, h->status, wg ? &cx : nullptr, wg};
+  g.issue_limit = h->issue_limit;
   CNN_CK(fwi::tc_gemm(g, st), "conv weight-gradient GEMM");
   if (S > 1) {
     fwi::k_split_sum<<<blocks_for((long long)O * d.K9), 256, 0, st>>>(part, S, (long long)O * d.K9, dw);

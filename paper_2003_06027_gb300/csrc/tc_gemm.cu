@@ -23,7 +23,8 @@
 // waits for; warp 8 loads B by TMA, warp 9 issues the MMAs.
 // Every mbarrier wait is bounded (2^24 polls or 1 s); a wait that gives up
 // records a timeout in the status word, the tile is written as NaN, and the
-// CTA frees its TMEM and exits.
+// CTA waits (again bounded) for its own TMA copies and MMAs still in flight,
+// frees its TMEM and exits (drain).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -57,6 +58,7 @@ struct TcArgs {
   uint32_t idesc;
   uint32_t tmem_cols;
   int stages;  // of the shared-memory ring: fewer than TC_STAGES if all k-blocks fit (CONV 0)
+  uint32_t issue_limit;  // k-blocks after which a CTA's MMA issuer gives up (self-test; no limit: 2^32 - 1)
 };
 
 // Shared-memory matrix descriptor of a K-major operand tile written by TMA with
@@ -115,6 +117,20 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 }
 __device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, uint32_t n) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(n) : "memory");
+}
+// After a wait that ran out, once every role of the CTA has left its loop: bounded waits
+// for what the CTA may still have in flight, so that no copy or MMA writes after it has
+// exited or freed its TMEM. The MMA issuer commits what it has issued onto a barrier of
+// its own; of the `armed` k-blocks that the TMA producer asked for, each stage's last
+// one completes that stage's phase (armed - 1 - s) / TC_STAGES.
+__device__ __forceinline__ void drain(bool issuer, bool producer, uint64_t* full, int armed, uint64_t* issued) {
+  if (issuer) {
+    tc_commit(issued);
+    mbar_wait(issued, 0);
+  }
+  if (producer)
+    for (int s = 0; s < TC_STAGES && s < armed; s++) mbar_wait(&full[s], (uint32_t)((armed - 1 - s) / TC_STAGES) & 1u);
+  __syncwarp();
 }
 __device__ __forceinline__ uint32_t mulhi_div(uint32_t n, unsigned long long m, uint32_t s) {
   return (uint32_t)(((unsigned long long)n * m) >> s);
@@ -407,9 +423,9 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
               const TcConvA conv) {
   using R = TcRoles<CONV>;
   extern __shared__ unsigned char tc_smem_raw[];
-  __shared__ uint64_t full[TC_STAGES], empty[TC_STAGES], fulla[TC_STAGES], accb;
+  __shared__ uint64_t full[TC_STAGES], empty[TC_STAGES], fulla[TC_STAGES], accb, issued;
   __shared__ uint32_t tmem_slot;
-  __shared__ int err;
+  __shared__ int err, armed;
   // the swizzled tiles need 1024-byte alignment
   const uint32_t raw = smem_u32(tc_smem_raw);
   unsigned char* smA = tc_smem_raw + ((1024u - (raw & 1023u)) & 1023u);
@@ -439,7 +455,8 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
       mbar_init(&fulla[s], R::ARRIVE);  // CONV: one arrival per gathering warp of the stage
     }
     mbar_init(&accb, 1);
-    err = 0;
+    mbar_init(&issued, 1);
+    err = armed = 0;
     fence_mbar_init();
   }
   if (warp == 0) {
@@ -455,7 +472,8 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
 
   if (warp == R::B_WARP && lane == 0) {
     // TMA producer: A and B, or B alone when A is gathered
-    for (int i = 0; i < nk; i++) {
+    int i = 0;
+    for (; i < nk; i++) {
       const int s = i % TC_STAGES;
       const uint32_t ph = (uint32_t)(i / TC_STAGES) & 1u;
       if (!mbar_wait(&empty[s], ph ^ 1u)) {
@@ -466,13 +484,15 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
       if (!CONV) tma_2d(smA + s * A_STAGE, &ta, (kb0 + i) * TC_BK, (int)m0, &full[s]);
       tma_2d(smB + s * B_STAGE, &tb, (kb0 + i) * TC_BK, n0, &full[s]);
     }
+    armed = i;
   } else if (warp == R::MMA_WARP && lane == 0) {
     // MMA issuer
     for (int i = 0; i < nk; i++) {
       const int s = i % TC_STAGES;
       const uint32_t ph = (uint32_t)(i / TC_STAGES) & 1u;
-      if (!mbar_wait(&full[s], ph) || (CONV && !mbar_wait(&fulla[s], ph))) {
+      if ((uint32_t)i >= a.issue_limit || !mbar_wait(&full[s], ph) || (CONV && !mbar_wait(&fulla[s], ph))) {
         err = 1;
+        __threadfence_block();  // seen by the epilogue with the commit below
         break;
       }
       tc_fence_after();
@@ -516,7 +536,7 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
     const bool ok = mbar_wait(&accb, 0);
     tc_fence_after();
     __syncwarp();
-    if (!ok && lane == 0) atomicOr(a.status, ST_TIMEOUT);
+    if (!ok) err = 1;
     const int row = warp * 32 + lane;
     const long long m = m0 + row;
     float* outp = a.out + (long long)blockIdx.z * a.split_stride;
@@ -540,7 +560,11 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
   }
   tc_fence_before();
   __syncthreads();
-  if (err && threadIdx.x == 0) atomicOr(a.status, ST_TIMEOUT);
+  if (err) {
+    if (threadIdx.x == 0) atomicOr(a.status, ST_TIMEOUT);
+    drain(warp == R::MMA_WARP && lane == 0, warp == R::B_WARP && lane == 0, full, armed, &issued);
+    __syncthreads();
+  }
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols) : "memory");
 }
@@ -558,9 +582,9 @@ __global__ void __launch_bounds__(64 * CP_SUBS + 192, 2)
     k_conv_pairs(const __grid_constant__ CUtensorMap tb, const TcArgs a, const TcConvA conv, int ntn, int ntiles) {
   constexpr int GW = 2 * CP_SUBS;  // gathering warps
   extern __shared__ unsigned char tc_smem_raw[];
-  __shared__ uint64_t full[TC_STAGES], empty[TC_STAGES], fulla[TC_STAGES], accf[2], acce[2];
+  __shared__ uint64_t full[TC_STAGES], empty[TC_STAGES], fulla[TC_STAGES], accf[2], acce[2], issued;
   __shared__ uint32_t tmem_slot;
-  __shared__ int err;
+  __shared__ int err, armed;
   const uint32_t raw = smem_u32(tc_smem_raw);
   unsigned char* smA = tc_smem_raw + ((1024u - (raw & 1023u)) & 1023u);
   const int B_STAGE = a.BN * TC_BK * 2;
@@ -576,7 +600,8 @@ __global__ void __launch_bounds__(64 * CP_SUBS + 192, 2)
       mbar_init(&accf[s], 1);
       mbar_init(&acce[s], 4);  // one arrival per epilogue warp
     }
-    err = 0;
+    mbar_init(&issued, 1);
+    err = armed = 0;
     fence_mbar_init();
   }
   if (warp == 0) {
@@ -606,6 +631,7 @@ __global__ void __launch_bounds__(64 * CP_SUBS + 192, 2)
           mbar_expect_tx(&full[s], (uint32_t)B_STAGE);
           tma_2d(smB + s * B_STAGE, &tb, i * TC_BK, (t % ntn) * a.BN, &full[s]);
         }
+      armed = kb;
     }
   } else if (warp == GW + 1) {
     if (lane == 0) {
@@ -620,8 +646,9 @@ __global__ void __launch_bounds__(64 * CP_SUBS + 192, 2)
         for (int i = 0; i < nk; i++, kb++) {
           const int s = kb % TC_STAGES;
           const uint32_t ph = (uint32_t)(kb / TC_STAGES) & 1u;
-          if (!mbar_wait(&full[s], ph) || !mbar_wait(&fulla[s], ph)) {
+          if ((uint32_t)kb >= a.issue_limit || !mbar_wait(&full[s], ph) || !mbar_wait(&fulla[s], ph)) {
             *verr = 1;
+            __threadfence_block();  // seen by the epilogue with the commit below
             break;
           }
           tc_fence_after();
@@ -672,12 +699,11 @@ __global__ void __launch_bounds__(64 * CP_SUBS + 192, 2)
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  if (err && threadIdx.x == 0) {
-    atomicOr(a.status, ST_TIMEOUT);
-    // copies and MMAs still in flight land before the CTA exits (bounded)
-    for (int s = 0; s < TC_STAGES; s++) mbar_wait(&full[s], 0) || mbar_wait(&full[s], 1);
+  if (err) {
+    if (threadIdx.x == 0) atomicOr(a.status, ST_TIMEOUT);
+    drain(warp == GW + 1 && lane == 0, warp == GW && lane == 0, full, armed, &issued);
+    __syncthreads();
   }
-  __syncthreads();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols) : "memory");
 }
@@ -789,6 +815,7 @@ cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st) {
   a.bias = g.bias;
   a.relu = g.relu;
   a.status = g.status;
+  a.issue_limit = g.issue_limit < 0 ? ~0u : (uint32_t)g.issue_limit;
   // instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
   // (bits 7-9 = 1, 10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
   a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);

@@ -58,6 +58,9 @@ struct TcGemm {
   // with conv: the weight gradient's product instead, A[m][k] = tap m of pixel k
   // (M = 9 C taps, K = B Ho Wo pixels); needs tc_conv_pairs(*conv) != 0
   bool wgrad = false;
+  // self-test of the bounded waits: each CTA's MMA issuer gives up after this many
+  // k-blocks (< 0: never), so that the waits for the stages it would free run out
+  int issue_limit = -1;
 };
 
 // Whether the gather can take a layer's outputs in pairs: horizontal stride 1 (or

@@ -50,6 +50,7 @@ def _lib():
         L.fwi_cnn_destroy.argtypes = [P]
         L.fwi_cnn_check.argtypes = [P, P]
         L.fwi_cnn_set_conv_gather.argtypes = [P, i32]
+        L.fwi_cnn_selftest_issue_limit.argtypes = [P, i32]
         L.fwi_cnn_gemm_bt.argtypes = [P, P, i64, P, i64, i64, i32, i64, P, i64, P, i32, i32, P]
         L.fwi_cnn_conv_forward.argtypes = [P, P, i32, i32, i32, i32, P, P, i32, i32, i32, i32, P, P]
         L.fwi_cnn_conv_backward.argtypes = [P, P, i32, i32, i32, i32, P, i32, i32, i32, i32, P, P, P, P, P, P]
@@ -95,6 +96,11 @@ class Handle:
         """Gather the convolution GEMMs' tap operand in the GEMM (default) or
         build the im2col matrix first (fwi_cnn_set_conv_gather)."""
         _chk(_lib().fwi_cnn_set_conv_gather(self.h, int(bool(on))))
+
+    def selftest_issue_limit(self, kblocks: int = -1):
+        """Have the GEMMs' MMA issuers give up after `kblocks` k-blocks (< 0: never),
+        so that their bounded waits run out (fwi_cnn_selftest_issue_limit)."""
+        _chk(_lib().fwi_cnn_selftest_issue_limit(self.h, int(kblocks)))
 
     def __del__(self):
         try:
