@@ -549,9 +549,10 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
         for (int j = 0; j < 16; j++) {
           const int n = n0 + c0 + j;
           if (n < a.N) {
-            float v = bad ? __int_as_float(0x7fc00000) : __uint_as_float(r[j]);
+            float v = __uint_as_float(r[j]);
             if (a.bias) v += a.bias[n];
             if (a.relu) v = fmaxf(v, 0.f);
+            if (bad) v = __int_as_float(0x7fc00000);  // last: the ReLU's maximum would drop it
             outp[(long long)n * a.ldo + m] = v;
           }
         }
@@ -683,9 +684,10 @@ __global__ void __launch_bounds__(64 * CP_SUBS + 192, 2)
           for (int j = 0; j < 16; j++) {
             const int n = n0 + c0 + j;
             if (n < a.N) {
-              float v = bad ? __int_as_float(0x7fc00000) : __uint_as_float(r[j]);
+              float v = __uint_as_float(r[j]);
               if (a.bias) v += a.bias[n];
               if (a.relu) v = fmaxf(v, 0.f);
+              if (bad) v = __int_as_float(0x7fc00000);  // last: the ReLU's maximum would drop it
               a.out[(long long)n * a.ldo + m] = v;
             }
           }

@@ -54,3 +54,16 @@ def test_wait_that_runs_out(fwi_lib, kind, limit):
     h.selftest_issue_limit(-1)
     assert torch.equal(run(h), want)
     h.check()
+
+
+@pytest.mark.parametrize("kind", ["pairs1", "pairs2", "table", "im2col", "gemm", "wgrad"])
+def test_output_of_a_timed_out_product_is_nan(fwi_lib, kind):
+    # with the ReLU too, whose maximum of NaN and 0 is 0
+    from paper_2003_06027_gb300 import fwi
+    from paper_2003_06027_gb300 import learned as L
+
+    h, run = L.Handle(0), _product(kind)
+    h.selftest_issue_limit(3)
+    assert bool(torch.isnan(run(h)).all())
+    with pytest.raises(fwi.FwiError, match="timed out"):
+        h.check()
