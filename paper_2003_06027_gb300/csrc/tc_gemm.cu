@@ -31,6 +31,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 
 #include "fwi_internal.cuh"
 #include "tc_gemm.h"
@@ -765,6 +766,48 @@ int tc_split_count(long long K, int want) {
 }
 
 namespace {
+// Per device: the SM count, and the dynamic shared memory that each kernel may be
+// launched with, raised once to all that a CTA can have. The attribute belongs to the
+// kernel, not to a launch: set to each launch's own size, one thread's smaller product
+// lowers it between another thread's set and launch, which then fails.
+enum { K_TMA, K_TABLE, K_WG1, K_WG2, K_PAIRS1, K_PAIRS2, TC_KERNELS };
+struct TcDev {
+  bool ready = false;
+  int sms = 0, smem[TC_KERNELS];
+};
+std::mutex g_tc_mu;
+TcDev g_tc[64];
+
+template <typename K>
+cudaError_t tc_setup(K kern, int optin, int* smem) {
+  cudaFuncAttributes at;
+  cudaError_t e = cudaFuncGetAttributes(&at, kern);
+  if (e != cudaSuccess) return e;
+  *smem = optin - (int)at.sharedSizeBytes;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem);
+}
+
+cudaError_t tc_device(const TcDev** out) {
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(g_tc_mu);
+  TcDev& d = g_tc[dev];
+  *out = &d;
+  if (d.ready) return cudaSuccess;
+  if ((e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+  if ((e = tc_setup(k_tc_gemm<0>, optin, &d.smem[K_TMA])) != cudaSuccess) return e;
+  if ((e = tc_setup(k_tc_gemm<1>, optin, &d.smem[K_TABLE])) != cudaSuccess) return e;
+  if ((e = tc_setup(k_tc_gemm<2>, optin, &d.smem[K_WG1])) != cudaSuccess) return e;
+  if ((e = tc_setup(k_tc_gemm<3>, optin, &d.smem[K_WG2])) != cudaSuccess) return e;
+  if ((e = tc_setup(k_conv_pairs<1>, optin, &d.smem[K_PAIRS1])) != cudaSuccess) return e;
+  if ((e = tc_setup(k_conv_pairs<2>, optin, &d.smem[K_PAIRS2])) != cudaSuccess) return e;
+  d.ready = true;
+  return cudaSuccess;
+}
+
 // Persistent launch of k_conv_pairs: two CTAs per SM while two stage rings fit in
 // shared memory (227 KB) and four accumulators in TMEM (512 columns).
 cudaError_t conv_pairs(const TcConvA& c, const CUtensorMap& tb, TcArgs a, int pairs, cudaStream_t st) {
@@ -773,13 +816,12 @@ cudaError_t conv_pairs(const TcConvA& c, const CUtensorMap& tb, TcArgs a, int pa
   const int per_sm = smem <= 112 * 1024 && a.tmem_cols <= 256 ? 2 : 1;
   const long long ntn = (a.N + a.BN - 1) / a.BN, ntiles = (a.M + TC_BM - 1) / TC_BM * ntn;
   if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-  int dev = 0, nsm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  auto kern = pairs == 1 ? k_conv_pairs<1> : k_conv_pairs<2>;
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const TcDev* dev;
+  const cudaError_t e = tc_device(&dev);
   if (e != cudaSuccess) return e;
-  const int grid = (int)std::min<long long>(ntiles, (long long)nsm * per_sm);
+  if (smem > dev->smem[pairs == 1 ? K_PAIRS1 : K_PAIRS2]) return cudaErrorInvalidValue;
+  auto kern = pairs == 1 ? k_conv_pairs<1> : k_conv_pairs<2>;
+  const int grid = (int)std::min<long long>(ntiles, (long long)dev->sms * per_sm);
   kern<<<grid, 64 * CP_SUBS + 192, smem, st>>>(tb, a, c, (int)ntn, (int)ntiles);
   return cudaGetLastError();
 }
@@ -851,8 +893,10 @@ cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st) {
   TcConvA c{};
   if (conv) c = *g.conv;
   auto kern = kind == 0 ? k_tc_gemm<0> : kind == 1 ? k_tc_gemm<1> : kind == 2 ? k_tc_gemm<2> : k_tc_gemm<3>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const TcDev* dev;
+  const cudaError_t e = tc_device(&dev);
   if (e != cudaSuccess) return e;
+  if (smem > dev->smem[K_TMA + kind]) return cudaErrorInvalidValue;
   kern<<<grid, conv ? TcRoles<1>::THREADS : TcRoles<0>::THREADS, smem, st>>>(ta, tb, a, c);
   return cudaGetLastError();
 }
