@@ -1258,6 +1258,7 @@ unsigned long long g_inited = 0;  // bit per device
 // and store), adjoint, and the multi-instance forward sweep / recompute and adjoint
 int g_grid_fwd[64][FWD_SHAPES][2][2][4], g_grid_adj[64][2], g_grid_fwd_m[64][2][2], g_grid_adj_m[64][2];
 int g_grid_adj_lap[64][2];  // the c^2 Laplacian operator
+int g_sms[64];
 
 template <typename K>
 cudaError_t setup_kernel(K k, int smem, int* grid, int threads = NTHREADS) {
@@ -1320,6 +1321,7 @@ cudaError_t ensure_init(int* dev_out) {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(g_init_mu);
   if (g_inited & (1ull << dev)) return cudaSuccess;
+  if ((e = cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   if ((e = setup_order<2>(dev, 0)) != cudaSuccess) return e;
   if ((e = setup_order<4>(dev, 1)) != cudaSuccess) return e;
   g_inited |= 1ull << dev;
@@ -1378,6 +1380,29 @@ cudaError_t acu_make_maps(AcuMaps* maps, const Grid& g, int S, float* u_pair, co
     if (!tma_host::encode(&maps->u[sp], u_pair, 3, d3, s3, b3)) return cudaErrorInvalidValue;
     if (!tma_host::encode(&maps->m[sp], const_cast<float*>(mh), 2, d2, s2, b2)) return cudaErrorInvalidValue;
   }
+  return cudaSuccess;
+}
+
+// Tile height of the forward steps (record, store) of S shots, launched as groups of at
+// most Sg. 32-row tiles need the fewest instructions per cell; 8-row tiles (four times as
+// many CTAs, each a quarter of the latency) are faster while a launch's all fit the
+// resident CTAs, so that each step is one wave of dependent launches. Per step, 8 against
+// 32 rows, 4th order, recording (2 groups) / storing (4 groups):
+//   one shot of 100 x 100 (15 tiles of 32 rows)  4.6 / -      against  4.9 / -
+//   16 shots of 128 x 256 (480)                  7.0 /  8.0   against  7.4 / 11.5
+//   20 (600; 1200 of 1216 places a group)        8.0 /  9.0   against  7.8 / 12.1
+//   24 (720; the recording groups do not fit)   12.3 / 10.3   against  8.2 / 12.5
+//   12 in one group (360, does not fit)         10.2          against  6.9
+// Storing groups fit up to 1216 tiles, but from some 850 on the four launches no longer
+// run beside each other: 840 tiles 11.7 against 12.9 us, 960 12.8 against 13.1 (8th order
+// 13.0 against 11.7), 1200 15.9 against 14.7; hence the second bound, 5 tiles per SM.
+cudaError_t acu_fwd_rows(int S, int Sg, const Grid& g, int N, bool record, bool store, bool lap, int* rows) {
+  int dev;
+  const cudaError_t e = ensure_init(&dev);
+  if (e != cudaSuccess) return e;
+  const int v = (record ? 1 : 0) + (store ? 2 : 0);
+  const long long fit = g_grid_fwd[dev][0][lap ? 1 : 0][N == 2 ? 0 : 1][v];
+  *rows = (long long)Sg * g.ntx * ((g.Nz + 7) / 8) <= fit && (long long)S * g.ntx * g.ntz < 5 * g_sms[dev] ? 8 : 32;
   return cudaSuccess;
 }
 

@@ -21,6 +21,7 @@
 #include "fwi_internal.cuh"
 
 namespace fwi {
+cudaError_t acu_fwd_rows(int S, int Sg, const Grid& g, int N, bool record, bool store, bool lap, int* rows);
 cudaError_t launch_acu_fwd(const AcuStep& p, const AcuMaps& maps, bool record, bool store, int rows, bool lap,
                            cudaStream_t st);
 void acu_coef_pairs(AcuCoef& c);
@@ -435,9 +436,12 @@ fwi_status join(fwi_ctx* ctx, const Groups& gr, cudaStream_t main) {
   return FWI_OK;
 }
 
-// Tile height of the context's acoustic forward steps.
-int fwd_rows(const fwi_ctx* ctx, int S, const Grid& g) {
-  return ctx->fwd_tile_rows ? ctx->fwd_tile_rows : acu_fwd_rows(S, g);
+// Tile height of the context's acoustic forward steps (record, store) in the groups gr.
+fwi_status fwd_rows(const fwi_ctx* ctx, const Plan& P, int N, const Groups& gr, bool record, bool store, bool lap,
+                    int* rows) {
+  *rows = ctx->fwd_tile_rows;
+  if (*rows == 0) CK(acu_fwd_rows(P.S, gr.n[0], P.g, N, record, store, lap, rows));
+  return FWI_OK;
 }
 
 // The step parameters of one group: shots [s0, s0 + Sg). Per-shot arrays are
@@ -676,7 +680,8 @@ fwi_status fwi_forward(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* Sv, 
   if ((v = fork(ctx, gr, st)) != FWI_OK) return v;
   const size_t fieldf = (size_t)P.S * P.g.slice;
   const float lscale = (float)((double)dt * dt / ((double)M->dx * M->dz));
-  const int rows = fwd_rows(ctx, P.S, P.g);
+  int rows;
+  if ((v = fwd_rows(ctx, P, p.N, gr, true, false, lap, &rows)) != FWI_OK) return v;
   for (int n = 0; n < nt; n++) {
     set_fwd_state(P, p, n);
     for (int g = 0; g < gr.G; g++) {
@@ -784,7 +789,10 @@ fwi_status acu_misfit_grad(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* 
   if ((v = make_groups(ctx, P.S, st, grs, ctx->fwd_groups ? ctx->fwd_groups : STORE_GROUPS)) != FWI_OK) return v;
   if ((v = make_groups(ctx, P.S, st, gra, ctx->adj_groups ? ctx->adj_groups : ADJ_GROUPS)) != FWI_OK) return v;
   const size_t sl = (size_t)P.g.slice;
-  const int rows = fwd_rows(ctx, P.S, P.g);
+  int rows_rec, rows_keep, rows_store;  // of recording steps, those that store too, recomputed ones
+  if ((v = fwd_rows(ctx, P, p.N, gr, true, false, lap, &rows_rec)) != FWI_OK) return v;
+  if ((v = fwd_rows(ctx, P, p.N, grs, true, true, lap, &rows_keep)) != FWI_OK) return v;
+  if ((v = fwd_rows(ctx, P, p.N, grs, false, true, lap, &rows_store)) != FWI_OK) return v;
 
   // forward sweep with a full-state checkpoint at the start of every segment
   // but the last: the sweep itself keeps the last segment's fluxes (recording
@@ -818,7 +826,8 @@ fwi_status acu_misfit_grad(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* 
       p.slot_pz = lap ? nullptr : p.slot_px + field;
     }
     for (int g = 0; g < sg->G; g++) {
-      LK(1, launch_acu_fwd(group_view(p, P, sg->s0[g], sg->n[g]), maps, true, keep, rows, lap, sg->st[g]));
+      LK(1, launch_acu_fwd(group_view(p, P, sg->s0[g], sg->n[g]), maps, true, keep, keep ? rows_keep : rows_rec, lap,
+                           sg->st[g]));
       if (P.L > 0)
         LK(1, launch_line_inject(sg->n[g], P.L, n, nt, lscale, P.stf + (size_t)sg->s0[g] * nt * P.L,
                                  P.line_cell + 2 * sg->s0[g], P.u + ((n + 1) & 1) * field + sg->s0[g] * sl, P.g,
@@ -857,7 +866,8 @@ fwi_status acu_misfit_grad(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* 
         p.slot_px = P.slot + (size_t)(n - n0) * P.slot_fields * field;
         p.slot_pz = lap ? nullptr : p.slot_px + field;
         for (int g = 0; g < grs.G; g++) {
-          LK(1, launch_acu_fwd(group_view(p, P, grs.s0[g], grs.n[g]), maps, false, true, rows, lap, grs.st[g]));
+          LK(1, launch_acu_fwd(group_view(p, P, grs.s0[g], grs.n[g]), maps, false, true, rows_store, lap,
+                             grs.st[g]));
           if (P.L > 0)
             LK(1, launch_line_inject(grs.n[g], P.L, n, nt, lscale, P.stf + (size_t)grs.s0[g] * nt * P.L,
                                      P.line_cell + 2 * grs.s0[g], P.u + ((n + 1) & 1) * field + grs.s0[g] * sl, P.g,

@@ -110,14 +110,6 @@ struct EleMaps {
 };
 
 constexpr int FWD_SHAPES = 3;  // forward tile heights: 8, 32 and 64 rows
-// Tile height of the forward steps of S shots. 32-row tiles need the fewest
-// instructions per cell; while a step has fewer than about five of them per SM,
-// 8-row tiles (four times as many CTAs, each a quarter of the latency) are faster:
-// 4.3 against 4.7 us per step for one shot of 100 x 100 (15 tiles of 32 rows), 6.8
-// against 7.2 us for 16 shots of 128 x 256 (480), but 18.2 against 15.1 us for 16
-// shots of 201 x 601 (1584).
-inline int acu_fwd_rows(int S, const Grid& g) { return (long long)S * g.ntx * g.ntz < 760 ? 8 : 32; }
-
 // TMA descriptors of one call: the wavefield pair [2][S] (forward), the
 // half-coefficient field m/2, and the adjoint operand pairs [2][S].
 struct AcuMaps {

@@ -35,6 +35,7 @@
 #include "fwi_internal.cuh"
 
 namespace fwi {
+cudaError_t acu_fwd_rows(int S, int Sg, const Grid& g, int N, bool record, bool store, bool lap, int* rows);
 cudaError_t launch_acu_fwd(const AcuStep& p, const AcuMaps& maps, bool record, bool store, int rows, bool lap,
                            cudaStream_t st);
 cudaError_t acu_make_maps(AcuMaps* maps, const Grid& g, int S, float* u_pair, const float* mh);
@@ -252,6 +253,8 @@ extern "C" fwi_status fwi_forward_noalloc(const fwi_model* M, const fwi_sources*
   p.dz = M->dz;
   AcuMaps maps;
   NA_CK(acu_make_maps(&maps, g, S, p.u, p.mh));
+  int rows;
+  NA_CK(acu_fwd_rows(S, S, g, p.N, true, false, false, &rows));
   for (int n = 0; n < nt; n++) {
     p.n = n;
     p.cur = n & 1;
@@ -259,7 +262,7 @@ extern "C" fwi_status fwi_forward_noalloc(const fwi_model* M, const fwi_sources*
     p.psix_out = psix[(n + 1) & 1];
     p.psiz_in = psiz[n & 1];
     p.psiz_out = psiz[(n + 1) & 1];
-    NA_CK(launch_acu_fwd(p, maps, true, false, acu_fwd_rows(S, g), false, st));
+    NA_CK(launch_acu_fwd(p, maps, true, false, rows, false, st));
   }
   const long long ns = (long long)S * nrec * nt;
   if (ns > 0) NA_CK(launch_finite_check(seis, ns, status, st));
