@@ -1406,6 +1406,22 @@ cudaError_t acu_fwd_rows(int S, int Sg, const Grid& g, int N, bool record, bool 
   return cudaSuccess;
 }
 
+// Launches that make one recording step of S shots by default: two, or three where two
+// would each take a second, nearly empty wave and three fit the resident CTAs (3 per SM:
+// 912 to 1368 tiles). Per step with 2 / 3 / 4 groups: 16 shots of 306 x 310 (1152 tiles)
+// 13.1 / 9.9 / 10.1 us, 40 of 128 x 256 at 8th order without layers (1200) 12.4 / 11.1 /
+// 11.5 (the scalar kernel that this replaced, in four groups, 10.3); beyond, 16 of 201 x
+// 601 (1584) 13.7 / 13.5 / 13.5, at 8th order 15.1 / 15.1 / 15.4, 100 of 128 x 256 (3000)
+// 27.5 / 27.9 / 28.6.
+cudaError_t acu_fwd_groups(int S, const Grid& g, int N, bool lap, int* groups) {
+  int dev;
+  const cudaError_t e = ensure_init(&dev);
+  if (e != cudaSuccess) return e;
+  const long long fit = g_grid_fwd[dev][1][lap ? 1 : 0][N == 2 ? 0 : 1][1], per = (long long)g.ntx * g.ntz;
+  *groups = (S + 1) / 2 * per > fit && (S + 2) / 3 * per <= fit ? 3 : 2;
+  return cudaSuccess;
+}
+
 // Forward step on tiles of `rows` rows (8, 32 or 64).
 cudaError_t launch_acu_fwd(const AcuStep& p_in, const AcuMaps& maps, bool record, bool store, int rows, bool lap,
                            cudaStream_t st) {

@@ -21,6 +21,7 @@
 #include "fwi_internal.cuh"
 
 namespace fwi {
+cudaError_t acu_fwd_groups(int S, const Grid& g, int N, bool lap, int* groups);
 cudaError_t acu_fwd_rows(int S, int Sg, const Grid& g, int N, bool record, bool store, bool lap, int* rows);
 cudaError_t launch_acu_fwd(const AcuStep& p, const AcuMaps& maps, bool record, bool store, int rows, bool lap,
                            cudaStream_t st);
@@ -388,10 +389,11 @@ fwi_status finish_status(fwi_ctx* ctx, const Plan& P, cudaStream_t st) { return 
 // fill them. Everything that couples shots (misfit, folds, source gradients)
 // runs on the call's stream after a join.
 constexpr int MAX_GROUPS = 4;
-// Groups by default, measured on 16 shots of the 201 x 601 problem: the recording
-// forward step 15.1 us with 2 groups against 15.6 with 4, the storing one (which
-// runs more CTAs per SM) 16.6 against 14.8, the adjoint step 25.0 against 25.9.
-constexpr int FWD_GROUPS = 2, STORE_GROUPS = 4, ADJ_GROUPS = 2;
+// Groups by default (the recording step's: acu_fwd_groups), measured on 16 shots of the
+// 201 x 601 problem: the recording forward step 15.1 us with 2 groups against 15.6 with 4,
+// the storing one (which runs more CTAs per SM) 16.6 against 14.8, the adjoint step 25.0
+// against 25.9.
+constexpr int STORE_GROUPS = 4, ADJ_GROUPS = 2;
 
 struct Groups {
   int G = 1;
@@ -675,7 +677,9 @@ fwi_status fwi_forward(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* Sv, 
   CK(acu_make_maps(&maps, P.g, P.S, P.u, P.m));
   ensure_events(ctx, 0);
   Groups gr;
-  if ((v = make_groups(ctx, P.S, st, gr, ctx->fwd_groups ? ctx->fwd_groups : FWD_GROUPS)) != FWI_OK) return v;
+  int G = ctx->fwd_groups;
+  if (G == 0) CK(acu_fwd_groups(P.S, P.g, p.N, lap, &G));
+  if ((v = make_groups(ctx, P.S, st, gr, G)) != FWI_OK) return v;
   CK(cudaEventRecord(ctx->ev[0], st));
   if ((v = fork(ctx, gr, st)) != FWI_OK) return v;
   const size_t fieldf = (size_t)P.S * P.g.slice;
@@ -785,7 +789,9 @@ fwi_status acu_misfit_grad(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* 
   ensure_events(ctx, P.nseg);
 
   Groups gr, grs, gra;  // forward sweep, recomputed segments, adjoint
-  if ((v = make_groups(ctx, P.S, st, gr, ctx->fwd_groups ? ctx->fwd_groups : FWD_GROUPS)) != FWI_OK) return v;
+  int G = ctx->fwd_groups;
+  if (G == 0) CK(acu_fwd_groups(P.S, P.g, p.N, lap, &G));
+  if ((v = make_groups(ctx, P.S, st, gr, G)) != FWI_OK) return v;
   if ((v = make_groups(ctx, P.S, st, grs, ctx->fwd_groups ? ctx->fwd_groups : STORE_GROUPS)) != FWI_OK) return v;
   if ((v = make_groups(ctx, P.S, st, gra, ctx->adj_groups ? ctx->adj_groups : ADJ_GROUPS)) != FWI_OK) return v;
   const size_t sl = (size_t)P.g.slice;

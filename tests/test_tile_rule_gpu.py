@@ -57,3 +57,26 @@ def test_mixed_heights_give_the_same_bits(fwi_lib, nz, nx, S):
             fwi.set_tile_shape(0)
     for a, b in zip(*out):
         assert a is None and b is None or torch.equal(a, b)
+
+
+# 1200 and 1152 tiles: two launches a step would each take a second wave, three fit
+@pytest.mark.parametrize("nz,nx,S,order,npml", [(192, 320, 40, 8, 0), (192, 320, 40, 4, 0), (306, 310, 16, 4, 32)])
+def test_default_groups_are_not_slower_than_four(fwi_lib, nz, nx, S, order, npml):
+    import torch
+
+    from paper_2003_06027_gb300 import fwi
+
+    d = synth.random_acoustic(S, nz, nx, 400, S, order, npml, nrec=6)
+    cu = lambda a: torch.as_tensor(np.ascontiguousarray(a)).cuda()
+    kw, args, best, seis = fwi.problem_kwargs(d), [cu(d[k]) for k in ("c", "stf", "x0", "rec_iz", "rec_ix")], {}, {}
+    try:
+        for _ in range(5):
+            for groups in (0, 4):
+                fwi.set_shot_groups(groups, 0)
+                seis[groups] = fwi.forward(*args, **kw)
+                best[groups] = min(best.get(groups, 1e9), fwi.last_timing().fwd_step_ms)
+    finally:
+        fwi.set_shot_groups(0, 0)
+    assert torch.equal(seis[0], seis[4])
+    # two groups took 1.08 to 1.3 times as long as four at these sizes
+    assert best[0] <= 1.05 * best[4]
