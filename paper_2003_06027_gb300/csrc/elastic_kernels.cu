@@ -1315,6 +1315,16 @@ cudaError_t ela_kernels_init() {
   return ela_ensure_init(&dev);
 }
 
+// CTAs of any step kernel of the order that are resident at once.
+cudaError_t ela_resident(int N, int* ctas) {
+  int dev;
+  const cudaError_t e = ela_ensure_init(&dev);
+  if (e != cudaSuccess) return e;
+  const int* gr = g_ela_grid[dev][N == 2 ? 0 : 1];
+  *ctas = *std::min_element(gr, gr + 8);
+  return cudaSuccess;
+}
+
 // TMA descriptors for a call over the five forward fields f = (vx, vz, sxx,
 // szz, sxz) and, if a is not null, the five adjoint fields in the same order;
 // each field is [S][rows][pitch].

@@ -23,6 +23,7 @@
 
 namespace fwi {
 cudaError_t ela_make_maps(EleMaps* maps, const Grid& g, int S, float* const* f, float* const* a);
+cudaError_t ela_resident(int N, int* ctas);
 cudaError_t launch_ela_vel(const EleStep& p, const EleMaps& m, bool record, bool store, cudaStream_t st);
 cudaError_t launch_ela_str(const EleStep& p, const EleMaps& m, bool store, cudaStream_t st);
 cudaError_t launch_ela_adj(const EleStep& p, const EleMaps& m, cudaStream_t st);
@@ -308,9 +309,11 @@ fwi_status ela_prepare(fwi_ctx* ctx, EPlan& P, const fwi_model* M, const fwi_sou
 // the next are filled by the other (every elastic field is per shot). Per step
 // (forward / recompute / adjoint pair), one group against two, 300 x 800: 32 shots
 // 185/208/334 -> 161/184/321 us, 8 shots 48/55/92 -> 42/49/82, 4 shots 28/31/49 ->
-// 24/28/39; three or four groups give no more, and below one tile per resident CTA
-// (3 on each of 152 SMs) the launches only wait for each other: 4 shots of 200 x 400
-// (288 tiles) 18.5/20/27 -> 20/23/26.5.
+// 24/28/39; three or four groups give no more, and below one tile per resident CTA the
+// launches only wait for each other: 4 shots of 200 x 400 (288 tiles) 18.5/20/27 ->
+// 20/23/26.5. That is 3 CTAs on each SM at 4th order (4 shots of 200 x 550, 360 tiles:
+// 18.0/19.2/27.3 -> 18.7/20.4/26.8) and 2 at 8th (22.0/23.8/35.1 -> 17.5/19.1/24.1; 24 of
+// 60 x 120, 288 tiles: 15.9/16.6/23.3 -> 16.2/17.0/23.3).
 struct EGroups {
   int G = 1;
   int s0[2] = {0, 0}, n[2] = {0, 0};
@@ -318,7 +321,9 @@ struct EGroups {
 };
 
 fwi_status ela_groups(fwi_ctx* ctx, const EPlan& P, cudaStream_t main, EGroups& gr) {
-  gr.G = P.S >= 2 && (long long)P.S * P.g.ntx * P.g.ntz > 3 * 152 ? 2 : 1;
+  int resident;
+  ECK(ela_resident(P.N, &resident));
+  gr.G = P.S >= 2 && (long long)P.S * P.g.ntx * P.g.ntz > resident ? 2 : 1;
   for (int g = 0, s0 = 0; g < gr.G; g++) {
     gr.n[g] = P.S / gr.G + (g < P.S % gr.G ? 1 : 0);
     gr.s0[g] = s0;
