@@ -494,14 +494,12 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
     armed = i;
   } else if (warp == R::MMA_WARP && lane == 0) {
     // MMA issuer
-    for (int i = 0; i < nk; i++) {
+    const int ni = (int)min((uint32_t)nk, a.issue_limit);
+    int i = 0;
+    for (; i < ni; i++) {
       const int s = i % TC_STAGES;
       const uint32_t ph = (uint32_t)(i / TC_STAGES) & 1u;
-      if ((uint32_t)i >= a.issue_limit || !mbar_wait(&full[s], ph) || (CONV && !mbar_wait(&fulla[s], ph))) {
-        err = 1;
-        __threadfence_block();  // seen by the epilogue with the commit below
-        break;
-      }
+      if (!mbar_wait(&full[s], ph) || (CONV && !mbar_wait(&fulla[s], ph))) break;
       tc_fence_after();
       const uint64_t ad = R::WG ? sdesc_sw128_mn(smem_u32(smA + s * A_STAGE), A_STAGE / 2)
                                 : sdesc_sw128(smem_u32(smA + s * A_STAGE));
@@ -510,6 +508,10 @@ __global__ void __launch_bounds__(TcRoles<CONV>::THREADS, TcRoles<CONV>::CTAS)
       for (int kk = 0; kk < TC_BK / 16; kk++)  // 16 values of K per MMA: 32 bytes, or 16 rows of an M-major A
         tc_mma(tmem, ad + (R::WG ? 128 : 2) * kk, bd + 2 * kk, a.idesc, (uint32_t)(i | kk));
       tc_commit(&empty[s]);
+    }
+    if (i < nk) {
+      err = 1;
+      __threadfence_block();  // seen by the epilogue with the commit
     }
     tc_commit(&accb);
   } else if (R::WG && (int)threadIdx.x < R::GATHER) {
@@ -652,14 +654,12 @@ __global__ void __launch_bounds__(64 * CP_SUBS + 192, 2)
           break;
         }
         tc_fence_after();
-        for (int i = 0; i < nk; i++, kb++) {
+        const int ni = (int)min((uint32_t)nk, a.issue_limit - (uint32_t)kb);
+        int i = 0;
+        for (; i < ni; i++, kb++) {
           const int s = kb % TC_STAGES;
           const uint32_t ph = (uint32_t)(kb / TC_STAGES) & 1u;
-          if ((uint32_t)kb >= a.issue_limit || !mbar_wait(&full[s], ph) || !mbar_wait(&fulla[s], ph)) {
-            *verr = 1;
-            __threadfence_block();  // seen by the epilogue with the commit below
-            break;
-          }
+          if (!mbar_wait(&full[s], ph) || !mbar_wait(&fulla[s], ph)) break;
           tc_fence_after();
           const uint64_t ad = sdesc_sw128(smem_u32(smA + s * A_STAGE));
           const uint64_t bd = sdesc_sw128(smem_u32(smB + s * B_STAGE));
@@ -667,6 +667,10 @@ __global__ void __launch_bounds__(64 * CP_SUBS + 192, 2)
           for (int kk = 0; kk < TC_BK / 16; kk++)
             tc_mma(tmem + b * acc_stride, ad + 2 * kk, bd + 2 * kk, a.idesc, (uint32_t)(i | kk));
           tc_commit(&empty[s]);
+        }
+        if (i < nk) {
+          *verr = 1;
+          __threadfence_block();  // seen by the epilogue with the commit
         }
         tc_commit(&accf[b]);
       }
