@@ -435,12 +435,25 @@ __global__ void k_wflip(const uint16_t* __restrict__ w, int O, int C, int ldf, u
   }
 }
 
-// out[e] = sum over splits s (in order) of part[s * n + e]
+// out[e] = sum over splits s (in order) of part[s * n + e]: eight loads in flight, and the
+// remainder's four, two and one together too (a loop unrolled by eight took it one by one:
+// 25781 x 44 outputs of four splits 21.6 -> 24.1 us for the whole product, now 21.0)
+template <int U>
+__device__ __forceinline__ void split_add(const float* p, long long n, float& s) {
+  float v[U];
+#pragma unroll
+  for (int u = 0; u < U; u++) v[u] = __ldg(p + u * n);
+#pragma unroll
+  for (int u = 0; u < U; u++) s += v[u];
+}
 __global__ void k_split_sum(const float* __restrict__ part, int splits, long long n, float* __restrict__ out) {
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+    const float* p = part + e;
     float s = 0.f;
-#pragma unroll 8
-    for (int k = 0; k < splits; k++) s += __ldg(part + (long long)k * n + e);
+    for (int k = splits; k >= 8; k -= 8, p += 8 * n) split_add<8>(p, n, s);
+    if (splits & 4) split_add<4>(p, n, s), p += 4 * n;
+    if (splits & 2) split_add<2>(p, n, s), p += 2 * n;
+    if (splits & 1) split_add<1>(p, n, s);
     out[e] = s;
   }
 }
