@@ -460,20 +460,22 @@ __global__ void k_split_sum(const float* __restrict__ part, int splits, long lon
 
 // Input row `row` (= cb H + r) of x feeds output rows 2 row and 2 row + 1 of y
 // (cb 2H + 2r = 2 row). Items are V consecutive input values of a row (W = V Wv),
-// numbered through all rows so that short rows fill the warps too; each is written
-// as two 2V-value stores. V = 2 needs even rows and 16-byte aligned y (8-byte x);
-// V = 1 takes the rest (y 8-byte aligned; the launcher checks). A block per row
-// with a thread per value kept a quarter to a half of its lanes busy (238 us for
-// the three layers of a batch of 32, this 97; backward 238 -> 95).
+// numbered through all rows so that short rows fill the warps too (item e reads x from
+// V e on); each is written as two 2V-value stores. V = 2 needs even rows and 16-byte
+// aligned y (8-byte x); V = 1 takes the rest (y 8-byte aligned; the launcher checks).
+// Offsets fit 32 bits (the launcher's limit on y). A block per row with a thread per
+// value kept a quarter to a half of its lanes busy (235 us for the three layers of a
+// batch of 32, this 102; backward 235 -> 92). With 64-bit offsets and 256 threads always,
+// calls of a few thousand values had become slower (100 x 100: 1.37 -> 1.55 us, 32
+// channels of 64 x 128 2.07 -> 2.23; now 1.37 and 1.90; 150 planes of 45 x 348 backward
+// 5.66 -> 5.86, now 3.91).
 template <int V>
-__global__ void __launch_bounds__(256) k_upsample2(const float* __restrict__ x, long long items, FastDiv fWv, int W,
+__global__ void __launch_bounds__(256) k_upsample2(const float* __restrict__ x, uint32_t items, FastDiv fWv, uint32_t W,
                                                    float* __restrict__ y) {
-  for (long long e = blockIdx.x * 256LL + threadIdx.x; e < items; e += gridDim.x * 256LL) {
-    const long long row = fWv.div((uint32_t)e);
-    const int s = V * (int)(e - row * fWv.d);
-    const float* xr = x + row * W + s;
-    float* y0 = y + 4 * row * W + 2 * s;
-    float* y1 = y0 + 2LL * W;
+  for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < items; e += gridDim.x * blockDim.x) {
+    const float* xr = x + V * e;
+    float* y0 = y + 2 * (V * e + fWv.div(e) * W);
+    float* y1 = y0 + 2 * W;
     if (V == 2) {
       const float2 v = __ldg(reinterpret_cast<const float2*>(xr));
       const float4 o = make_float4(v.x, v.x, v.y, v.y);
@@ -490,14 +492,12 @@ __global__ void __launch_bounds__(256) k_upsample2(const float* __restrict__ x, 
 // dx[row][s] = (dy[2 row][2s] + dy[2 row][2s + 1]) + (dy[2 row + 1][2s] + dy[2 row + 1][2s + 1]),
 // items as in k_upsample2 (dy 16- or 8-byte aligned).
 template <int V>
-__global__ void __launch_bounds__(256) k_upsample2_back(const float* __restrict__ dy, long long items, FastDiv fWv,
-                                                        int W, float* __restrict__ dx) {
-  for (long long e = blockIdx.x * 256LL + threadIdx.x; e < items; e += gridDim.x * 256LL) {
-    const long long row = fWv.div((uint32_t)e);
-    const int s = V * (int)(e - row * fWv.d);
-    const float* d0 = dy + 4 * row * W + 2 * s;
-    const float* d1 = d0 + 2LL * W;
-    float* o = dx + row * W + s;
+__global__ void __launch_bounds__(256) k_upsample2_back(const float* __restrict__ dy, uint32_t items, FastDiv fWv,
+                                                        uint32_t W, float* __restrict__ dx) {
+  for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < items; e += gridDim.x * blockDim.x) {
+    const float* d0 = dy + 2 * (V * e + fWv.div(e) * W);
+    const float* d1 = d0 + 2 * W;
+    float* o = dx + V * e;
     if (V == 2) {
       const float4 a = __ldg(reinterpret_cast<const float4*>(d0)), b = __ldg(reinterpret_cast<const float4*>(d1));
       *reinterpret_cast<float2*>(o) = make_float2((a.x + a.y) + (b.x + b.y), (a.z + a.w) + (b.z + b.w));
@@ -663,6 +663,14 @@ cudaError_t im2col_n(const float* x, const fwi::ConvDims& d, long long ldn, uint
     fwi::k_im2col_n<<<dim3((d.Npix + 1023) / 1024, d.K9), 256, 0, st>>>(x, d, ldn, col);
   }
   return cudaGetLastError();
+}
+
+// Threads per block of the upsampling kernels: 256, less while there is not a block for
+// each of the 152 SMs.
+int up_threads(long long items) {
+  int nt = 256;
+  while (nt > 64 && items < 152 * nt) nt /= 2;
+  return nt;
 }
 
 // Splits of a product of few tiles: as many as two CTAs for each of the 152 SMs hold,
@@ -891,8 +899,9 @@ fwi_status fwi_cnn_upsample2(const float* x, int32_t C, int32_t B, int32_t H, in
   const int Wv = pairs ? W / 2 : W;
   const long long items = (long long)C * B * H * Wv;
   auto up = pairs ? fwi::k_upsample2<2> : fwi::k_upsample2<1>;
-  up<<<(unsigned)std::min<long long>((items + 255) / 256, 152 * 32), 256, 0, (cudaStream_t)stream>>>(
-      x, items, fwi::FastDiv((uint32_t)Wv), W, y);
+  const int nt = up_threads(items);
+  up<<<(unsigned)std::min<long long>((items + nt - 1) / nt, 152 * 8192 / nt), nt, 0, (cudaStream_t)stream>>>(
+      x, (uint32_t)items, fwi::FastDiv((uint32_t)Wv), (uint32_t)W, y);
   CNN_CK(cudaGetLastError(), "upsample");
   return FWI_OK;
 }
@@ -907,8 +916,9 @@ fwi_status fwi_cnn_upsample2_backward(const float* dy, int32_t C, int32_t B, int
   const int Wv = pairs ? W / 2 : W;
   const long long items = (long long)C * B * H * Wv;
   auto back = pairs ? fwi::k_upsample2_back<2> : fwi::k_upsample2_back<1>;
-  back<<<(unsigned)std::min<long long>((items + 255) / 256, 152 * 32), 256, 0, (cudaStream_t)stream>>>(
-      dy, items, fwi::FastDiv((uint32_t)Wv), W, dx);
+  const int nt = up_threads(items);
+  back<<<(unsigned)std::min<long long>((items + nt - 1) / nt, 152 * 8192 / nt), nt, 0, (cudaStream_t)stream>>>(
+      dy, (uint32_t)items, fwi::FastDiv((uint32_t)Wv), (uint32_t)W, dx);
   CNN_CK(cudaGetLastError(), "upsample backward");
   return FWI_OK;
 }
