@@ -819,17 +819,33 @@ cudaError_t tc_device(const TcDev** out) {
   return cudaSuccess;
 }
 
-// Persistent launch of k_conv_pairs: two CTAs per SM while two stage rings fit in
-// shared memory (227 KB) and four accumulators in TMEM (512 columns).
-cudaError_t conv_pairs(const TcConvA& c, const CUtensorMap& tb, TcArgs a, int pairs, cudaStream_t st) {
-  const int smem = TC_STAGES * (A_STAGE + a.BN * TC_BK * 2) + 1024;
+// Launch of k_conv_pairs: its tiles, and two CTAs per SM while two stage rings fit in
+// shared memory (227 KB) and four accumulators in TMEM (512 columns), else one.
+int pairs_smem(const TcArgs& a) { return TC_STAGES * (A_STAGE + a.BN * TC_BK * 2) + 1024; }
+int pairs_per_sm(const TcArgs& a) { return pairs_smem(a) <= 112 * 1024 && a.tmem_cols <= 128 ? 2 : 1; }
+long long pairs_tiles(const TcArgs& a) { return (a.M + TC_BM - 1) / TC_BM * ((a.N + a.BN - 1) / a.BN); }
+
+// Whether a layer of C channels whose outputs come in pairs goes to k_conv_pairs rather
+// than to the tap table. A run of 8 channels is four load rounds one after the other in two
+// warps, so the persistent kernel pays where a CTA has several tiles, whose runs the warp
+// groups share, or a tile has enough runs; with one tile a CTA the table, all of whose
+// threads load all taps of a k-block at once, has the shorter chain. us, pairs / table:
+//   100 tiles, 16 columns (96): 8 channels 6.3 / 5.5 (10.6 / 10.0), 9: 8.0 / 7.5 (12.4 / 11.7),
+//     24: 7.3 / 7.3 (11.7 / 11.6), 40: 8.7 / 8.7 (12.7 / 12.7); 64 tiles of 64 columns, 128 channels: 17.2 / 20.3
+//   280 tiles, 16 columns, two CTAs an SM: 8: 7.5 / 7.1, 9: 10.0 / 9.3, 12: 8.1 / 8.4, 24: 8.3 / 9.8
+//   380 tiles, 144 columns: 8: 28.1 / 30.9, 9: 30.7 / 33.0, 24: 29.7 / 36.5
+// With fewer than 8 channels most of a run would be padding.
+bool pairs_pay(const TcArgs& a, int C, int sms) {
+  const long long t = pairs_tiles(a);
+  if (t <= sms) return C >= 32;
+  return C >= (t <= (long long)sms * pairs_per_sm(a) ? 12 : 8);
+}
+
+cudaError_t conv_pairs(const TcConvA& c, const CUtensorMap& tb, TcArgs a, int pairs, const TcDev* dev, cudaStream_t st) {
+  const int smem = pairs_smem(a), per_sm = pairs_per_sm(a);
+  const long long ntn = (a.N + a.BN - 1) / a.BN, ntiles = pairs_tiles(a);
   a.tmem_cols *= 2;
-  const int per_sm = smem <= 112 * 1024 && a.tmem_cols <= 256 ? 2 : 1;
-  const long long ntn = (a.N + a.BN - 1) / a.BN, ntiles = (a.M + TC_BM - 1) / TC_BM * ntn;
   if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-  const TcDev* dev;
-  const cudaError_t e = tc_device(&dev);
-  if (e != cudaSuccess) return e;
   if (smem > dev->smem[pairs == 1 ? K_PAIRS1 : K_PAIRS2]) return cudaErrorInvalidValue;
   auto kern = pairs == 1 ? k_conv_pairs<1> : k_conv_pairs<2>;
   const int grid = (int)std::min<long long>(ntiles, (long long)dev->sms * per_sm);
@@ -879,6 +895,9 @@ cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st) {
   if (!encode_bf16_sw128(&tb, g.B, g.K, g.N, g.ldb, BN)) return cudaErrorInvalidValue;
   if (conv) ta = tb;  // unused: A is gathered
   else if (!encode_bf16_sw128(&ta, g.A, g.K, g.M, g.lda, TC_BM)) return cudaErrorInvalidValue;
+  const TcDev* dev;
+  const cudaError_t e = tc_device(&dev);
+  if (e != cudaSuccess) return e;
   int kind = 0, bm = TC_BM;
   if (conv) {
     const int pairs = tc_conv_pairs(*g.conv);
@@ -887,9 +906,8 @@ cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st) {
       kind = 1 + pairs;
       bm = TC_WG_ROWS;
       a.idesc |= 1u << 15;  // A is M-major
-    } else if (pairs && g.conv->C >= 8 && splits == 1) {
-      // (with fewer than 8 channels most of a run of 8 would be padding)
-      return conv_pairs(*g.conv, tb, a, pairs, st);
+    } else if (pairs && splits == 1 && pairs_pay(a, g.conv->C, dev->sms)) {
+      return conv_pairs(*g.conv, tb, a, pairs, dev, st);
     }
   }
   // Products of few k-blocks (a strided layer's data gradient has one to four) are bound
@@ -904,9 +922,6 @@ cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st) {
   TcConvA c{};
   if (conv) c = *g.conv;
   auto kern = kind == 0 ? k_tc_gemm<0> : kind == 1 ? k_tc_gemm<1> : kind == 2 ? k_tc_gemm<2> : k_tc_gemm<3>;
-  const TcDev* dev;
-  const cudaError_t e = tc_device(&dev);
-  if (e != cudaSuccess) return e;
   if (smem > dev->smem[K_TMA + kind]) return cudaErrorInvalidValue;
   kern<<<grid, conv ? TcRoles<1>::THREADS : TcRoles<0>::THREADS, smem, st>>>(ta, tb, a, c);
   return cudaGetLastError();
