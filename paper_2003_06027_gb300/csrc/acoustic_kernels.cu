@@ -269,7 +269,7 @@ __device__ __forceinline__ void cta_sum3(float v[3], float* red) {
   __syncthreads();
 }
 
-// Issue the TMA fetches of tile t (8 R rows) into one buffer (one elected thread).
+// Issue the TMA fetches of tile t (R TY rows) into one buffer (one elected thread).
 // plane0: the pair plane of this launch's first shot.
 template <int R, int TY>
 __device__ __forceinline__ void fetch_tile(const CUtensorMap* fmap, const CUtensorMap* mmap, const Grid& g, int plane0,
@@ -1256,7 +1256,8 @@ std::mutex g_init_mu;
 unsigned long long g_inited = 0;  // bit per device
 // resident-CTA grids: forward variants (rows per thread, operator, order, record
 // and store), adjoint, and the multi-instance forward sweep / recompute and adjoint
-int g_grid_fwd[64][FWD_SHAPES][2][2][4], g_grid_adj[64][2], g_grid_fwd_m[64][2][2], g_grid_adj_m[64][2];
+constexpr int FWD_VARIANTS = 3;
+int g_grid_fwd[64][FWD_SHAPES][2][2][FWD_VARIANTS], g_grid_adj[64][2], g_grid_fwd_m[64][2][2], g_grid_adj_m[64][2];
 int g_grid_adj_lap[64][2];  // the c^2 Laplacian operator
 int g_sms[64];
 
@@ -1275,14 +1276,14 @@ cudaError_t setup_kernel(K k, int smem, int* grid, int threads = NTHREADS) {
 constexpr int FWD_SMEM_M = (int)(FWD_SMEM_MAIN<2, 16> + sizeof(AcuStep));
 constexpr int ADJ_SMEM_M = (int)(ADJ_SMEM_MAIN + sizeof(AcuStep));
 
-// The forward kernel of one variant.
+// The forward kernel of one variant: recording, recording and storing, storing.
 template <int N, int R, int TY, bool LAP>
 auto fwd_kernel(int v) {
-  return v == 0   ? acu_fwd_step<N, false, false, false, R, TY, LAP>
-         : v == 1 ? acu_fwd_step<N, true, false, false, R, TY, LAP>
-         : v == 2 ? acu_fwd_step<N, false, true, false, R, TY, LAP>
-                  : acu_fwd_step<N, true, true, false, R, TY, LAP>;
+  return v == 0   ? acu_fwd_step<N, true, false, false, R, TY, LAP>
+         : v == 1 ? acu_fwd_step<N, true, true, false, R, TY, LAP>
+                  : acu_fwd_step<N, false, true, false, R, TY, LAP>;
 }
+int fwd_variant(bool record, bool store) { return !store ? 0 : record ? 1 : 2; }
 // Tile heights 8, 32 and 64: one, two and four rows per thread.
 template <int N, bool LAP>
 auto fwd_kernel(int shape, int v) {
@@ -1299,7 +1300,7 @@ cudaError_t setup_order(int dev, int o) {
   const int as = (int)sizeof(AdjSmem);
   cudaError_t e;
   for (int sp = 0; sp < FWD_SHAPES; sp++)
-    for (int v = 0; v < 4; v++) {
+    for (int v = 0; v < FWD_VARIANTS; v++) {
       const int fs = (int)fwd_smem(sp);
       if ((e = setup_kernel(fwd_kernel<N, false>(sp, v), fs, &g_grid_fwd[dev][sp][0][o][v], fwd_threads(sp))) != cudaSuccess) return e;
       if ((e = setup_kernel(fwd_kernel<N, true>(sp, v), fs, &g_grid_fwd[dev][sp][1][o][v], fwd_threads(sp))) != cudaSuccess) return e;
@@ -1400,7 +1401,7 @@ cudaError_t acu_fwd_rows(int S, int Sg, const Grid& g, int N, bool record, bool 
   int dev;
   const cudaError_t e = ensure_init(&dev);
   if (e != cudaSuccess) return e;
-  const int v = (record ? 1 : 0) + (store ? 2 : 0);
+  const int v = fwd_variant(record, store);
   const long long fit = g_grid_fwd[dev][0][lap ? 1 : 0][N == 2 ? 0 : 1][v];
   *rows = (long long)Sg * g.ntx * ((g.Nz + 7) / 8) <= fit && (long long)S * g.ntx * g.ntz < 5 * g_sms[dev] ? 8 : 32;
   return cudaSuccess;
@@ -1417,7 +1418,7 @@ cudaError_t acu_fwd_groups(int S, const Grid& g, int N, bool lap, int* groups) {
   int dev;
   const cudaError_t e = ensure_init(&dev);
   if (e != cudaSuccess) return e;
-  const long long fit = g_grid_fwd[dev][1][lap ? 1 : 0][N == 2 ? 0 : 1][1], per = (long long)g.ntx * g.ntz;
+  const long long fit = g_grid_fwd[dev][1][lap ? 1 : 0][N == 2 ? 0 : 1][fwd_variant(true, false)], per = (long long)g.ntx * g.ntz;
   *groups = (S + 1) / 2 * per > fit && (S + 2) / 3 * per <= fit ? 3 : 2;
   return cudaSuccess;
 }
@@ -1428,7 +1429,7 @@ cudaError_t launch_acu_fwd(const AcuStep& p_in, const AcuMaps& maps, bool record
   int dev;
   cudaError_t e = ensure_init(&dev);
   if (e != cudaSuccess) return e;
-  const int v = (record ? 1 : 0) + (store ? 2 : 0);
+  const int v = fwd_variant(record, store);
   const int o = p_in.N == 2 ? 0 : 1;
   const int sp = rows == 64 ? 2 : rows == 32 ? 1 : 0;
   const AcuCoef cf = coef_of(p_in);
@@ -1485,18 +1486,9 @@ cudaError_t launch_acu_adj(const AcuStep& p, const AcuMaps& maps, cudaStream_t s
   const AcuCoef cf = coef_of(p);
   BatchArgs nb;
   memset(&nb, 0, sizeof nb);
-  if (lap) {
-    if (p.N == 2)
-      return launch_step(acu_adj_step<2, false, true>, p.ntiles, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
-    else
-      return launch_step(acu_adj_step<4, false, true>, p.ntiles, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
-    return cudaGetLastError();
-  }
-  if (p.N == 2)
-    return launch_step(acu_adj_step<2, false>, p.ntiles, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
-  else
-    return launch_step(acu_adj_step<4, false>, p.ntiles, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
-  return cudaGetLastError();
+  auto k = p.N == 2 ? (lap ? acu_adj_step<2, false, true> : acu_adj_step<2, false>)
+                    : (lap ? acu_adj_step<4, false, true> : acu_adj_step<4, false>);
+  return launch_step(k, p.ntiles, grid, NTHREADS, smem, st, maps.lx, maps.lz, maps.hx, maps.hz, maps.m[1], p, cf, nb);
 }
 
 // Multi-instance adjoint step b.n over the tiles of instances [0, b.n_active).
@@ -1510,9 +1502,8 @@ cudaError_t launch_acu_adj_batch(const BatchArgs& b, const AcuCoef& cf, int N, c
   memset(&none, 0, sizeof none);
   AcuStep p0;
   memset(&p0, 0, sizeof p0);
-  if (N == 2) return launch_step(acu_adj_step<2, true>, b.ntiles, grid, NTHREADS, ADJ_SMEM_M, st, none, none, none, none, none, p0, cf, b);
-  else return launch_step(acu_adj_step<4, true>, b.ntiles, grid, NTHREADS, ADJ_SMEM_M, st, none, none, none, none, none, p0, cf, b);
-  return cudaGetLastError();
+  auto k = N == 2 ? acu_adj_step<2, true> : acu_adj_step<4, true>;
+  return launch_step(k, b.ntiles, grid, NTHREADS, ADJ_SMEM_M, st, none, none, none, none, none, p0, cf, b);
 }
 
 }  // namespace fwi
