@@ -63,9 +63,14 @@ constexpr int XS_BYTES = TILE_Z * UW * 4;  // 10240: adjoint x operand tile
 // The 32-row tile runs 3 CTAs per SM with the CPML operands held in registers, or
 // 4 without (PRE): the recording step measured 15.1 against 16.2 us, the storing
 // one, which has the flux stores to cover, 16.1 against 14.8 us (16 shots of 201 x
-// 601). The 8-row tile (8 CTAs) and the 64-row one (2) hold them.
-__host__ __device__ constexpr bool fwd_pre(int R, bool store) { return R != 2 || !store; }
-__host__ __device__ constexpr int fwd_ctas(int R, bool store) { return R == 1 ? 8 : R == 4 ? 2 : fwd_pre(R, store) ? 3 : 4; }
+// 601). Without layers there is nothing to hold, and the recording step runs 4 too
+// (per step, 3 -> 4 CTAs: 40 shots of 192 x 320, 1200 tiles, at 8th order 11.1 -> 10.1 us,
+// at 4th 9.0 -> 8.4; 100 shots 25.3 -> 23.6 and 20.0 -> 18.9; 60 of 370 x 374, 4320 tiles,
+// 32.2 -> 30.8 and 26.1 -> 25.4), but not where fields stream from memory (128 of 265 x
+// 665, 12 672 tiles: 86.8 -> 87.2 and 72.7 -> 74.7). The 8-row tile (8 CTAs) and the
+// 64-row one (2) hold them.
+__host__ __device__ constexpr bool fwd_pre(int R, bool store, bool layers) { return R != 2 || (!store && layers); }
+__host__ __device__ constexpr int fwd_ctas(int R, bool pre) { return R == 1 ? 8 : R == 4 ? 2 : pre ? 3 : 4; }
 template <int R, int TY>
 struct FwdGeo {
   static constexpr int NT = 16 * TY;          // threads
@@ -391,12 +396,11 @@ __device__ __forceinline__ void batch_load_step(const BatchArgs& b, int i, AcuSt
 // u^{n+1} = 2u^n - u^{n-1} + m dt^2 (D-q + zeta) + dt^2 w g(t_n) with m = c^2 at
 // the cell, and STORE keeps r = dt^2 (D-q + zeta) at the cells (the operand of
 // its gradient correlation dJ/dm = sum_n lambda_{n+1} r^n) instead of the fluxes.
-template <int N, bool RECORD, bool STORE, bool MULTI, int R, int TY, bool LAP = false>
-__global__ void __launch_bounds__(16 * TY, fwd_ctas(R, STORE))
+template <int N, bool RECORD, bool STORE, bool MULTI, int R, int TY, bool LAP = false, bool PRE = fwd_pre(R, STORE, true)>
+__global__ void __launch_bounds__(16 * TY, fwd_ctas(R, PRE))
     acu_fwd_step(const __grid_constant__ CUtensorMap tmap_u, const __grid_constant__ CUtensorMap tmap_m,
                  const __grid_constant__ AcuStep p0, const __grid_constant__ AcuCoef cf, const BatchArgs b) {
   static_assert(!LAP || !MULTI, "the Laplacian operator runs on single-instance launches");
-  constexpr bool PRE = fwd_pre(R, STORE);
   constexpr int NT = 16 * TY, TZ = FwdGeo<R, TY>::TZ, WR = R + 2 * N - 1;  // rows of a z stencil window
   extern __shared__ __align__(128) unsigned char smem_raw[];
   FwdSmemT<R, TY>& sh = *reinterpret_cast<FwdSmemT<R, TY>*>(smem_raw);
@@ -1256,7 +1260,7 @@ std::mutex g_init_mu;
 unsigned long long g_inited = 0;  // bit per device
 // resident-CTA grids: forward variants (rows per thread, operator, order, record
 // and store), adjoint, and the multi-instance forward sweep / recompute and adjoint
-constexpr int FWD_VARIANTS = 3;
+constexpr int FWD_VARIANTS = 4;
 int g_grid_fwd[64][FWD_SHAPES][2][2][FWD_VARIANTS], g_grid_adj[64][2], g_grid_fwd_m[64][2][2], g_grid_adj_m[64][2];
 int g_grid_adj_lap[64][2];  // the c^2 Laplacian operator
 int g_sms[64];
@@ -1276,14 +1280,19 @@ cudaError_t setup_kernel(K k, int smem, int* grid, int threads = NTHREADS) {
 constexpr int FWD_SMEM_M = (int)(FWD_SMEM_MAIN<2, 16> + sizeof(AcuStep));
 constexpr int ADJ_SMEM_M = (int)(ADJ_SMEM_MAIN + sizeof(AcuStep));
 
-// The forward kernel of one variant: recording, recording and storing, storing.
+// The forward kernel of one variant: recording, recording and storing, storing, and
+// recording without absorbing layers (up to 40 tiles of 32 rows per SM in all: 6080).
 template <int N, int R, int TY, bool LAP>
 auto fwd_kernel(int v) {
   return v == 0   ? acu_fwd_step<N, true, false, false, R, TY, LAP>
          : v == 1 ? acu_fwd_step<N, true, true, false, R, TY, LAP>
-                  : acu_fwd_step<N, false, true, false, R, TY, LAP>;
+         : v == 2 ? acu_fwd_step<N, false, true, false, R, TY, LAP>
+                  : acu_fwd_step<N, true, false, false, R, TY, LAP, fwd_pre(R, false, false)>;
 }
-int fwd_variant(bool record, bool store) { return !store ? 0 : record ? 1 : 2; }
+int fwd_variant(bool record, bool store, int S, const Grid& g, int dev) {
+  if (store) return record ? 1 : 2;
+  return g.npml == 0 && (long long)S * g.ntx * g.ntz <= 40 * g_sms[dev] ? 3 : 0;
+}
 // Tile heights 8, 32 and 64: one, two and four rows per thread.
 template <int N, bool LAP>
 auto fwd_kernel(int shape, int v) {
@@ -1401,7 +1410,7 @@ cudaError_t acu_fwd_rows(int S, int Sg, const Grid& g, int N, bool record, bool 
   int dev;
   const cudaError_t e = ensure_init(&dev);
   if (e != cudaSuccess) return e;
-  const int v = fwd_variant(record, store);
+  const int v = fwd_variant(record, store, S, g, dev);
   const long long fit = g_grid_fwd[dev][0][lap ? 1 : 0][N == 2 ? 0 : 1][v];
   *rows = (long long)Sg * g.ntx * ((g.Nz + 7) / 8) <= fit && (long long)S * g.ntx * g.ntz < 5 * g_sms[dev] ? 8 : 32;
   return cudaSuccess;
@@ -1418,7 +1427,7 @@ cudaError_t acu_fwd_groups(int S, const Grid& g, int N, bool lap, int* groups) {
   int dev;
   const cudaError_t e = ensure_init(&dev);
   if (e != cudaSuccess) return e;
-  const long long fit = g_grid_fwd[dev][1][lap ? 1 : 0][N == 2 ? 0 : 1][fwd_variant(true, false)], per = (long long)g.ntx * g.ntz;
+  const long long fit = g_grid_fwd[dev][1][lap ? 1 : 0][N == 2 ? 0 : 1][fwd_variant(true, false, S, g, dev)], per = (long long)g.ntx * g.ntz;
   *groups = (S + 1) / 2 * per > fit && (S + 2) / 3 * per <= fit ? 3 : 2;
   return cudaSuccess;
 }
@@ -1429,7 +1438,7 @@ cudaError_t launch_acu_fwd(const AcuStep& p_in, const AcuMaps& maps, bool record
   int dev;
   cudaError_t e = ensure_init(&dev);
   if (e != cudaSuccess) return e;
-  const int v = fwd_variant(record, store);
+  const int v = fwd_variant(record, store, p_in.S_pair, p_in.g, dev);
   const int o = p_in.N == 2 ? 0 : 1;
   const int sp = rows == 64 ? 2 : rows == 32 ? 1 : 0;
   const AcuCoef cf = coef_of(p_in);
