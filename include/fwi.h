@@ -246,7 +246,7 @@ fwi_status fwi_set_tile_shape(fwi_ctx *ctx, int32_t forward_tile_rows);
  * into forward_groups (forward and recompute steps) and adjoint_groups
  * (adjoint steps) contiguous groups, each step launched once per group on its
  * own stream, so that the groups' launches fill each other's idle SMs. 0 keeps
- * the library's default (2 or 3 for the forward sweep, 4 for recomputed steps, 2
+ * the library's default (2 to 4 for the forward sweep, 4 for recomputed steps, 2
  * for the adjoint); at most 4; never more groups than shots.
  * Results do not depend on it (the per-shot arithmetic and the fixed-order
  * cross-shot sums are the same). Takes effect for later calls and recordings;

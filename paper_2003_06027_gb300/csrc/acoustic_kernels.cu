@@ -1416,19 +1416,33 @@ cudaError_t acu_fwd_rows(int S, int Sg, const Grid& g, int N, bool record, bool 
   return cudaSuccess;
 }
 
-// Launches that make one recording step of S shots by default: two, or three where two
-// would each take a second, nearly empty wave and three fit the resident CTAs (3 per SM:
-// 912 to 1368 tiles). Per step with 2 / 3 / 4 groups: 16 shots of 306 x 310 (1152 tiles)
-// 13.1 / 9.9 / 10.1 us, 40 of 128 x 256 at 8th order without layers (1200) 12.4 / 11.1 /
-// 11.5 (the scalar kernel that this replaced, in four groups, 10.3); beyond, 16 of 201 x
-// 601 (1584) 13.7 / 13.5 / 13.5, at 8th order 15.1 / 15.1 / 15.4, 100 of 128 x 256 (3000)
-// 27.5 / 27.9 / 28.6.
+// Launches that make one recording step of S shots by default, from how many tiles of 32
+// rows fit the kernel's resident CTAs (3 per SM, 4 without layers). One wave each if two or
+// three launches allow it; else three that all take several waves, or four where three
+// would mix launches of one wave (dependent ones) with longer ones; two where they fill two
+// waves each (1.7 or more) and beyond 18 tiles per SM. Per step with 2 / 3 / 4 launches, 4th and 8th order:
+//   16 shots of 306 x 310 (1152 tiles)        13.1 /  9.9 / 10.1   14.4 / 11.3 / 11.6 us
+//   46 of 128 x 256 (1380: 480, 450, 450)     14.4 / 16.4 / 13.3   15.6 / 18.2 / 15.0
+//   8 of 536 x 636 (1672: 627, 627, 418)      13.7 / 14.4 / 12.3   14.9 / 16.1 / 14.0
+//   16 of 201 x 601 (1584; two: 1.74 waves)   13.7 / 13.5 / 13.5   15.1 / 15.1 / 15.4, and in
+//     a recorded gradient                                          14.8 / 15.1 / 15.0
+//   7 of 500 x 736 (1638: 702, 468, 468)      17.4 / 15.0 / 15.4   18.6 / 16.5 / 16.9
+//   30 of 306 x 310 (2160)                    18.4 / 17.1 / 17.6   20.5 / 19.8 / 20.3
+//   100 of 128 x 256 (3000)                   27.5 / 27.9 / 28.6   30.1 / 30.8 / 31.4
+// (the scalar kernel that this one replaced, in four launches: 12.9, 14.2, 14.6, 14.8,
+// 14.4, 18.6, 32.1 and 13.7, 14.9, 15.5, 15.8, 15.6, 20.7, 34.3).
 cudaError_t acu_fwd_groups(int S, const Grid& g, int N, bool lap, int* groups) {
   int dev;
   const cudaError_t e = ensure_init(&dev);
   if (e != cudaSuccess) return e;
-  const long long fit = g_grid_fwd[dev][1][lap ? 1 : 0][N == 2 ? 0 : 1][fwd_variant(true, false, S, g, dev)], per = (long long)g.ntx * g.ntz;
-  *groups = (S + 1) / 2 * per > fit && (S + 2) / 3 * per <= fit ? 3 : 2;
+  const long long fit = g_grid_fwd[dev][1][lap ? 1 : 0][N == 2 ? 0 : 1][fwd_variant(true, false, S, g, dev)];
+  const long long per = (long long)g.ntx * g.ntz;
+  auto most = [&](int G) { return (S + G - 1) / G * per; };  // tiles of the largest of G launches
+  *groups = 2;
+  if (S < 3 || most(2) <= fit) return cudaSuccess;
+  if (most(3) <= fit) *groups = 3;
+  else if (S / 3 * per <= fit) *groups = most(4) <= fit ? 4 : 2;
+  else if (S * per <= 18LL * g_sms[dev] && (10 * most(2) < 17 * fit || most(2) > 2 * fit)) *groups = 3;
   return cudaSuccess;
 }
 

@@ -59,8 +59,12 @@ def test_mixed_heights_give_the_same_bits(fwi_lib, nz, nx, S):
         assert a is None and b is None or torch.equal(a, b)
 
 
-# 1200 and 1152 tiles: two launches a step would each take a second wave, three fit
-@pytest.mark.parametrize("nz,nx,S,order,npml", [(192, 320, 40, 8, 0), (192, 320, 40, 4, 0), (306, 310, 16, 4, 32)])
+# 1200 and 1152 tiles: two launches a step would each take a second wave, three fit; 1380, 1408 and 1672: three
+# launches, not all of one wave; 1500 and 2160 tiles: none of two, three or four fits
+@pytest.mark.parametrize("nz,nx,S,order,npml", [
+    (192, 320, 40, 8, 0), (192, 320, 40, 4, 0), (306, 310, 16, 4, 32), (128, 256, 46, 8, 32), (436, 436, 11, 4, 32),
+    (536, 636, 8, 4, 32), (306, 310, 30, 4, 32), (32, 236, 100, 8, 32),
+])
 def test_default_groups_are_not_slower_than_four(fwi_lib, nz, nx, S, order, npml):
     import torch
 
@@ -78,5 +82,5 @@ def test_default_groups_are_not_slower_than_four(fwi_lib, nz, nx, S, order, npml
     finally:
         fwi.set_shot_groups(0, 0)
     assert torch.equal(seis[0], seis[4])
-    # two groups took 1.08 to 1.3 times as long as four at these sizes
+    # two groups took 1.04 to 1.3 times as long as four at most of these sizes
     assert best[0] <= 1.05 * best[4]
