@@ -104,7 +104,9 @@ cudaError_t launch_step(void (*kern)(P...), long long items, int grid, int threa
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = items <= grid ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
+  if (e != cudaSuccess) cudaGetLastError();  // reported here: not again by the next launch's check
+  return e;
 }
 
 namespace tma_host {
