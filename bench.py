@@ -346,7 +346,7 @@ def batched_measure(n_inst=16):
 
     inst = batch.prepare([synth.uneven_instance(4, i) for i in range(n_inst)])
     cells = sum(i.cell_steps for i in inst)
-    modes, tiles = ("persistent", "graph", "batched"), (32, 64)
+    modes, tiles = ("persistent", "graph", "batched"), (0, 64)  # 0: the default, 8 or 32 rows
     best, table = batch.autotune(inst, workers=(1, 2, 4, 8), ckpt=(100,), modes=modes, tiles=tiles)
     mode, W, K, _, tile = batch.candidate(best, tiles=tiles)
     _, _, tb = batch.sweep(inst, mode, W, K, tile_rows=tile)

@@ -276,8 +276,9 @@ def autotune(instances, workers=(1, 2, 4, 8), ckpt=(50, 100, 200), modes=("batch
     candidate also sizes the arenas or records the graphs, so each candidate is
     run twice and the second run counts). ``groups`` lists (forward, adjoint)
     shot-group counts, the step kernels' launch shape (fwi_set_shot_groups);
-    ``tiles`` lists forward tile heights (fwi_set_tile_shape: 0 or 32, 64; the
-    persistent mode runs 32-row tiles only). A candidate's key is (mode, W, K),
+    ``tiles`` lists forward tile heights (fwi_set_tile_shape: 0, the default of 8
+    or 32 rows by each launch's size; 32; 64; the persistent mode runs 32-row
+    tiles only). A candidate's key is (mode, W, K),
     followed by the shot groups if more than one is listed and by the tile
     height if more than one is listed (`candidate` unpacks it). The pools of
     the losing worker counts are closed, and the graphs and batches the winner

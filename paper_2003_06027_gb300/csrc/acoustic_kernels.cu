@@ -1398,7 +1398,7 @@ cudaError_t acu_make_maps(AcuMaps* maps, const Grid& g, int S, float* u_pair, co
 // many CTAs, each a quarter of the latency) are faster while a launch's all fit the
 // resident CTAs, so that each step is one wave of dependent launches. Per step, 8 against
 // 32 rows, 4th order, recording (2 groups) / storing (4 groups):
-//   one shot of 100 x 100 (15 tiles of 32 rows)  4.6 / -      against  4.9 / -
+//   one shot of 100 x 100 (15 tiles of 32 rows)  4.6 / -      against  5.1 / -
 //   16 shots of 128 x 256 (480)                  7.0 /  8.0   against  7.4 / 11.5
 //   20 (600; 1200 of 1216 places a group)        8.0 /  9.0   against  7.8 / 12.1
 //   24 (720; the recording groups do not fit)   12.3 / 10.3   against  8.2 / 12.5

@@ -803,9 +803,8 @@ fwi_status acu_misfit_grad(fwi_ctx* ctx, const fwi_model* M, const fwi_sources* 
   // forward sweep with a full-state checkpoint at the start of every segment
   // but the last: the sweep itself keeps the last segment's fluxes (recording
   // and storing in one launch), so that segment is never recomputed. Its steps run in
-  // the storing steps' groups (16 shots of 201 x 601, 600 steps of which 600 / 100 are
-  // stored by the sweep: 25.6 / 33.4 ms a gradient; 3000 steps, all stored: 129.5 ms
-  // in two groups, 121.3 in four)
+  // the storing steps' groups (16 shots of 201 x 601, 3000 steps, all of them stored by
+  // the sweep: a gradient takes 129.5 ms in two groups, 121.3 in four)
   const int nlast = (P.nseg - 1) * K;
   CK(mark(ctx->ev[0], st, capture));
   const Groups* sg = nlast > 0 ? &gr : &grs;

@@ -163,8 +163,8 @@ def set_shot_groups(forward_groups: int = 0, adjoint_groups: int = 0, device: in
 
 
 def set_tile_shape(forward_tile_rows: int = 0, device: int = 0):
-    """Tile height (32 or 64 rows; 0: the default) of the acoustic forward steps
-    of this thread's context (fwi_set_tile_shape)."""
+    """Tile height (32 or 64 rows; 0: the default, 8 or 32 by each launch's size)
+    of the acoustic forward steps of this thread's context (fwi_set_tile_shape)."""
     _check(library().fwi_set_tile_shape(context(device), int(forward_tile_rows)))
 
 
