@@ -67,9 +67,13 @@ constexpr int XS_BYTES = TILE_Z * UW * 4;  // 10240: adjoint x operand tile
 // (per step, 3 -> 4 CTAs: 40 shots of 192 x 320, 1200 tiles, at 8th order 11.1 -> 10.1 us,
 // at 4th 9.0 -> 8.4; 100 shots 25.3 -> 23.6 and 20.0 -> 18.9; 60 of 370 x 374, 4320 tiles,
 // 32.2 -> 30.8 and 26.1 -> 25.4), but not where fields stream from memory (128 of 265 x
-// 665, 12 672 tiles: 86.8 -> 87.2 and 72.7 -> 74.7). The 8-row tile (8 CTAs) and the
-// 64-row one (2) hold them.
-__host__ __device__ constexpr bool fwd_pre(int R, bool store, bool layers) { return R != 2 || (!store && layers); }
+// 665, 12 672 tiles: 86.8 -> 87.2 and 72.7 -> 74.7). The c^2 Laplacian's recording step
+// at 4th order spills when it holds them (128 shots of 201 x 601 113.0 us against 92.2
+// without, 60 of 306 x 310 42.4 against 32.6); at 8th it does not (110.9 against 114.3).
+// The 8-row tile (8 CTAs) and the 64-row one (2) hold them.
+__host__ __device__ constexpr bool fwd_pre(int N, int R, bool store, bool lap, bool layers) {
+  return R != 2 || (!store && layers && !(lap && N == 2));
+}
 __host__ __device__ constexpr int fwd_ctas(int R, bool pre) { return R == 1 ? 8 : R == 4 ? 2 : pre ? 3 : 4; }
 template <int R, int TY>
 struct FwdGeo {
@@ -396,7 +400,7 @@ __device__ __forceinline__ void batch_load_step(const BatchArgs& b, int i, AcuSt
 // u^{n+1} = 2u^n - u^{n-1} + m dt^2 (D-q + zeta) + dt^2 w g(t_n) with m = c^2 at
 // the cell, and STORE keeps r = dt^2 (D-q + zeta) at the cells (the operand of
 // its gradient correlation dJ/dm = sum_n lambda_{n+1} r^n) instead of the fluxes.
-template <int N, bool RECORD, bool STORE, bool MULTI, int R, int TY, bool LAP = false, bool PRE = fwd_pre(R, STORE, true)>
+template <int N, bool RECORD, bool STORE, bool MULTI, int R, int TY, bool LAP = false, bool PRE = fwd_pre(N, R, STORE, LAP, true)>
 __global__ void __launch_bounds__(16 * TY, fwd_ctas(R, PRE))
     acu_fwd_step(const __grid_constant__ CUtensorMap tmap_u, const __grid_constant__ CUtensorMap tmap_m,
                  const __grid_constant__ AcuStep p0, const __grid_constant__ AcuCoef cf, const BatchArgs b) {
@@ -1287,7 +1291,7 @@ auto fwd_kernel(int v) {
   return v == 0   ? acu_fwd_step<N, true, false, false, R, TY, LAP>
          : v == 1 ? acu_fwd_step<N, true, true, false, R, TY, LAP>
          : v == 2 ? acu_fwd_step<N, false, true, false, R, TY, LAP>
-                  : acu_fwd_step<N, true, false, false, R, TY, LAP, fwd_pre(R, false, false)>;
+                  : acu_fwd_step<N, true, false, false, R, TY, LAP, fwd_pre(N, R, false, LAP, false)>;
 }
 int fwd_variant(bool record, bool store, int S, const Grid& g, int dev) {
   if (store) return record ? 1 : 2;
