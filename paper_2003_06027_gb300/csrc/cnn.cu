@@ -686,6 +686,7 @@ extern "C" {
 fwi_status fwi_cnn_create(fwi_cnn** h, int device) {
   if (!h) return fwi::host_fail(FWI_EINVAL, "h must not be NULL");
   CNN_CK(cudaSetDevice(device), "cudaSetDevice");
+  CNN_CK(fwi::tc_gemm_init(), "GEMM set-up");
   fwi_cnn* c = new fwi_cnn;
   c->device = device;
   cudaError_t e = cudaMalloc(&c->status, sizeof(int));

@@ -798,15 +798,17 @@ cudaError_t tc_setup(K kern, int optin, int* smem) {
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, *smem);
 }
 
-cudaError_t tc_device(const TcDev** out) {
+// The current device's entry, set up at its first use; `again` repeats that (a new
+// handle: the device may have been reset since).
+cudaError_t tc_device(const TcDev** out, bool again = false) {
   int dev = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(g_tc_mu);
-  TcDev& d = g_tc[dev];
-  *out = &d;
-  if (d.ready) return cudaSuccess;
+  *out = &g_tc[dev];
+  if (g_tc[dev].ready && !again) return cudaSuccess;
+  TcDev d;
   if ((e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
   if ((e = tc_setup(k_tc_gemm<0>, optin, &d.smem[K_TMA])) != cudaSuccess) return e;
@@ -816,6 +818,7 @@ cudaError_t tc_device(const TcDev** out) {
   if ((e = tc_setup(k_conv_pairs<1>, optin, &d.smem[K_PAIRS1])) != cudaSuccess) return e;
   if ((e = tc_setup(k_conv_pairs<2>, optin, &d.smem[K_PAIRS2])) != cudaSuccess) return e;
   d.ready = true;
+  if (!g_tc[dev].ready) g_tc[dev] = d;  // others may be reading it
   return cudaSuccess;
 }
 
@@ -853,6 +856,11 @@ cudaError_t conv_pairs(const TcConvA& c, const CUtensorMap& tb, TcArgs a, int pa
   return cudaGetLastError();
 }
 }  // namespace
+
+cudaError_t tc_gemm_init() {
+  const TcDev* dev;
+  return tc_device(&dev, true);
+}
 
 cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st) {
   const bool conv = g.conv != nullptr;

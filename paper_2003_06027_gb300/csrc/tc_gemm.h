@@ -68,6 +68,7 @@ struct TcGemm {
 // aligned pairs of inputs. 0 if not.
 int tc_conv_pairs(const TcConvA& c);
 
+cudaError_t tc_gemm_init();  // sets the kernels up on the current device (each new handle)
 cudaError_t tc_gemm(const TcGemm& g, cudaStream_t st);
 
 // Number of 64-wide k-blocks of a K-long contraction, and the number of
