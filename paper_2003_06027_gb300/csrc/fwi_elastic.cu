@@ -313,7 +313,10 @@ fwi_status ela_prepare(fwi_ctx* ctx, EPlan& P, const fwi_model* M, const fwi_sou
 // launches only wait for each other: 4 shots of 200 x 400 (288 tiles) 18.5/20/27 ->
 // 20/23/26.5. That is 3 CTAs on each SM at 4th order (4 shots of 200 x 550, 360 tiles:
 // 18.0/19.2/27.3 -> 18.7/20.4/26.8) and 2 at 8th (22.0/23.8/35.1 -> 17.5/19.1/24.1; 24 of
-// 60 x 120, 288 tiles: 15.9/16.6/23.3 -> 16.2/17.0/23.3).
+// 60 x 120, 288 tiles: 15.9/16.6/23.3 -> 16.2/17.0/23.3). Nor do two pay where one launch
+// takes two waves and the larger of two would too: 13 shots of 66 x 914 at 8th order, 585
+// tiles of 304 places as 315 + 270, 29.7/33.2/41.0 -> 31.4/34.4/44.4 (624 as 312 + 312,
+// three waves alone: 36.5/39.6/64.9 -> 31.0/33.5/50.7).
 struct EGroups {
   int G = 1;
   int s0[2] = {0, 0}, n[2] = {0, 0};
@@ -323,7 +326,8 @@ struct EGroups {
 fwi_status ela_groups(fwi_ctx* ctx, const EPlan& P, cudaStream_t main, EGroups& gr) {
   int resident;
   ECK(ela_resident(P.N, &resident));
-  gr.G = P.S >= 2 && (long long)P.S * P.g.ntx * P.g.ntz > resident ? 2 : 1;
+  const long long tiles = (long long)P.S * P.g.ntx * P.g.ntz, most = (long long)(P.S + 1) / 2 * P.g.ntx * P.g.ntz;
+  gr.G = P.S >= 2 && tiles > resident && (most <= resident || tiles > 2LL * resident) ? 2 : 1;
   for (int g = 0, s0 = 0; g < gr.G; g++) {
     gr.n[g] = P.S / gr.G + (g < P.S % gr.G ? 1 : 0);
     gr.s0[g] = s0;

@@ -38,3 +38,21 @@ def test_groups_from_one_tile_per_resident_cta(fwi_lib, nshots, groups):
     # sums over shots in FP64, rounded to FP32 once here and once per part there
     a, b = (p[0][1].double() for p in parts)
     assert float((g.double() - (a + b)).norm()) <= 4 * 2.0**-24 * float(a.norm() + b.norm())
+
+
+@pytest.mark.parametrize("nz,nx,nshots,groups", [(66, 914, 13, 1), (66, 914, 12, 2), (400, 700, 3, 1), (76, 108, 104, 2)])
+def test_one_launch_of_two_waves_stays_one(fwi_lib, nz, nx, nshots, groups):
+    # 585 tiles as 315 + 270, 540 as 270 + 270, 504 as 336 + 168, 624 as 312 + 312, of 304 places
+    import torch
+
+    from paper_2003_06027_gb300 import fwi
+
+    d = synth.random_elastic(5, nz, nx, 20, nshots, 8, 10, dx=5.0, dt=4e-4, nrec=3)
+    cu = lambda a: torch.as_tensor(np.ascontiguousarray(a)).cuda()
+    kw, model = fwi.problem_kwargs(d), [cu(d[k]) for k in ("vp", "vs", "rho")]
+    src, rec = [cu(d[k]) for k in ("stf", "x0", "mt")], [cu(d[k]) for k in ("rec_iz", "rec_ix")]
+    seis = fwi.forward_elastic(*model, *src, *rec, **kw)
+    n = fwi.last_timing().launches
+    part = fwi.forward_elastic(*model, *[a[:1].contiguous() for a in src], *rec, **kw)  # one group
+    assert n - fwi.last_timing().launches == (groups - 1) * 40  # 2 launches for each of 20 steps
+    assert torch.equal(part, seis[:1])
