@@ -233,9 +233,9 @@ fwi_status fwi_choose_ckpt(fwi_ctx *ctx, const fwi_model *model, const fwi_sourc
                            int32_t *ckpt_every);
 
 /* Tile shape of the acoustic forward steps of ctx's calls (forward sweep and
- * segment recompute): tiles of 64 columns x forward_tile_rows rows, 32 or 64 (256
- * threads per CTA; 64 halves the z-halo flux recompute per cell in fewer and
- * larger CTAs). 0 keeps the library's default: 32, or 8 (which cannot be asked
+ * segment recompute): tiles of 64 columns x forward_tile_rows rows, 32 or 64 (64
+ * halves the z-halo flux recompute per cell in fewer and larger CTAs; calls of the
+ * c^2 Laplacian operator run 32 for it). 0 keeps the library's default: 32, or 8 (which cannot be asked
  * for) while a launch's 8-row tiles all run at once. Results do not
  * depend on it (each cell's arithmetic is the same). Takes effect for later
  * calls and recordings; FWI_EINVAL for other values. The batched autotuner

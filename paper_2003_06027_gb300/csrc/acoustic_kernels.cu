@@ -70,11 +70,15 @@ constexpr int XS_BYTES = TILE_Z * UW * 4;  // 10240: adjoint x operand tile
 // 665, 12 672 tiles: 86.8 -> 87.2 and 72.7 -> 74.7). The c^2 Laplacian's recording step
 // at 4th order spills when it holds them (128 shots of 201 x 601 113.0 us against 92.2
 // without, 60 of 306 x 310 42.4 against 32.6); at 8th it does not (110.9 against 114.3).
-// The 8-row tile (8 CTAs) and the 64-row one (2) hold them.
-__host__ __device__ constexpr bool fwd_pre(int N, int R, bool store, bool lap, bool layers) {
-  return R != 2 || (!store && layers && !(lap && N == 2));
+// The 8-row tile (8 CTAs) holds them. The 64-row tile runs 2 CTAs of 512 threads without;
+// storing at 4th order, 2 of 256 threads (4 rows each) with them. Recording / storing step
+// in 64-row tiles, 256 -> 512 threads: 29 shots of 408 x 248 without layers, 8th order
+// 17.5 / 18.9 -> 13.5 / 16.0 us, 4th 14.6 / 16.0 -> 12.0 / 16.5; 85 of 146 x 133 20.4 / 23.6
+// -> 19.6 / 22.5, 4th 19.0 / 22.3 -> 18.2 / 24.3.
+__host__ __device__ constexpr bool fwd_pre(int N, int R, int TY, bool store, bool lap, bool layers) {
+  return TY != 32 && (R != 2 || (!store && layers && !(lap && N == 2)));
 }
-__host__ __device__ constexpr int fwd_ctas(int R, bool pre) { return R == 1 ? 8 : R == 4 ? 2 : pre ? 3 : 4; }
+__host__ __device__ constexpr int fwd_ctas(int R, int TY, bool pre) { return R == 1 ? 8 : R == 4 || TY == 32 ? 2 : pre ? 3 : 4; }
 template <int R, int TY>
 struct FwdGeo {
   static constexpr int NT = 16 * TY;          // threads
@@ -400,8 +404,8 @@ __device__ __forceinline__ void batch_load_step(const BatchArgs& b, int i, AcuSt
 // u^{n+1} = 2u^n - u^{n-1} + m dt^2 (D-q + zeta) + dt^2 w g(t_n) with m = c^2 at
 // the cell, and STORE keeps r = dt^2 (D-q + zeta) at the cells (the operand of
 // its gradient correlation dJ/dm = sum_n lambda_{n+1} r^n) instead of the fluxes.
-template <int N, bool RECORD, bool STORE, bool MULTI, int R, int TY, bool LAP = false, bool PRE = fwd_pre(N, R, STORE, LAP, true)>
-__global__ void __launch_bounds__(16 * TY, fwd_ctas(R, PRE))
+template <int N, bool RECORD, bool STORE, bool MULTI, int R, int TY, bool LAP = false, bool PRE = fwd_pre(N, R, TY, STORE, LAP, true)>
+__global__ void __launch_bounds__(16 * TY, fwd_ctas(R, TY, PRE))
     acu_fwd_step(const __grid_constant__ CUtensorMap tmap_u, const __grid_constant__ CUtensorMap tmap_m,
                  const __grid_constant__ AcuStep p0, const __grid_constant__ AcuCoef cf, const BatchArgs b) {
   static_assert(!LAP || !MULTI, "the Laplacian operator runs on single-instance launches");
@@ -1291,21 +1295,29 @@ auto fwd_kernel(int v) {
   return v == 0   ? acu_fwd_step<N, true, false, false, R, TY, LAP>
          : v == 1 ? acu_fwd_step<N, true, true, false, R, TY, LAP>
          : v == 2 ? acu_fwd_step<N, false, true, false, R, TY, LAP>
-                  : acu_fwd_step<N, true, false, false, R, TY, LAP, fwd_pre(N, R, false, LAP, false)>;
+                  : acu_fwd_step<N, true, false, false, R, TY, LAP, fwd_pre(N, R, TY, false, LAP, false)>;
 }
 int fwd_variant(bool record, bool store, int S, const Grid& g, int dev) {
   if (store) return record ? 1 : 2;
   return g.npml == 0 && (long long)S * g.ntx * g.ntz <= 40 * g_sms[dev] ? 3 : 0;
 }
-// Tile heights 8, 32 and 64: one, two and four rows per thread.
+// Tile heights 8, 32 and 64 (64 for the divergence form only).
+bool tall_rows(int N, int v) { return N == 2 && (v == 1 || v == 2); }  // 64-row tiles of 4 rows a thread
 template <int N, bool LAP>
 auto fwd_kernel(int shape, int v) {
-  return shape == 0 ? fwd_kernel<N, 1, 8, LAP>(v) : shape == 1 ? fwd_kernel<N, 2, 16, LAP>(v) : fwd_kernel<N, 4, 16, LAP>(v);
+  if (shape == 0) return fwd_kernel<N, 1, 8, LAP>(v);
+  if constexpr (!LAP) {
+    if constexpr (N == 2)
+      if (shape == 2 && tall_rows(N, v)) return v == 1 ? acu_fwd_step<N, true, true, false, 4, 16> : acu_fwd_step<N, false, true, false, 4, 16>;
+    if (shape == 2) return fwd_kernel<N, 2, 32, LAP>(v);
+  }
+  return fwd_kernel<N, 2, 16, LAP>(v);
 }
 size_t fwd_smem(int shape) {
-  return shape == 0 ? sizeof(FwdSmemT<1, 8>) : shape == 1 ? sizeof(FwdSmemT<2, 16>) : sizeof(FwdSmemT<4, 16>);
+  static_assert(sizeof(FwdSmemT<4, 16>) == sizeof(FwdSmemT<2, 32>), "64-row tiles");
+  return shape == 0 ? sizeof(FwdSmemT<1, 8>) : shape == 1 ? sizeof(FwdSmemT<2, 16>) : sizeof(FwdSmemT<2, 32>);
 }
-int fwd_threads(int shape) { return shape == 0 ? 128 : 256; }
+int fwd_threads(int shape, int N, int v) { return shape == 0 ? 128 : shape == 1 || tall_rows(N, v) ? 256 : 512; }
 constexpr int fwd_tz(int shape) { return shape == 0 ? 8 : shape == 1 ? 32 : 64; }
 
 template <int N>
@@ -1315,8 +1327,10 @@ cudaError_t setup_order(int dev, int o) {
   for (int sp = 0; sp < FWD_SHAPES; sp++)
     for (int v = 0; v < FWD_VARIANTS; v++) {
       const int fs = (int)fwd_smem(sp);
-      if ((e = setup_kernel(fwd_kernel<N, false>(sp, v), fs, &g_grid_fwd[dev][sp][0][o][v], fwd_threads(sp))) != cudaSuccess) return e;
-      if ((e = setup_kernel(fwd_kernel<N, true>(sp, v), fs, &g_grid_fwd[dev][sp][1][o][v], fwd_threads(sp))) != cudaSuccess) return e;
+      const int nt = fwd_threads(sp, N, v);
+      if ((e = setup_kernel(fwd_kernel<N, false>(sp, v), fs, &g_grid_fwd[dev][sp][0][o][v], nt)) != cudaSuccess) return e;
+      if (sp < 2 && (e = setup_kernel(fwd_kernel<N, true>(sp, v), fs, &g_grid_fwd[dev][sp][1][o][v], nt)) != cudaSuccess)
+        return e;
     }
   if ((e = setup_kernel(acu_fwd_step<N, true, true, true, 2, 16>, FWD_SMEM_M, &g_grid_fwd_m[dev][o][0], 256)) != cudaSuccess)
     return e;
@@ -1450,7 +1464,8 @@ cudaError_t acu_fwd_groups(int S, const Grid& g, int N, bool lap, int* groups) {
   return cudaSuccess;
 }
 
-// Forward step on tiles of `rows` rows (8, 32 or 64).
+// Forward step on tiles of `rows` rows (8, 32 or 64; the c^2 Laplacian runs 32 for 64, which
+// takes up to 1.5 times as long: 16 shots of 201 x 601 22.0 against 14.4 us).
 cudaError_t launch_acu_fwd(const AcuStep& p_in, const AcuMaps& maps, bool record, bool store, int rows, bool lap,
                            cudaStream_t st) {
   int dev;
@@ -1458,7 +1473,7 @@ cudaError_t launch_acu_fwd(const AcuStep& p_in, const AcuMaps& maps, bool record
   if (e != cudaSuccess) return e;
   const int v = fwd_variant(record, store, p_in.S_pair, p_in.g, dev);
   const int o = p_in.N == 2 ? 0 : 1;
-  const int sp = rows == 64 ? 2 : rows == 32 ? 1 : 0;
+  const int sp = rows == 64 && !lap ? 2 : rows == 8 ? 0 : 1;
   const AcuCoef cf = coef_of(p_in);
   BatchArgs nb;
   memset(&nb, 0, sizeof nb);
@@ -1467,7 +1482,7 @@ cudaError_t launch_acu_fwd(const AcuStep& p_in, const AcuMaps& maps, bool record
   const int grid = std::min(p.ntiles, g_grid_fwd[dev][sp][lap ? 1 : 0][o][v]);
   auto k = p.N == 2 ? (lap ? fwd_kernel<2, true>(sp, v) : fwd_kernel<2, false>(sp, v))
                     : (lap ? fwd_kernel<4, true>(sp, v) : fwd_kernel<4, false>(sp, v));
-  return launch_step(k, p.ntiles, grid, fwd_threads(sp), fwd_smem(sp), st, maps.u[sp], maps.m[sp], p, cf, nb);
+  return launch_step(k, p.ntiles, grid, fwd_threads(sp, p.N, v), fwd_smem(sp), st, maps.u[sp], maps.m[sp], p, cf, nb);
 }
 
 // Multi-instance forward step b.n over the tiles of instances [0, b.n_active):
