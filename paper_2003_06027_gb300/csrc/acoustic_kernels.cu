@@ -70,13 +70,16 @@ constexpr int XS_BYTES = TILE_Z * UW * 4;  // 10240: adjoint x operand tile
 // 665, 12 672 tiles: 86.8 -> 87.2 and 72.7 -> 74.7). The c^2 Laplacian's recording step
 // at 4th order spills when it holds them (128 shots of 201 x 601 113.0 us against 92.2
 // without, 60 of 306 x 310 42.4 against 32.6); at 8th it does not (110.9 against 114.3).
+// The divergence form's storing step at 4th order is the other way round: it spills at 4
+// CTAs (47 shots of 141 x 144 22.6 us against 18.4 holding them, 24 of 201 x 601 31.0
+// against 26.6, 128 148.4 against 142.1).
 // The 8-row tile (8 CTAs) holds them. The 64-row tile runs 2 CTAs of 512 threads without;
 // storing at 4th order, 2 of 256 threads (4 rows each) with them. Recording / storing step
 // in 64-row tiles, 256 -> 512 threads: 29 shots of 408 x 248 without layers, 8th order
 // 17.5 / 18.9 -> 13.5 / 16.0 us, 4th 14.6 / 16.0 -> 12.0 / 16.5; 85 of 146 x 133 20.4 / 23.6
 // -> 19.6 / 22.5, 4th 19.0 / 22.3 -> 18.2 / 24.3.
 __host__ __device__ constexpr bool fwd_pre(int N, int R, int TY, bool store, bool lap, bool layers) {
-  return TY != 32 && (R != 2 || (!store && layers && !(lap && N == 2)));
+  return TY != 32 && (R != 2 || (store ? N == 2 && !lap : layers && !(lap && N == 2)));
 }
 __host__ __device__ constexpr int fwd_ctas(int R, int TY, bool pre) { return R == 1 ? 8 : R == 4 || TY == 32 ? 2 : pre ? 3 : 4; }
 template <int R, int TY>
@@ -404,7 +407,7 @@ __device__ __forceinline__ void batch_load_step(const BatchArgs& b, int i, AcuSt
 // u^{n+1} = 2u^n - u^{n-1} + m dt^2 (D-q + zeta) + dt^2 w g(t_n) with m = c^2 at
 // the cell, and STORE keeps r = dt^2 (D-q + zeta) at the cells (the operand of
 // its gradient correlation dJ/dm = sum_n lambda_{n+1} r^n) instead of the fluxes.
-template <int N, bool RECORD, bool STORE, bool MULTI, int R, int TY, bool LAP = false, bool PRE = fwd_pre(N, R, TY, STORE, LAP, true)>
+template <int N, bool RECORD, bool STORE, bool MULTI, int R, int TY, bool LAP = false, bool PRE = !MULTI && fwd_pre(N, R, TY, STORE, LAP, true)>
 __global__ void __launch_bounds__(16 * TY, fwd_ctas(R, TY, PRE))
     acu_fwd_step(const __grid_constant__ CUtensorMap tmap_u, const __grid_constant__ CUtensorMap tmap_m,
                  const __grid_constant__ AcuStep p0, const __grid_constant__ AcuCoef cf, const BatchArgs b) {
@@ -1415,22 +1418,25 @@ cudaError_t acu_make_maps(AcuMaps* maps, const Grid& g, int S, float* u_pair, co
 // most Sg. 32-row tiles need the fewest instructions per cell; 8-row tiles (four times as
 // many CTAs, each a quarter of the latency) are faster while a launch's all fit the
 // resident CTAs, so that each step is one wave of dependent launches. Per step, 8 against
-// 32 rows, 4th order, recording (2 groups) / storing (4 groups):
-//   one shot of 100 x 100 (15 tiles of 32 rows)  4.6 / -      against  5.1 / -
-//   16 shots of 128 x 256 (480)                  7.0 /  8.0   against  7.4 / 11.5
-//   20 (600; 1200 of 1216 places a group)        8.0 /  9.0   against  7.8 / 12.1
-//   24 (720; the recording groups do not fit)   12.3 / 10.3   against  8.2 / 12.5
-//   12 in one group (360, does not fit)         10.2          against  6.9
+// 32 rows, 8th order, recording (2 groups) / storing (4 groups):
+//   one shot of 100 x 100 (15 tiles of 32 rows)  4.6 / -      against  5.2 / -
+//   16 shots of 128 x 256 (480)                  7.8 /  7.9   against  7.9 / 10.0
+//   20 (600; 1200 of 1216 places a group)        8.8 /  9.0   against  8.4 / 10.5
+//   24 (720; the recording groups do not fit)   12.3 / 10.4   against  9.0 / 11.0
+//   12 in one group (360, does not fit)         10.3          against  7.4
 // Storing groups fit up to 1216 tiles, but from some 850 on the four launches no longer
-// run beside each other: 840 tiles 11.7 against 12.9 us, 960 12.8 against 13.1 (8th order
-// 13.0 against 11.7), 1200 15.9 against 14.7; hence the second bound, 5 tiles per SM.
+// run beside each other: 840 tiles 11.8 against 11.5 us, 960 13.0 against 11.7; hence the
+// second bound, 5 tiles per SM. The divergence form's storing step at 4th order, the one
+// that holds its layer operands, passes its 8-row tiles earlier: 3 tiles per SM (480 tiles
+// 10.0 against 9.9, 594 11.9 against 11.5, 720 13.7 against 12.7, in calls of 60 steps).
 cudaError_t acu_fwd_rows(int S, int Sg, const Grid& g, int N, bool record, bool store, bool lap, int* rows) {
   int dev;
   const cudaError_t e = ensure_init(&dev);
   if (e != cudaSuccess) return e;
   const int v = fwd_variant(record, store, S, g, dev);
   const long long fit = g_grid_fwd[dev][0][lap ? 1 : 0][N == 2 ? 0 : 1][v];
-  *rows = (long long)Sg * g.ntx * ((g.Nz + 7) / 8) <= fit && (long long)S * g.ntx * g.ntz < 5 * g_sms[dev] ? 8 : 32;
+  const int most = store && N == 2 && !lap ? 3 : 5;  // tiles of 32 rows per SM
+  *rows = (long long)Sg * g.ntx * ((g.Nz + 7) / 8) <= fit && (long long)S * g.ntx * g.ntz < most * g_sms[dev] ? 8 : 32;
   return cudaSuccess;
 }
 
